@@ -22,60 +22,6 @@ namespace fmm {
 
 #define TWO_PI 6.283185307179586476925
 
-// ------------------------------------------------------------------ FP64 form
-
-#define TILE64 512
-
-__global__ void __launch_bounds__(64) k_p2p64(Work w)
-{
-    __shared__ double shx[TILE64], shy[TILE64], shg[TILE64];
-    int leaf = blockIdx.x;
-    int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
-    if (c == 0)
-        return;
-    int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
-    const SysDev &d = w.sys[k];
-    int L = d.depth, ns = 1 << L, local = leaf - (int)d.leaf0;
-    int ix = local & (ns - 1), iy = local >> L;
-    double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
-    int jx0 = ix > 0 ? ix - 1 : 0, jx1 = ix < ns - 1 ? ix + 1 : ns - 1;
-    for (int t0 = 0; t0 < c; t0 += blockDim.x) {
-        int tpos = s0 + t0 + threadIdx.x;
-        bool valid = t0 + threadIdx.x < c;
-        double xt = valid ? w.sx[tpos] : 0.0, yt = valid ? w.sy[tpos] : 0.0;
-        double au = 0.0, av = 0.0;
-        for (int dy = -1; dy <= 1; ++dy) {
-            int row = iy + dy;
-            if (row < 0 || row >= ns)
-                continue;
-            int r0 = w.start[d.leaf0 + row * ns + jx0], r1 = w.start[d.leaf0 + row * ns + jx1 + 1];
-            for (int q0 = r0; q0 < r1; q0 += TILE64) {
-                int m = min(TILE64, r1 - q0);
-                __syncthreads();
-                for (int j = threadIdx.x; j < m; j += blockDim.x) {
-                    shx[j] = w.sx[q0 + j];
-                    shy[j] = w.sy[q0 + j];
-                    shg[j] = w.sg[q0 + j];
-                }
-                __syncthreads();
-                if (valid) {
-                    for (int j = 0; j < m; ++j) {
-                        double ax = xt - shx[j], ay = yt - shy[j];
-                        double r2 = ax * ax + ay * ay;
-                        if (r2 > 0.0) {
-                            double f = -expm1(-r2 * k2) / r2 * shg[j];
-                            au -= ay * f;
-                            av += ax * f;
-                        }
-                    }
-                }
-            }
-        }
-        if (valid)
-            w.near64[tpos] = make_double2(au / TWO_PI, av / TWO_PI);
-    }
-}
-
 // ------------------------------------------------------------------ precision form
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -1012,10 +958,8 @@ int launch_p2p(const Work &w, int threads, int kt, cudaStream_t s)
 {
     if (w.nleaf == 0)
         return 0;
-    if (!w.mixed) {
-        k_p2p64<<<w.nleaf, 64, 0, s>>>(w);
-        return 1;
-    }
+    if (!w.mixed)
+        return launch_near64(w, s);
     int ktmax = kt == 2 ? 2 : 4;
     int nl = 0;
     if (threads == 128 && w.p2p_sym) {
