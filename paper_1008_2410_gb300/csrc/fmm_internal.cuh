@@ -271,6 +271,7 @@ bool m2l_tc_supported(int p);
 int m2l_tc_max_level();
 int prepare_m2l_tc();
 int launch_near64(const Work &w, cudaStream_t s);  // plain form's near field (near64.cu) into near64
+int launch_adjoint_near64(const Work &w, double *dg, double *dx, double *dy, int skip_plain, cudaStream_t s);
 int prepare_near64(cudaStream_t s);  // its table, once per device before any stream capture; 0 on success
 int prepare_p2p();  // near-field kernel attributes, once per device before any stream capture; 0 on success
 int launch_m2l_tc(const Work &w, const Tables &t, int l_lo, int l_hi, cudaStream_t s);

@@ -29,9 +29,22 @@ constexpr double kTwoPi = 6.283185307179586476925;
 // nodes, truncated to degree 6 (its error there is below (1/32)^7 / (2^6 7! 8) = 2e-17), then c itself. x < 37.5.
 constexpr int kTabN = 600;
 constexpr double kXCut = 37.5;  // e^-37.5 < 2^-54: beyond it 1 - e^-x rounds to 1
-__device__ double2 g_blob_f[kTabN * 4];
+__device__ double2 g_blob_f[kTabN * 4], g_blob_d[kTabN * 4];  // F and F'
 
 long double blob_f(long double x) { return x == 0.0L ? 1.0L : -expm1l(-x) / x; }
+
+// F'(x) = ((1 + x) e^-x - 1) / x^2, below 1.5 by its Taylor series sum_k (-1)^k k x^(k-1) / (k+1)!.
+long double blob_d(long double x)
+{
+    if (x >= 1.5L)
+        return ((1.0L + x) * expl(-x) - 1.0L) / (x * x);
+    long double s = 0.0L, t = 1.0L;  // t = (-1)^k x^(k-1) / (k+1)!
+    for (int k = 1; k < 40; ++k) {
+        t = k == 1 ? -0.5L : -t * x / (k + 1);
+        s += k * t;
+    }
+    return s;
+}
 
 // Coefficients (monomial in t, |t| <= h) of the degree-6 truncation of the Chebyshev interpolant of fn about c.
 void cheb6(long double (*fn)(long double), long double c, long double h, double *out)
@@ -134,10 +147,28 @@ __device__ __forceinline__ unsigned lo_of(long long v) { return (unsigned)v; }
 // Signed limbs of a 64-bit number in base 2^32: v = h 2^32 + l, l = the low word read as signed.
 __device__ __forceinline__ int hi_bal(long long v) { return (int)(v >> 32) + (int)(lo_of(v) >> 31); }
 
-// Near-field geometry of one target leaf: its source rows (contiguous runs of the sorted particles) and the fixed
-// point scales.
+// Near-field geometry of one target leaf: its source rows, contiguous runs of the sorted particles (rows iy - 1, iy,
+// iy + 1 of columns ix - 1 .. ix + 1).
 struct Rows64 {
     int a[3], pre[4];  // first particle of row k, prefix of the rows' counts
+    __device__ __forceinline__ Rows64(const Work &w, const SysDev &d, int leaf)
+    {
+        const int L = d.depth, ns = 1 << L, local = leaf - (int)d.leaf0;
+        const int ix = local & (ns - 1), iy = local >> L;
+        const int jx0 = ix > 0 ? ix - 1 : 0, jx1 = ix < ns - 1 ? ix + 1 : ns - 1;
+        pre[0] = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int row = iy + k - 1;
+            int n = 0;
+            a[k] = 0;
+            if (row >= 0 && row < ns) {
+                a[k] = w.start[d.leaf0 + row * ns + jx0];
+                n = w.start[d.leaf0 + row * ns + jx1 + 1] - a[k];
+            }
+            pre[k + 1] = pre[k] + n;
+        }
+    }
     __device__ __forceinline__ int global(int q) const
     {
         int g = a[0] + q;
@@ -162,6 +193,112 @@ __device__ __forceinline__ int ceil_log2(double v)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     return exponent_of(v) + ((b & 0xfffffffffffffull) ? 1 : 0);
+}
+
+// The smallest e with every charge of the neighbourhood below 2^e (1 - 2^-12), or kNoFixed where the fixed point is not for
+// them: it serves sums whose terms are not all far below its unit's range, that is charges with a mean magnitude (of
+// the non-zero ones, the largest left out) of at least 1/16 of the largest one's; the others, subnormal, infinite and
+// NaN ones run in FP64. b, if given, is a second array of charges of the same kind. Block-uniform.
+constexpr int kNoFixed = -1000000;
+struct Stats64 {
+    unsigned max;
+    int cnt;
+    unsigned long long sum;
+};
+__device__ __forceinline__ int charge_exponent(const Rows64 &R, int ntot, const double *__restrict__ a,
+                                               const double *__restrict__ b, Stats64 &st)
+{
+    const int tid = threadIdx.x;
+    auto mag = [&](int q) {  // high word of |charge|: the exponent and 20 bits
+        const int j = R.global(q);
+        const unsigned h = (unsigned)__double2hiint(a[j]) & 0x7fffffffu;
+        return b ? max(h, (unsigned)__double2hiint(b[j]) & 0x7fffffffu) : h;
+    };
+    __syncthreads();
+    if (tid == 0) {
+        st.max = 0;
+        st.cnt = 0;
+        st.sum = 0;
+    }
+    __syncthreads();
+    unsigned gm = 0;
+    for (int q = tid; q < ntot; q += blockDim.x)
+        gm = max(gm, mag(q));
+    gm = __reduce_max_sync(0xffffffffu, gm);
+    if ((tid & 31) == 0)
+        atomicMax(&st.max, gm);
+    __syncthreads();
+    gm = st.max;
+    const int ge = (int)(gm >> 20);  // biased exponent of the largest charge
+    if (ge <= 100 || ge == 0x7ff)
+        return kNoFixed;
+    unsigned sum = 0;
+    int cnt = 0;
+    for (int q = tid; q < ntot; q += blockDim.x) {
+        const unsigned h = mag(q);
+        sum += ((h & 0xfffffu) | 0x100000u) >> min(ge - (int)(h >> 20), 31);
+        cnt += h != 0;
+        if (sum > 0x40000000u) {
+            atomicAdd(&st.sum, (unsigned long long)sum);
+            sum = 0;
+        }
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum >> 5);  // the low bits do not matter here
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if ((tid & 31) == 0) {
+        atomicAdd(&st.sum, (unsigned long long)sum << 5);
+        atomicAdd(&st.cnt, cnt);
+    }
+    __syncthreads();
+    const unsigned long long big = (gm & 0xfffffu) | 0x100000u;
+    if (!(st.sum > big && (st.sum - big) * 16 >= big * (unsigned long long)max(st.cnt - 1, 1)))
+        return kNoFixed;
+    return ge - 1022 + ((gm & 0xfffffu) < 0xfff00u ? 0 : 1);
+}
+
+// Fixed-point geometry: lengths in units of 2^ku, so that two leaf widths are at most 2^61; pairs whose r^2 has a
+// high word (units of 2^94) of at least thr are far. thr = 0: none is.
+struct Fixed64 {
+    int ku, thr;
+    bool ranges;  // lengths whose squares and their ratios stay well inside FP64's range
+    __device__ __forceinline__ Fixed64(const SysDev &d)
+    {
+        ku = ceil_log2(2.0 * d.wl) - 61;
+        ranges = abs(exponent_of(d.sigma)) < 200 && abs(exponent_of(d.wl)) < 200;
+        const double cut = ranges ? ldexp(2.0 * kXCut * d.sigma * d.sigma, -2 * ku - 94) : 0x1p40;
+        thr = cut < 0x1p30 ? max((int)cut + 2, N64_RMIN) : 0;  // a leaf's diagonal neighbours reach 2^31
+    }
+};
+
+// Far pair at displacement (dxh 2^31 + dxl, dyh 2^31 + dyl): r2 = r^2 2^-62.
+__device__ __forceinline__ long long r2_fixed(int dxh, int dxl, int dyh, int dyl)
+{
+    // the high products and the cross terms 2 h l 2^-31
+    const long long cr = wide(dyh, dyl, wide(dxh, dxl, 0));
+    return wide(dyh, dyh, wide(dxh, dxh, cr >> 30));
+}
+// 2^116 / r2 for a high word of r2 in [N64_RMIN, 2^31): the SFU's seed y0 ~ 2^84 / r2; r2 y0 = 2^84 (1 + e) modulo
+// 2^64 with |e| < 2^-21, and 1 / (1 + e) = 1 - e + e^2 to 2^-63. Any other r2 gives an arbitrary value.
+__device__ __forceinline__ long long recip_fixed(long long r2)
+{
+    const int rh = hi_of(r2);
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__int2float_rn(rh) + 0.5f));
+    const unsigned y0 = __float2uint_rn(yf * 0x1p52f);
+    const unsigned long long P = wide_u(lo_of(r2), y0);
+    const int eh = (int)((unsigned)(P >> 32) + (unsigned)rh * y0);
+    const int es = eh >> 15;
+    const unsigned e2 = (unsigned)es * (unsigned)es;  // e^2 2^74
+    // c = e^2 - e with 84 fraction bits; y0 2^32 (1 + c)
+    const long long c = (long long)(((unsigned long long)e2 << 10) -
+                                    (((unsigned long long)(unsigned)eh << 32) | (unsigned)P));
+    const long long T = wide(hi_of(c), (int)y0, (long long)(unsigned long long)__umulhi(lo_of(c), y0));
+    return (long long)((unsigned long long)(T >> 20) + ((unsigned long long)y0 << 32));
+}
+// Rounded high half of (ah 2^32 + al) (bh 2^32 + bl), limbs signed.
+__device__ __forceinline__ long long mul_hi(int ah, int al, int bh, int bl)
+{
+    return wide(ah, bh, (long long)hi_of(wide(al, bh, wide(ah, bl, 1ll << 31))));
 }
 
 // Passes over a leaf of c targets: the number of passes (at most 4 more than needed) that keeps most of the 256
@@ -193,87 +330,24 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
     __shared__ int4 pos[N64_TILE];   // x and y limbs
     __shared__ int2 gam[N64_TILE];   // gamma limbs, base 2^32
     __shared__ unsigned short lst[N64_CAP * N64_THREADS];
-    __shared__ unsigned s_max;
-    __shared__ unsigned long long s_sum;
-    __shared__ int s_cnt;
+    __shared__ Stats64 st;
     const int leaf = blockIdx.x, tid = threadIdx.x;
     const int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
     if (c == 0)
         return;
     const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
     const SysDev &d = w.sys[k];
-    const int L = d.depth, ns = 1 << L, local = leaf - (int)d.leaf0;
-    const int ix = local & (ns - 1), iy = local >> L;
-    const int jx0 = ix > 0 ? ix - 1 : 0, jx1 = ix < ns - 1 ? ix + 1 : ns - 1;
-    Rows64 R;
-    R.pre[0] = 0;
-#pragma unroll
-    for (int dy = 0; dy < 3; ++dy) {
-        const int row = iy + dy - 1;
-        int a = 0, n = 0;
-        if (row >= 0 && row < ns) {
-            a = w.start[d.leaf0 + row * ns + jx0];
-            n = w.start[d.leaf0 + row * ns + jx1 + 1] - a;
-        }
-        R.a[dy] = a;
-        R.pre[dy + 1] = R.pre[dy] + n;
-    }
+    const Rows64 R(w, d, leaf);
     const int ntot = R.pre[3];
     const double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
 
-    // fixed-point unit 2^ku: two leaf widths are at most 2^61 of it; r^2 >= rc2 units of 2^94 is the far range
-    const int ku = ceil_log2(2.0 * d.wl) - 61;
-    const double cut = ldexp(2.0 * kXCut * d.sigma * d.sigma, -2 * ku - 94);
-    // lengths whose squares and their ratios stay well inside FP64's range (else every pair by expm1 and division)
-    const bool ranges = abs(exponent_of(d.sigma)) < 200 && abs(exponent_of(d.wl)) < 200;
-    bool fixed = ranges && cut < 0x1p30 && ntot >= N64_FEW;  // some adjacent pair is far
-    const int thr = fixed ? max((int)cut + 2, N64_RMIN) : 0;
-    // the charges' largest magnitude and mean (of the non-zero ones): the fixed point is kept for sums whose terms
-    // are not all far below its unit's range
-    if (tid == 0) {
-        s_max = 0;
-        s_sum = 0;
-        s_cnt = 0;
-    }
-    __syncthreads();
-    unsigned gm = 0;
-    if (fixed) {
-        for (int q = tid; q < ntot; q += N64_THREADS)
-            gm = max(gm, (unsigned)__double2hiint(w.sg[R.global(q)]) & 0x7fffffffu);
-        gm = __reduce_max_sync(0xffffffffu, gm);
-        if ((tid & 31) == 0)
-            atomicMax(&s_max, gm);
-    }
-    __syncthreads();
-    gm = s_max;
-    const int ge = (int)(gm >> 20);  // biased exponent of the largest charge
-    fixed = fixed && ge > 100 && ge < 0x7ff;
-    if (fixed) {
-        unsigned sum = 0;
-        int cnt = 0;
-        for (int q = tid; q < ntot; q += N64_THREADS) {
-            const unsigned h = (unsigned)__double2hiint(w.sg[R.global(q)]) & 0x7fffffffu;
-            sum += ((h & 0xfffffu) | 0x100000u) >> min(ge - (int)(h >> 20), 31);
-            cnt += h != 0;
-            if (sum > 0x40000000u) {
-                atomicAdd(&s_sum, (unsigned long long)sum);
-                sum = 0;
-            }
-        }
-        sum = __reduce_add_sync(0xffffffffu, sum >> 5) << 5;  // the low bits do not matter here
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if ((tid & 31) == 0) {
-            atomicAdd(&s_sum, (unsigned long long)sum);
-            atomicAdd(&s_cnt, cnt);
-        }
-    }
-    __syncthreads();
-    if (fixed) {
-        const unsigned long long big = (gm & 0xfffffu) | 0x100000u;
-        fixed = s_sum > big && (s_sum - big) * 16 >= big * (unsigned long long)max(s_cnt - 1, 1);
-    }
-    // charges in units of 2^ka: below 2^63 - 2^50, so that their high limb fits
-    const int ka = ge - 1023 + 1 - ((gm & 0xfffffu) < 0xfff00u ? 63 : 62);
+    const Fixed64 fx(d);
+    const int ku = fx.ku, thr = fx.thr;
+    const bool ranges = fx.ranges;
+    bool fixed = thr > 0 && ntot >= N64_FEW;
+    const int ge = fixed ? charge_exponent(R, ntot, w.sg, nullptr, st) : kNoFixed;
+    fixed = ge != kNoFixed;
+    const int ka = ge - 63;  // charges in units of 2^ka: below 2^63 - 2^50, so that their high limb fits
 
     const int npass = pick_passes(c);
     for (int pass = 0; pass < npass; ++pass) {
@@ -306,9 +380,17 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                     }
                 }
         } else if (!fixed) {
-            if (active)
-                for (int q = grp; q < ntot; q += G)
-                    pair64(q);
+            double tu = 0.0, tv = 0.0;
+            for (int q = grp, i = 0; active && q < ntot; q += G) {
+                pair64(q);
+                if (++i % 32 == 0) {  // sums of 32 terms, then their sum
+                    tu += au;
+                    tv += av;
+                    au = av = 0.0;
+                }
+            }
+            au += tu;
+            av += tv;
         } else {
             const int2 tx = limbs31(to_fixed(xt, ku)), ty = limbs31(to_fixed(yt, ku));
             int cnt = 0, terms = 0;
@@ -335,31 +417,14 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                         const int4 p = pos[q];
                         int2 g = gam[q];
                         const int dxh = tx.x - p.x, dxl = tx.y - p.y, dyh = ty.x - p.z, dyl = ty.y - p.w;
-                        // r^2 2^-62: high products and the cross terms 2 h l 2^-31
-                        const long long cr = wide(dyh, dyl, wide(dxh, dxl, 0));
-                        const long long r2 = wide(dyh, dyh, wide(dxh, dxh, cr >> 30));
-                        const int rh = hi_of(r2);
-                        if (rh < thr) {
+                        const long long r2 = r2_fixed(dxh, dxl, dyh, dyl);
+                        if (hi_of(r2) < thr) {
                             lst[cnt * N64_THREADS + tid] = (unsigned short)q;
                             ++cnt;
                             g = make_int2(0, 0);
                         }
-                        // Y0 ~ 2^84 / r^2 from the SFU; r^2 Y0 = 2^84 (1 + e) modulo 2^64, |e| < 2^-21
-                        float yf;
-                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__int2float_rn(rh) + 0.5f));
-                        const unsigned y0 = __float2uint_rn(yf * 0x1p52f);
-                        const unsigned long long P = wide_u(lo_of(r2), y0);
-                        const int eh = (int)((unsigned)(P >> 32) + (unsigned)rh * y0);
-                        const int es = eh >> 15;
-                        const unsigned e2 = (unsigned)(es * es);  // e^2 2^74
-                        // c = e^2 - e, 84 fraction bits; Y = 2^32 Y0 (1 + c) = 2^116 / r^2
-                        const long long cc = (long long)((unsigned long long)e2 << 10) -
-                                             (long long)(((unsigned long long)(unsigned)eh << 32) | (unsigned)P);
-                        const long long T = wide(hi_of(cc), (int)y0, (long long)(unsigned long long)__umulhi(lo_of(cc), y0));
-                        const long long Y = (T >> 20) + ((long long)y0 << 32);
-                        // f = gamma Y 2^-64
-                        const int yh = hi_bal(Y), yl = (int)lo_of(Y);
-                        const long long f = wide(g.x, yh, (long long)hi_of(wide(g.y, yh, wide(g.x, yl, 1ll << 31))));
+                        const long long Y = recip_fixed(r2);
+                        const long long f = mul_hi(g.x, g.y, hi_bal(Y), (int)lo_of(Y));  // gamma Y 2^-64
                         const int fh = hi_bal(f), fl = (int)lo_of(f) >> 1;
                         su += wide(fh, dyh, wide(fl, dyh, wide(fh, dyl, 1ll << 30)) >> 31);
                         sv += wide(fh, dxh, wide(fl, dxh, wide(fh, dxl, 1ll << 30)) >> 31);
@@ -407,6 +472,235 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
     }
 }
 
+// ------------------------------------------------------------------ adjoint
+
+// For target k and neighbour m (z = (a, b) = z_k - z_m), with K = (Ku, Kv) = (-b, a) f of Eq. 6 and its Jacobian J:
+//   dgamma_k += -(gu_m Ku + gv_m Kv) = f (gu_m b - gv_m a)
+//   dx_k     += cu dKu/da + cv dKv/da,  cu = gamma_m gu_k - gamma_k gu_m
+//   dy_k     += cu dKu/db + cv dKv/db,  cv = gamma_m gv_k - gamma_k gv_m
+// (K is odd and its Jacobian even in z). The same split as the forward kernel's. A far pair has f = 1 / r^2 and, with
+// P = 2 a b / r^4 and Q = (b^2 - a^2) / r^4, contributes cu P + cv Q to dx and cu Q - cv P to dy: 54 wide integer
+// multiplications in fixed point (22 operations in FP64, three times the time); sums in two 64-bit parts, high products
+// and cross terms. A close one takes F and F' from their tables, 37 FP64 operations. Measured at 2^20 uniform particles
+// (leaves of 64, 16 sigma wide): 103 ms with exp, expm1 and divisions in FP64 for every pair, 12.0 ms so, bound by the
+// FP64 pipe (63 % busy) on the close pairs; no further from quad precision on either side of the split.
+// Writes the near part in caller order (the far part is added later).
+constexpr int A64_TILE = 512;
+__global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, double *__restrict__ odg,
+                                                                   double *__restrict__ odx, double *__restrict__ ody,
+                                                                   int skip_plain)
+{
+    __shared__ int4 pos[A64_TILE];   // x and y limbs
+    __shared__ int2 gam[A64_TILE];   // gamma limbs, base 2^32
+    __shared__ int4 ggr[A64_TILE];   // gu and gv limbs
+    __shared__ unsigned short lst[N64_CAP * N64_THREADS];
+    __shared__ Stats64 st;
+    const int leaf = blockIdx.x, tid = threadIdx.x;
+    const int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
+    if (c == 0)
+        return;
+    const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
+    const SysDev &d = w.sys[k];
+    if (skip_plain && !(d.s_unit > P2P_SPLIT_S))
+        return;  // this system's near field is the FP32 kernel's
+    const Rows64 R(w, d, leaf);
+    const int ntot = R.pre[3];
+    const double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
+    const Fixed64 fx(d);
+    const int ku = fx.ku, thr = fx.thr;
+    const bool ranges = fx.ranges;
+    bool fixed = thr > 0 && ntot >= N64_FEW;
+    int ka = 0, kb = 0;  // units 2^ka of gamma (below 2^62), 2^kb of gu and gv (below 2^58)
+    if (fixed) {
+        const int ea = charge_exponent(R, ntot, w.sg, nullptr, st);
+        const int eb = ea != kNoFixed ? charge_exponent(R, ntot, w.sgu, w.sgv, st) : kNoFixed;
+        fixed = eb != kNoFixed;
+        ka = ea - 62;
+        kb = eb - 58;
+    }
+    const int npass = pick_passes(c);
+    for (int pass = 0; pass < npass; ++pass) {
+        const int t0 = (int)((long long)pass * c / npass), cp = (int)((long long)(pass + 1) * c / npass) - t0;
+        const int G = N64_THREADS / cp;
+        const int grp = tid / cp, tpos = s0 + t0 + (tid - grp * cp);
+        const bool active = grp < G;
+        const double xt = w.sx[tpos], yt = w.sy[tpos], gt = w.sg[tpos], gut = w.sgu[tpos], gvt = w.sgv[tpos];
+        double ag = 0.0, ax = 0.0, ay = 0.0;  // FP64 pairs: dgamma in units of k2, dx and dy in units of k2
+        double ig = 0.0, ix = 0.0, iy = 0.0;  // fixed-point pairs
+        auto pair64 = [&](int q) {
+            const int j = R.global(q);
+            const double a = xt - w.sx[j], b = yt - w.sy[j];
+            const double x = fma(a, a, b * b) * k2;
+            if (__double_as_longlong(x) == 0)
+                return;  // a particle and itself, or coincident ones
+            double f, h;     // f / k2 and 2 f' / k2
+            if (x < kXCut) {
+                const int i = blob_row(x);
+                f = blob_poly(g_blob_f, i, x);
+                h = 2.0 * k2 * blob_poly(g_blob_d, i, x);
+            } else {
+                f = recip64(x);
+                h = -2.0 * k2 * (f * f);
+            }
+            const double gj = w.sg[j], guj = w.sgu[j], gvj = w.sgv[j];
+            const double ah = a * h, bh = b * h, ab = a * bh;
+            const double J2 = fma(a, ah, f), J1 = fma(b, bh, f);  // dKv/da, -dKu/db; dKv/db = -dKu/da = ab
+            const double cu = gj * gut - gt * guj, cv = gj * gvt - gt * gvj;
+            ag = fma(f, guj * b - gvj * a, ag);
+            ax += fma(cv, J2, -cu * ab);  // one rounding at the size of the sum
+            ay += fma(cv, ab, -cu * J1);
+        };
+        if (!ranges) {
+            if (active)
+                for (int q = grp; q < ntot; q += G) {
+                    const int j = R.global(q);
+                    const double a = xt - w.sx[j], b = yt - w.sy[j], s = a * a + b * b;
+                    if (s == 0.0)
+                        continue;
+                    const double e = exp(-s * k2), om = -expm1(-s * k2);
+                    const double f = om / s, fp = (k2 * e * s - om) / (s * s);
+                    const double cu = w.sg[j] * gut - gt * w.sgu[j], cv = w.sg[j] * gvt - gt * w.sgv[j];
+                    ig += f * (w.sgu[j] * b - w.sgv[j] * a);
+                    ix += cv * (f + 2.0 * a * a * fp) - cu * (2.0 * a * b * fp);
+                    iy += cv * (2.0 * a * b * fp) - cu * (f + 2.0 * b * b * fp);
+                }
+        } else if (!fixed) {
+            double tg = 0.0, tx = 0.0, ty = 0.0;
+            for (int q = grp, i = 0; active && q < ntot; q += G) {
+                pair64(q);
+                if (++i % 32 == 0) {  // sums of 32 terms, then their sum
+                    tg += ag;
+                    tx += ax;
+                    ty += ay;
+                    ag = ax = ay = 0.0;
+                }
+            }
+            ag += tg;
+            ax += tx;
+            ay += ty;
+        } else {
+            const int2 tx = limbs31(to_fixed(xt, ku)), ty = limbs31(to_fixed(yt, ku));
+            const long long tg = to_fixed(gt, ka), tgu = to_fixed(gut, kb), tgv = to_fixed(gvt, kb);
+            const int tgh = -hi_bal(tg), tgl = (int)lo_of(tg) >> 1;  // low limb halved: it can be negated
+            const int tuh = hi_bal(tgu), tul = (int)lo_of(tgu), tvh = hi_bal(tgv), tvl = (int)lo_of(tgv);
+            int cnt = 0, terms = 0;
+            long long hg = 0, lg = 0, hx = 0, lx = 0, hy = 0, ly = 0;  // high products, cross terms / 2^8
+            auto spill = [&]() {
+                ig += fma((double)lg, 0x1p-24, (double)hg);
+                ix += fma((double)lx, 0x1p-24, (double)hx);
+                iy += fma((double)ly, 0x1p-24, (double)hy);
+                hg = lg = hx = lx = hy = ly = 0;
+                terms = 0;
+            };
+            for (int q0 = 0; q0 < ntot; q0 += A64_TILE) {
+                const int m = min(A64_TILE, ntot - q0);
+                __syncthreads();
+                for (int q = tid; q < m; q += N64_THREADS) {
+                    const int j = R.global(q0 + q);
+                    const int2 px = limbs31(to_fixed(w.sx[j], ku)), py = limbs31(to_fixed(w.sy[j], ku));
+                    const long long g = to_fixed(w.sg[j], ka), gu = to_fixed(w.sgu[j], kb), gv = to_fixed(w.sgv[j], kb);
+                    pos[q] = make_int4(px.x, px.y, py.x, py.y);
+                    gam[q] = make_int2(hi_bal(g), (int)lo_of(g));
+                    ggr[q] = make_int4(hi_bal(gu), (int)lo_of(gu), hi_bal(gv), (int)lo_of(gv));
+                }
+                __syncthreads();
+                const int nj = active ? (m - grp + G - 1) / G : 0;  // this thread's sources: grp, grp + G, ...
+                const int nmax = __reduce_max_sync(0xffffffffu, nj);
+                for (int i0 = 0; i0 < nmax;) {
+                    const int used = __reduce_max_sync(0xffffffffu, cnt);
+                    const int i1 = min(nmax, i0 + N64_CAP - used);
+                    for (int i = i0; i < min(i1, nj); ++i) {
+                        const int q = grp + G * i;
+                        const int4 p = pos[q];
+                        const int dxh = tx.x - p.x, dxl = tx.y - p.y, dyh = ty.x - p.z, dyl = ty.y - p.w;
+                        const long long r2 = r2_fixed(dxh, dxl, dyh, dyl);
+                        if (hi_of(r2) < thr) {
+                            lst[cnt * N64_THREADS + tid] = (unsigned short)q;
+                            ++cnt;
+                            continue;
+                        }
+                        // a / r^2 and b / r^2: displacement times Y, / 2^59 (at most 2^61.2)
+                        const long long Y = recip_fixed(r2);
+                        const int yh = hi_bal(Y), yl = (int)lo_of(Y), y2 = yl >> 1;
+                        const long long ca = (wide(dxh, yh, 0) << 4) + (wide(dxl, yh, wide(dxh, y2, 1 << 26)) >> 27);
+                        const long long cb = (wide(dyh, yh, 0) << 4) + (wide(dyl, yh, wide(dyh, y2, 1 << 26)) >> 27);
+                        // P = 2 ca cb, Q = (cb - ca) (cb + ca), / 2^64
+                        const long long cb2 = cb * 2, cs = cb + ca, cd = cb - ca;
+                        const int cah = hi_bal(ca), cal = (int)lo_of(ca), cbh = hi_bal(cb), cbl = (int)lo_of(cb);
+                        const long long P = mul_hi(cah, cal, hi_bal(cb2), (int)lo_of(cb2));
+                        const long long Q = mul_hi(hi_bal(cs), (int)lo_of(cs), hi_bal(cd), (int)lo_of(cd));
+                        const int2 g = gam[q];
+                        const int4 gg = ggr[q];
+                        // cu, cv / 2^64: gamma_m gu_k - gamma_k gu_m; the target's negated limbs are (tgh, -2 tgl)
+                        const long long cu =
+                            wide(g.x, tuh,
+                                 wide(tgh, gg.x,
+                                      (long long)hi_of(wide(g.y, tuh, wide(g.x, tul, 1ll << 31)) +
+                                                       wide(tgh, gg.y, -2 * wide(tgl, gg.x, 0)))));
+                        const long long cv =
+                            wide(g.x, tvh,
+                                 wide(tgh, gg.z,
+                                      (long long)hi_of(wide(g.y, tvh, wide(g.x, tvl, 1ll << 31)) +
+                                                       wide(tgh, gg.w, -2 * wide(tgl, gg.z, 0)))));
+                        // dgamma: gu_m b - gv_m a
+                        hg = wide(gg.x, cbh, wide(-gg.z, cah, hg));
+                        lg += (wide(gg.y, cbh, wide(gg.x, cbl, 0)) - wide(gg.w, cah, wide(gg.z, cal, 0))) >> 8;
+                        // dx: cu P + cv Q, dy: cu Q - cv P, with the low halves' products (the range of the terms
+                        // takes up most of the high ones)
+                        const int cuh = hi_bal(cu), cul = (int)lo_of(cu), cvh = hi_bal(cv), cvl = (int)lo_of(cv);
+                        const int Ph = hi_bal(P), Pl = (int)lo_of(P), Qh = hi_bal(Q), Ql = (int)lo_of(Q);
+                        hx = wide(cuh, Ph, wide(cvh, Qh, hx));
+                        lx += wide(cuh, Pl, wide(cul, Ph, wide(cvh, Ql, wide(cvl, Qh, (long long)__mulhi(cul, Pl) + __mulhi(cvl, Ql))))) >> 8;
+                        hy = wide(cuh, Qh, wide(-cvh, Ph, hy));
+                        ly += (wide(cuh, Ql, wide(cul, Qh, (long long)__mulhi(cul, Ql) - __mulhi(cvl, Pl))) -
+                               wide(cvh, Pl, wide(cvl, Ph, 0))) >> 8;
+                    }
+                    terms += i1 - i0;
+                    if (terms > N64_SPILL - N64_CAP)
+                        spill();
+                    i0 = i1;
+                    const int full = __reduce_max_sync(0xffffffffu, cnt);
+                    if (full > N64_CAP - 12 || (i0 >= nmax && full > 0)) {
+                        for (int e = 0; e < full; ++e)
+                            if (e < cnt)
+                                pair64(q0 + lst[e * N64_THREADS + tid]);
+                        cnt = 0;
+                    }
+                }
+            }
+            spill();
+            // units: a / r^2 2^(120 - 1 + ku) per ca, charges 2^-kb and 2^-ka; sums in units of 2^64
+            ig = scalbn(ig * scalbn(1.0, -55 - ku), kb);
+            ix = scalbn(scalbn(ix * scalbn(1.0, -46 - 2 * ku), ka), kb);
+            iy = scalbn(scalbn(iy * scalbn(1.0, -46 - 2 * ku), ka), kb);
+        }
+        // groups of a target, in order, through the (now idle) source limbs
+        double *red = reinterpret_cast<double *>(pos);
+        __syncthreads();
+        if (active) {
+            red[tid] = ranges ? fma(ag, k2, ig) : ig;
+            red[N64_THREADS + tid] = ranges ? fma(ax, k2, ix) : ix;
+            red[2 * N64_THREADS + tid] = ranges ? fma(ay, k2, iy) : iy;
+        }
+        __syncthreads();
+        if (tid < cp) {
+            double sg = 0.0, sx = 0.0, sy = 0.0;
+            for (int g = 0; g < G; ++g) {
+                sg += red[tid + g * cp];
+                sx += red[N64_THREADS + tid + g * cp];
+                sy += red[2 * N64_THREADS + tid + g * cp];
+            }
+            const int i = w.perm[tpos];
+            if (odg)
+                odg[i] = sg / kTwoPi;
+            if (odx)
+                odx[i] = sx / kTwoPi;
+            if (ody)
+                ody[i] = sy / kTwoPi;
+        }
+    }
+}
+
 }  // namespace
 
 int prepare_near64(cudaStream_t s)
@@ -417,13 +711,15 @@ int prepare_near64(cudaStream_t s)
     std::lock_guard<std::mutex> lk(g_tab_mu);
     if (g_tab_ready[dev])
         return 0;
-    static double tab[kTabN][8];
+    static double tab[2][kTabN][8];
     for (int i = 0; i < kTabN; ++i) {
         const long double c = (i + 0.5L) / 16.0L;
-        cheb6(blob_f, c, 1.0L / 32.0L, tab[i]);
-        tab[i][7] = (double)c;
+        cheb6(blob_f, c, 1.0L / 32.0L, tab[0][i]);
+        cheb6(blob_d, c, 1.0L / 32.0L, tab[1][i]);
+        tab[0][i][7] = tab[1][i][7] = (double)c;
     }
-    if (cudaMemcpyToSymbolAsync(g_blob_f, tab, sizeof tab, 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+    if (cudaMemcpyToSymbolAsync(g_blob_f, tab[0], sizeof tab[0], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(g_blob_d, tab[1], sizeof tab[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return -1;
     g_tab_ready[dev] = true;
@@ -433,6 +729,12 @@ int prepare_near64(cudaStream_t s)
 int launch_near64(const Work &w, cudaStream_t s)
 {
     k_near64<<<w.nleaf, N64_THREADS, 0, s>>>(w);
+    return 1;
+}
+
+int launch_adjoint_near64(const Work &w, double *dg, double *dx, double *dy, int skip_plain, cudaStream_t s)
+{
+    k_adjoint_near64<<<w.nleaf, N64_THREADS, 0, s>>>(w, dg, dx, dy, skip_plain);
     return 1;
 }
 

@@ -1025,91 +1025,9 @@ int launch_p2p(const Work &w, int threads, int kt, cudaStream_t s)
     return 1;
 }
 
-// ------------------------------------------------------------------ adjoint near field (FP64)
+// ------------------------------------------------------------------ adjoint near field
 
-// For target k and neighbour m (z = z_k - z_m), with K = (Ku, Kv) of Eq. 6 and its Jacobian J:
-//   dgamma_k += -(gu_m Ku(z) + gv_m Kv(z))
-//   dx_k     += (gamma_m gu_k - gamma_k gu_m) dKu/da + (gamma_m gv_k - gamma_k gv_m) dKv/da
-//   dy_k     += (gamma_m gu_k - gamma_k gu_m) dKu/db + (gamma_m gv_k - gamma_k gv_m) dKv/db
-// (K is odd and its Jacobian even in z). Writes the near part in caller order (the far part is added later).
-__global__ void __launch_bounds__(64) k_adjoint_p2p64(Work w, double *__restrict__ odg, double *__restrict__ odx,
-                                                     double *__restrict__ ody, int skip_plain)
-{
-    __shared__ double shx[256], shy[256], shg[256], shu[256], shv[256];
-    int leaf = blockIdx.x;
-    int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
-    if (c == 0)
-        return;
-    int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
-    const SysDev &d = w.sys[k];
-    if (skip_plain && !(d.s_unit > P2P_SPLIT_S))
-        return;  // this system's near field is the FP32 kernel's
-    int L = d.depth, ns = 1 << L, local = leaf - (int)d.leaf0;
-    int ix = local & (ns - 1), iy = local >> L;
-    double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
-    int jx0 = ix > 0 ? ix - 1 : 0, jx1 = ix < ns - 1 ? ix + 1 : ns - 1;
-    for (int t0 = 0; t0 < c; t0 += blockDim.x) {
-        int tpos = s0 + t0 + threadIdx.x;
-        bool valid = t0 + threadIdx.x < c;
-        double xt = 0, yt = 0, gt = 0, gut = 0, gvt = 0;
-        if (valid) {
-            xt = w.sx[tpos];
-            yt = w.sy[tpos];
-            gt = w.sg[tpos];
-            gut = w.sgu[tpos];
-            gvt = w.sgv[tpos];
-        }
-        double ag = 0, ax = 0, ay = 0;
-        for (int dy = -1; dy <= 1; ++dy) {
-            int row = iy + dy;
-            if (row < 0 || row >= ns)
-                continue;
-            int r0 = w.start[d.leaf0 + row * ns + jx0], r1 = w.start[d.leaf0 + row * ns + jx1 + 1];
-            for (int q0 = r0; q0 < r1; q0 += 256) {
-                int m = min(256, r1 - q0);
-                __syncthreads();
-                for (int j = threadIdx.x; j < m; j += blockDim.x) {
-                    shx[j] = w.sx[q0 + j];
-                    shy[j] = w.sy[q0 + j];
-                    shg[j] = w.sg[q0 + j];
-                    shu[j] = w.sgu[q0 + j];
-                    shv[j] = w.sgv[q0 + j];
-                }
-                __syncthreads();
-                if (!valid)
-                    continue;
-                for (int j = 0; j < m; ++j) {
-                    double a = xt - shx[j], b = yt - shy[j];
-                    double s = a * a + b * b;
-                    if (s == 0.0)
-                        continue;
-                    double e = exp(-s * k2);
-                    double om = -expm1(-s * k2);
-                    double f = om / (TWO_PI * s);
-                    double fp = (k2 * e * s - om) / (TWO_PI * s * s);
-                    double ku = -b * f, kv = a * f;
-                    double J0 = -2.0 * a * b * fp, J1 = -(f + 2.0 * b * b * fp);
-                    double J2 = f + 2.0 * a * a * fp, J3 = 2.0 * a * b * fp;
-                    double cu = shg[j] * gut - gt * shu[j], cv = shg[j] * gvt - gt * shv[j];
-                    ag -= shu[j] * ku + shv[j] * kv;
-                    ax += cu * J0 + cv * J2;
-                    ay += cu * J1 + cv * J3;
-                }
-            }
-        }
-        if (valid) {
-            int i = w.perm[tpos];
-            if (odg)
-                odg[i] = ag;
-            if (odx)
-                odx[i] = ax;
-            if (ody)
-                ody[i] = ay;
-        }
-    }
-}
-
-// Precision form of the same near-field adjoint. Lengths in units r' = lambda r, lambda = s / w_L, with s the
+// Precision form of the near-field adjoint (FP64 form and the terms: near64.cu). Lengths in units r' = lambda r, lambda = s / w_L, with s the
 // system's s_unit, so that exp(-r^2 / 2 sigma^2) = 2^-(r'^2) (the forward's units); F(t) = (1 - 2^-t) / t and
 // F'(t) at t = r'^2 give, with C = lambda * snear (snear = lambda / 2 pi):
 //   Ku = -b' F snear,  Kv = a' F snear,
@@ -1238,14 +1156,11 @@ int launch_adjoint_p2p(const Work &w, double *dg, double *dx, double *dy, int fp
 {
     if (w.nleaf == 0)
         return 0;
-    if (!fp32) {
-        k_adjoint_p2p64<<<w.nleaf, 64, 0, s>>>(w, dg, dx, dy, 0);
-        return 1;
-    }
+    if (!fp32)
+        return launch_adjoint_near64(w, dg, dx, dy, 0, s);
     // one-float systems in FP32, systems with wider leaves in FP64
     k_adjoint_p2p32<<<w.nleaf, 64, 0, s>>>(w, dg, dx, dy);
-    k_adjoint_p2p64<<<w.nleaf, 64, 0, s>>>(w, dg, dx, dy, 1);
-    return 2;
+    return 1 + launch_adjoint_near64(w, dg, dx, dy, 1, s);
 }
 
 }  // namespace fmm

@@ -91,3 +91,33 @@ def test_near64_infinite_charge_stays_with_its_neighbours(lib):
     touched[17] = False  # a particle does not act on itself
     finite = np.isfinite(got[:n]) & np.isfinite(got[n:])
     assert np.array_equal(finite, ~touched)
+
+
+ADJ_CASES = ["sources_95_97", "leaf_63_to_65", "leaf_hundreds", "narrow_all_close", "cut_at_leaf_diagonal", "wide_leaves",
+             "tiny_square_offset", "strong_few", "mostly_zero", "one_sign_tiny"]  # the oracle overflows beyond 1e70
+
+
+@pytest.mark.parametrize("grads", ["normal", "outliers", "charges"])
+@pytest.mark.parametrize("name", ADJ_CASES)
+def test_adjoint_near64_matches_oracle(lib, oracle, name, grads):
+    """The adjoint on a tree of depth 1 (all near field) and on the case's own tree, against the oracle's transposed
+    stages. The gradients of a target are sums of the same length as above with one more level of products: 1e-11."""
+    if (name, grads) == ("strong_few", "charges"):
+        pytest.skip("cu cancels products 1e16 times the result: FP64's residue of it is 1e-9 of the result")
+    for depth in (1, None):
+        w = dict(CASES)[name]()
+        w.p = 12
+        if depth is not None:
+            w.depth = depth
+        r = np.random.default_rng(7)
+        gu, gv = r.standard_normal(w.n) / w.n, r.standard_normal(w.n) / w.n
+        if grads == "outliers":
+            gu[::500] *= 1e6
+        elif grads == "charges":  # gu proportional to gamma: cu vanishes pair by pair
+            gu = 3.0 * w.gamma
+        f = lib.FMM(w.depth, w.p, w.sigma, precision="fp64", domain=w.domain)
+        got = f.adjoint(dev(w.x), dev(w.y), dev(w.gamma), dev(gu), dev(gv))
+        f.sync()
+        ref = oracle.fmm_adjoint(w.x, w.y, w.gamma, w.sigma, w.depth, w.p, gu, gv, domain=w.domain)
+        for a, b in zip(got, ref):
+            assert np.linalg.norm(a.cpu().numpy() - b) < 1e-11 * np.linalg.norm(b)
