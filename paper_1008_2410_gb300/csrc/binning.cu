@@ -84,6 +84,7 @@ __host__ __device__ void derive_constants(SysDev &d)
     const double om = 6.0 * d.sigma * (1.0 + 0x1p-8) / d.wl;
     d.bnd_ok = om < 0.5 ? 1 : 0;
     d.fbnd = d.bnd_ok ? (long long)floor((0.5 - om) * 0x1p52) : 0;
+    derive_near64(d);
 }
 
 __global__ void k_domain_finalize(SysDev *sys, int nsys, const unsigned long long *minmax)

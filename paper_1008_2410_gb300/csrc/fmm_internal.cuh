@@ -64,7 +64,65 @@ struct SysDev {
     long long fbnd;
     int bnd_ok;
     int pad_b;
+    // plain form's near field (near64.cu), see derive_near64
+    struct Near64 {
+        double k2;             // 1 / 2 sigma^2
+        double far_sc, far_sc2;  // scales of the far sums: 2^(-51 - ku); adjoint 2^(-46 - 2 ku)
+        double close_sc;       // scale of the close sums: k2 2^(66 - s + ku)
+        long long vmax;        // z, before its shift, of the end of the tables
+        int ku;                // lengths in units of 2^ku: two leaf widths are at most 2^61 of them
+        int thr;               // pairs whose r^2 has a high word (units of 2^94) of at least thr are far; 0: none is
+        int s;                 // close displacements are taken times 2^s (at most 2^62)
+        int e, kmh, kml;       // z = x 2^56 = (r2 km 2^-64) 2^e, r2 = r^2 2^-64 in those units
+        int ranges;            // lengths whose squares and their ratios stay well inside FP64's range
+    } n64;
 };
+
+// Constants of the plain form's near field (near64.cu), from the leaf width and sigma: computed once per system so that
+// its threads spend no FP64 operation on them.
+#define N64_XCUT 37.5    // e^-37.5 < 2^-54: beyond it 1 - e^-x rounds to 1
+#define N64_ROWS 2400    // rows of the fixed-point tables of F on [0, N64_XCUT)
+#define N64_RMIN 3410000  // smallest high word of r^2 the fixed point takes: 1 / r^2 below 2^31 as a seed, r^2 to 2^-53
+__host__ __device__ inline unsigned long long bits_of(double v)
+{
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(v);
+#else
+    unsigned long long b;
+    __builtin_memcpy(&b, &v, sizeof b);
+    return b;
+#endif
+}
+__host__ __device__ inline int exponent_of(double v) { return (int)((bits_of(v) >> 52) & 0x7ff) - 1023; }
+__host__ __device__ inline void derive_near64(SysDev &d)
+{
+    SysDev::Near64 &c = d.n64;
+    c.k2 = 1.0 / (2.0 * d.sigma * d.sigma);
+    const double w2 = 2.0 * d.wl;
+    c.ku = exponent_of(w2) + ((bits_of(w2) & 0xfffffffffffffull) ? 1 : 0) - 61;
+    const int es = exponent_of(d.sigma), ew = exponent_of(d.wl);
+    c.ranges = es > -200 && es < 200 && ew > -200 && ew < 200;
+    const double cut = c.ranges ? ldexp(2.0 * N64_XCUT * d.sigma * d.sigma, -2 * c.ku - 94) : 0x1p40;
+    c.thr = 0;
+    if (cut < 0x1p30)  // a leaf's diagonal neighbours reach 2^29
+        c.thr = (int)cut + 2 > N64_RMIN ? (int)cut + 2 : N64_RMIN;
+    // a listed pair has r^2 below thr 2^94 units; in an all-close leaf |dx| is at most 2^61
+    int lg = 0;
+    while (c.thr > 0 && (1ll << lg) < c.thr)
+        ++lg;
+    c.s = c.thr > 0 && lg < 30 ? (30 - lg) >> 1 : 0;
+    const int ek = exponent_of(c.k2) + 1;  // k2 = m 2^ek, m in [1/2, 1); km = m 2^62
+    const long long km = c.ranges ? (long long)ldexp(c.k2, 62 - ek) : 0;
+    c.kmh = (int)((km + 0x80000000ll) >> 32);
+    c.kml = (int)(unsigned)(unsigned long long)km;
+    c.e = ek + 2 * c.ku + 64 - 2 * c.s + 56 + 2;
+    const int sh = c.e < 63 ? c.e : 63;
+    c.vmax = c.e >= 0 ? ((long long)N64_ROWS << 50) >> sh : 0x7fffffffffffffffll;
+    c.e = c.e > -63 ? c.e : -63;
+    c.far_sc = c.ranges ? ldexp(1.0, -51 - c.ku) : 1.0;
+    c.far_sc2 = c.ranges ? ldexp(1.0, -46 - 2 * c.ku) : 1.0;
+    c.close_sc = c.ranges ? ldexp(c.k2, 66 - c.s + c.ku) : 1.0;
+}
 
 // Per-level work lists for the tree sweeps, computed on the host and passed by value. The systems that have
 // level l (depth >= l) are sys_list[first_at[l] .. first_at[l] + nsys_at[l]) (device array, ascending).

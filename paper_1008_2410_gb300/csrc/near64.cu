@@ -28,7 +28,7 @@ constexpr double kTwoPi = 6.283185307179586476925;
 // Row i: the polynomial in t = x - c, c = (i + 1/2) / 16, that interpolates F on [i / 16, (i + 1) / 16) at Chebyshev
 // nodes, truncated to degree 6 (its error there is below (1/32)^7 / (2^6 7! 8) = 2e-17), then c itself. x < 37.5.
 constexpr int kTabN = 600;
-constexpr double kXCut = 37.5;  // e^-37.5 < 2^-54: beyond it 1 - e^-x rounds to 1
+constexpr double kXCut = N64_XCUT;
 __device__ double2 g_blob_f[kTabN * 4], g_blob_d[kTabN * 4];  // F and F'
 
 long double blob_f(long double x) { return x == 0.0L ? 1.0L : -expm1l(-x) / x; }
@@ -46,10 +46,11 @@ long double blob_d(long double x)
     return s;
 }
 
-// Coefficients (monomial in t, |t| <= h) of the degree-6 truncation of the Chebyshev interpolant of fn about c.
-void cheb6(long double (*fn)(long double), long double c, long double h, double *out)
+// Coefficients (monomial in t / h, |t| <= h) of the degree-D truncation of the Chebyshev interpolant of fn about c.
+template <int D>
+void cheb(long double (*fn)(long double), long double c, long double h, long double *out)
 {
-    constexpr int N = 16, D = 6;
+    constexpr int N = 16;
     const long double pi = 3.141592653589793238462643383279502884L;
     long double a[D + 1];
     for (int k = 0; k <= D; ++k) {
@@ -64,15 +65,18 @@ void cheb6(long double (*fn)(long double), long double c, long double h, double 
     for (int k = 2; k <= D; ++k)
         for (int m = 0; m <= k; ++m)
             T[k][m] = (m ? 2.0L * T[k - 1][m - 1] : 0.0L) - T[k - 2][m];
-    long double hm = 1.0L;
     for (int m = 0; m <= D; ++m) {
-        long double s = 0.0L;
+        out[m] = 0.0L;
         for (int k = D; k >= m; --k)
-            s += a[k] * T[k][m];
-        out[m] = (double)(s / hm);
-        hm *= h;
+            out[m] += a[k] * T[k][m];
     }
 }
+
+// The same functions for the fixed point: row i, the degree-5 polynomials of F and of -F' in u = 128 (x - c), c = (i +
+// 1/2) / 64 (interpolation error below 2^-59), as 32 bytes: c0 2^62, c1 2^64, c2 2^66 (50 bits, |c5| 2^58 above
+// them), c3 2^56, c4 2^58. Both functions are completely monotone, so the signs alternate: c2 > 0 > c5.
+constexpr int kFixN = N64_ROWS;
+__device__ int4 g_fix_f[kFixN * 2], g_fix_d[kFixN * 2];
 
 std::mutex g_tab_mu;
 bool g_tab_ready[64];
@@ -181,20 +185,8 @@ constexpr int N64_THREADS = 256;
 constexpr int N64_TILE = 640;   // sources staged at a time
 constexpr int N64_CAP = 48;     // close pairs listed per thread before they are run
 constexpr int N64_SPILL = 96;   // terms a 64-bit sum holds: 96 * 2^56.2 < 2^63
+constexpr int N64_CSPILL = 16;  // close terms a 64-bit sum holds: 16 * 2^59 at most
 constexpr int N64_FEW = 96;     // fewer sources than this run in FP64
-// smallest high word of r^2 (62 fraction bits dropped) that the fixed point takes: 1 / r^2 below 2^31 as a seed and
-// r^2 to 2^-53 relative
-constexpr int N64_RMIN = 3410000;
-
-__device__ __forceinline__ int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1023; }
-
-// Smallest k with v <= 2^k, v > 0 normal.
-__device__ __forceinline__ int ceil_log2(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return exponent_of(v) + ((b & 0xfffffffffffffull) ? 1 : 0);
-}
-
 // The smallest e with every charge of the neighbourhood below 2^e (1 - 2^-12), or kNoFixed where the fixed point is not for
 // them: it serves sums whose terms are not all far below its unit's range, that is charges with a mean magnitude (of
 // the non-zero ones, the largest left out) of at least 1/16 of the largest one's; the others, subnormal, infinite and
@@ -256,20 +248,6 @@ __device__ __forceinline__ int charge_exponent(const Rows64 &R, int ntot, const 
     return ge - 1022 + ((gm & 0xfffffu) < 0xfff00u ? 0 : 1);
 }
 
-// Fixed-point geometry: lengths in units of 2^ku, so that two leaf widths are at most 2^61; pairs whose r^2 has a
-// high word (units of 2^94) of at least thr are far. thr = 0: none is.
-struct Fixed64 {
-    int ku, thr;
-    bool ranges;  // lengths whose squares and their ratios stay well inside FP64's range
-    __device__ __forceinline__ Fixed64(const SysDev &d)
-    {
-        ku = ceil_log2(2.0 * d.wl) - 61;
-        ranges = abs(exponent_of(d.sigma)) < 200 && abs(exponent_of(d.wl)) < 200;
-        const double cut = ranges ? ldexp(2.0 * kXCut * d.sigma * d.sigma, -2 * ku - 94) : 0x1p40;
-        thr = cut < 0x1p30 ? max((int)cut + 2, N64_RMIN) : 0;  // a leaf's diagonal neighbours reach 2^31
-    }
-};
-
 // Far pair at displacement (dxh 2^31 + dxl, dyh 2^31 + dyl): r2 = r^2 2^-62.
 __device__ __forceinline__ long long r2_fixed(int dxh, int dxl, int dyh, int dyl)
 {
@@ -299,6 +277,38 @@ __device__ __forceinline__ long long recip_fixed(long long r2)
 __device__ __forceinline__ long long mul_hi(int ah, int al, int bh, int bl)
 {
     return wide(ah, bh, (long long)hi_of(wide(al, bh, wide(ah, bl, 1ll << 31))));
+}
+
+// Close pairs in fixed point: displacements D = dx 2^s (at most 2^62), r2 = r^2 2^-64 in their units.
+__device__ __forceinline__ long long scale_close(int h, int l, int s)
+{
+    return (long long)(((unsigned long long)(long long)h << 31) + (unsigned long long)(long long)l) << s;
+}
+// z = x 2^56 from r2, or -1 beyond the tables
+__device__ __forceinline__ long long z_close(const SysDev::Near64 &c, long long r2)
+{
+    const long long v = mul_hi(hi_bal(r2), (int)lo_of(r2), c.kmh, c.kml);
+    return v >= c.vmax ? -1 : (c.e >= 0 ? v << c.e : v >> -c.e);
+}
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }  // normal range only
+// D^2-like sums: (ah 2^32 + al)(bh 2^32 + bl) + (ch 2^32 + cl)(dh 2^32 + dl), / 2^64.
+__device__ __forceinline__ long long dot_hi(int ah, int al, int bh, int bl, int ch, int cl, int dh, int dl)
+{
+    return wide(ah, bh, wide(ch, dh, (long long)hi_of(wide(al, bh, wide(ah, bl, wide(cl, dh, wide(ch, dl, 1ll << 31)))))));
+}
+// F 2^62 (or -F' 2^62) from a row and z, of which 50 bits lie below the row number.
+__device__ __forceinline__ long long blob_fixed(const int4 *__restrict__ tab, long long z)
+{
+    const int i = hi_of(z) >> 18;
+    const int4 a = __ldg(tab + 2 * i), b = __ldg(tab + 2 * i + 1);
+    const long long U = (long long)(((unsigned long long)z << 14) ^ 0x8000000000000000ull) >> 1;  // u 2^62
+    const int uh = hi_bal(U), ul = (int)lo_of(U);
+    const int e4 = b.w - (__mulhi(uh, (int)((unsigned)b.y >> 18) << 2));
+    const int e3 = b.z + __mulhi(uh, e4);
+    const long long c2 = ((long long)(b.y & 0x3ffff) << 32) | (unsigned)b.x;
+    const long long e2 = c2 + (wide(uh, e3, 1 << 19) >> 20);
+    const long long e1 = (((long long)a.w << 32) | (unsigned)a.z) + mul_hi(uh, ul, hi_bal(e2), (int)lo_of(e2));
+    return (((long long)a.y << 32) | (unsigned)a.x) + mul_hi(uh, ul, hi_bal(e1), (int)lo_of(e1));
 }
 
 // Passes over a leaf of c targets: the number of passes (at most 4 more than needed) that keeps most of the 256
@@ -339,12 +349,11 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
     const SysDev &d = w.sys[k];
     const Rows64 R(w, d, leaf);
     const int ntot = R.pre[3];
-    const double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
-
-    const Fixed64 fx(d);
-    const int ku = fx.ku, thr = fx.thr;
-    const bool ranges = fx.ranges;
-    bool fixed = thr > 0 && ntot >= N64_FEW;
+    const SysDev::Near64 cl = d.n64;
+    const double k2 = cl.k2;
+    const int ku = cl.ku, thr = cl.thr;
+    const bool ranges = cl.ranges;
+    bool fixed = ranges && ntot >= N64_FEW;
     const int ge = fixed ? charge_exponent(R, ntot, w.sg, nullptr, st) : kNoFixed;
     fixed = ge != kNoFixed;
     const int ka = ge - 63;  // charges in units of 2^ka: below 2^63 - 2^50, so that their high limb fits
@@ -357,7 +366,8 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
         const bool active = grp < G;
         const double xt = w.sx[tpos], yt = w.sy[tpos];
         double au = 0.0, av = 0.0;    // FP64 pairs: sums of gamma F(x) (-dy, dx), in units of k2
-        double iu = 0.0, iv = 0.0;    // fixed-point pairs, in units of 2^-(...) (scaled at the end)
+        double iu = 0.0, iv = 0.0;    // far pairs in fixed point
+        double cu = 0.0, cv = 0.0;    // close pairs in fixed point
         auto pair64 = [&](int q) {
             const int j = R.global(q);
             const double ax = xt - w.sx[j], ay = yt - w.sy[j];
@@ -393,8 +403,29 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
             av += tv;
         } else {
             const int2 tx = limbs31(to_fixed(xt, ku)), ty = limbs31(to_fixed(yt, ku));
-            int cnt = 0, terms = 0;
-            long long su = 0, sv = 0;
+            int cnt = 0, terms = 0, cterms = 0;
+            long long su = 0, sv = 0, wu = 0, wv = 0;
+            auto close = [&](int q0, int q) {
+                const int4 p = pos[q];
+                const int2 g = gam[q];
+                const long long X = scale_close(tx.x - p.x, tx.y - p.y, cl.s), Y = scale_close(ty.x - p.z, ty.y - p.w, cl.s);
+                const int xh = hi_bal(X), xl = (int)lo_of(X), yh = hi_bal(Y), yl = (int)lo_of(Y);
+                const long long z = z_close(cl, dot_hi(xh, xl, xh, xl, yh, yl, yh, yl));
+                if (z < 0) {  // leaves so wide that r^2 of a far pair is below the fixed point
+                    pair64(q0 + q);
+                    return;
+                }
+                const long long F = blob_fixed(g_fix_f, z);
+                const long long f = mul_hi(g.x, g.y, hi_bal(F), (int)lo_of(F));
+                const int fh = hi_bal(f), fl = (int)lo_of(f);
+                wu += mul_hi(fh, fl, yh, yl);
+                wv += mul_hi(fh, fl, xh, xl);
+            };
+            auto spill_close = [&]() {
+                cu += (double)wu;
+                cv += (double)wv;
+                wu = wv = 0;
+            };
             for (int q0 = 0; q0 < ntot; q0 += N64_TILE) {
                 const int m = min(N64_TILE, ntot - q0);
                 __syncthreads();
@@ -408,6 +439,15 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                 __syncthreads();
                 const int nj = active ? (m - grp + G - 1) / G : 0;  // this thread's sources: grp, grp + G, ...
                 const int nmax = __reduce_max_sync(0xffffffffu, nj);
+                if (thr == 0) {  // every pair is close
+                    for (int i = 0; i < nj; ++i) {
+                        close(q0, grp + G * i);
+                        if (i % N64_CSPILL == N64_CSPILL - 1)
+                            spill_close();
+                    }
+                    spill_close();
+                    continue;
+                }
                 for (int i0 = 0; i0 < nmax;) {
                     // as many sources as the fullest list of the warp still takes
                     const int used = __reduce_max_sync(0xffffffffu, cnt);
@@ -441,17 +481,23 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                     if (full > N64_CAP - 12 || (i0 >= nmax && full > 0)) {
                         for (int e = 0; e < full; ++e)
                             if (e < cnt)
-                                pair64(q0 + lst[e * N64_THREADS + tid]);
+                                close(q0, lst[e * N64_THREADS + tid]);
                         cnt = 0;
+                        cterms += full;  // here F D is at most 0.64 sqrt(2) / 12.2 2^124: 96 terms fit, as for far pairs
+                        if (cterms > N64_SPILL - N64_CAP) {
+                            spill_close();
+                            cterms = 0;
+                        }
                     }
                 }
             }
             iu += (double)su;
             iv += (double)sv;
-            // a fixed-point term is gamma dx / r^2 * 2^(51 + ku - ka)
-            const double sc = scalbn(1.0, -51 - ku) ;
-            iu = scalbn(iu * sc, ka);
-            iv = scalbn(iv * sc, ka);
+            // a far term is gamma dx / r^2 2^(51 + ku - ka), a close one gamma F dx 2^(s - 66 - ku - ka)
+            spill_close();
+            const double gs = pow2(ka);
+            iu = fma(cu, cl.close_sc, iu * cl.far_sc) * gs;
+            iv = fma(cv, cl.close_sc, iv * cl.far_sc) * gs;
         }
         // groups of a target, in order, through the (now idle) list
         double2 *red = reinterpret_cast<double2 *>(pos);
@@ -505,10 +551,10 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
         return;  // this system's near field is the FP32 kernel's
     const Rows64 R(w, d, leaf);
     const int ntot = R.pre[3];
-    const double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
-    const Fixed64 fx(d);
-    const int ku = fx.ku, thr = fx.thr;
-    const bool ranges = fx.ranges;
+    const SysDev::Near64 cl = d.n64;
+    const double k2 = cl.k2;
+    const int ku = cl.ku, thr = cl.thr;
+    const bool ranges = cl.ranges;
     bool fixed = thr > 0 && ntot >= N64_FEW;
     int ka = 0, kb = 0;  // units 2^ka of gamma (below 2^62), 2^kb of gu and gv (below 2^58)
     if (fixed) {
@@ -670,9 +716,10 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
             }
             spill();
             // units: a / r^2 2^(120 - 1 + ku) per ca, charges 2^-kb and 2^-ka; sums in units of 2^64
-            ig = scalbn(ig * scalbn(1.0, -55 - ku), kb);
-            ix = scalbn(scalbn(ix * scalbn(1.0, -46 - 2 * ku), ka), kb);
-            iy = scalbn(scalbn(iy * scalbn(1.0, -46 - 2 * ku), ka), kb);
+            const double sa = pow2(ka), sb = pow2(kb);
+            ig *= cl.far_sc * 0x1p-4 * sb;
+            ix = ix * cl.far_sc2 * sa * sb;
+            iy = iy * cl.far_sc2 * sa * sb;
         }
         // groups of a target, in order, through the (now idle) source limbs
         double *red = reinterpret_cast<double *>(pos);
@@ -712,14 +759,37 @@ int prepare_near64(cudaStream_t s)
     if (g_tab_ready[dev])
         return 0;
     static double tab[2][kTabN][8];
-    for (int i = 0; i < kTabN; ++i) {
-        const long double c = (i + 0.5L) / 16.0L;
-        cheb6(blob_f, c, 1.0L / 32.0L, tab[0][i]);
-        cheb6(blob_d, c, 1.0L / 32.0L, tab[1][i]);
-        tab[0][i][7] = tab[1][i][7] = (double)c;
+    static int fix[2][kFixN][8];
+    for (int k = 0; k < 2; ++k) {
+        long double a[7];
+        for (int i = 0; i < kTabN; ++i) {
+            const long double c = (i + 0.5L) / 16.0L;
+            cheb<6>(k ? blob_d : blob_f, c, 1.0L / 32.0L, a);
+            for (int m = 0; m <= 6; ++m)
+                tab[k][i][m] = (double)ldexpl(a[m], 5 * m);  // t in place of t / h
+            tab[k][i][7] = (double)c;
+        }
+        for (int i = 0; i < kFixN; ++i) {
+            cheb<5>(k ? blob_d : blob_f, (i + 0.5L) / 64.0L, 1.0L / 128.0L, a);
+            for (int m = 0; m <= 5; ++m)
+                a[m] = k ? -a[m] : a[m];
+            const long long c0 = llroundl(ldexpl(a[0], 62)), c1 = llroundl(ldexpl(a[1], 64)),
+                            c2 = llroundl(ldexpl(a[2], 66)) | (llroundl(ldexpl(-a[5], 58)) << 50);
+            int *r = fix[k][i];
+            r[0] = (int)c0;
+            r[1] = (int)(c0 >> 32);
+            r[2] = (int)c1;
+            r[3] = (int)(c1 >> 32);
+            r[4] = (int)c2;
+            r[5] = (int)(c2 >> 32);
+            r[6] = (int)llroundl(ldexpl(a[3], 56));
+            r[7] = (int)llroundl(ldexpl(a[4], 58));
+        }
     }
     if (cudaMemcpyToSymbolAsync(g_blob_f, tab[0], sizeof tab[0], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(g_blob_d, tab[1], sizeof tab[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(g_fix_f, fix[0], sizeof fix[0], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(g_fix_d, fix[1], sizeof fix[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return -1;
     g_tab_ready[dev] = true;
