@@ -535,7 +535,7 @@ static fmm_status enqueue_adaptive(fmm_handle h, cudaStream_t s, int mode, const
     (void)cudaGetLastError();
     if (timed)
         CU(record_timing(h->ev_t[0], s));
-    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 1) * sizeof(int), s));  // counts and overflow flag
+    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the plain form's next leaf
     if (!h->has_domain) {
         nl += launch_bbox(w, x, y, s);
         nl += launch_domain_finalize(w, s);
@@ -611,7 +611,7 @@ static fmm_status enqueue_forward(fmm_handle h, cudaStream_t s, int mode, const 
     (void)cudaGetLastError();  // drop a stale, non-sticky error left by an unrelated runtime call
     if (timed && all_ev)
         CU(record_timing(h->ev_t[0], s));
-    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 1) * sizeof(int), s));  // counts and overflow flag
+    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the plain form's next leaf
     bool any_bbox = false;
     for (auto &c : h->sys_cfg)
         any_bbox |= !c.explicit_domain;
@@ -625,34 +625,50 @@ static fmm_status enqueue_forward(fmm_handle h, cudaStream_t s, int mode, const 
     nl += launch_gather(w, x, y, g, nullptr, nullptr, s);
     if (timed)
         CU(record_timing(h->ev_t[1], s));
+    // The precision form's sweep goes to the high-priority side stream: its small grids fill the SMs that the near
+    // field's blocks release. The plain form's near field (integer pipe) leaves room on every SM for the sweep (FP64
+    // pipe), so there the near field has the priority and the sweep runs beside it on the caller's stream.
+    const bool swap = far && near && !w.mixed;
+    cudaStream_t sn = swap ? h->side : s, sf = swap || !far ? s : h->side;
     if (far) {
         CU(cudaEventRecord(h->ev_fork, s));
         CU(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-        nl += launch_p2m(w, h->t, 0, h->side);
-        if (h->ext_level == w.lv.maxdepth)
-            nl += launch_level_import(w, h->ext_level, h->ext_M, h->ext_cnt, h->side);
-        for (int l = w.lv.maxdepth - 1; l >= 2; --l) {
-            nl += launch_m2m(w, h->t, l, 0, h->side, 1);
-            if (l == h->ext_level)  // the coarse levels carry every particle the given level stands for
-                nl += launch_level_import(w, l, h->ext_M, h->ext_cnt, h->side);
-        }
-        if (timed && all_ev)
-            CU(record_timing(h->ev_t[2], h->side));
-        nl += launch_m2l(w, h->t, 0, h->side, 1);
-        if (timed && all_ev)
-            CU(record_timing(h->ev_t[3], h->side));
-        for (int l = 2; l < w.lv.maxdepth; ++l)
-            nl += launch_l2l(w, h->t, l, 0, h->side, 1);
-        nl += launch_l2p(w, h->side);  // precision form: the far field before the join
-        if (timed && all_ev)
-            CU(record_timing(h->ev_t[4], h->side));
+    }
+    auto near_part = [&]() {
+        nl += launch_p2p(w, h->p2p_threads, h->p2p_kt, sn);
+        nl += launch_far_tail(w, h->tail_rings, sn);
+    };
+    if (near && swap) {
+        near_part();
+        if (timed)
+            CU(record_timing(h->ev_t[5], sn));
         CU(cudaEventRecord(h->ev_join, h->side));
     }
-    if (near) {
-        nl += launch_p2p(w, h->p2p_threads, h->p2p_kt, s);
-        nl += launch_far_tail(w, h->tail_rings, s);
+    if (far) {
+        nl += launch_p2m(w, h->t, 0, sf);
+        if (h->ext_level == w.lv.maxdepth)
+            nl += launch_level_import(w, h->ext_level, h->ext_M, h->ext_cnt, sf);
+        for (int l = w.lv.maxdepth - 1; l >= 2; --l) {
+            nl += launch_m2m(w, h->t, l, 0, sf, 1);
+            if (l == h->ext_level)  // the coarse levels carry every particle the given level stands for
+                nl += launch_level_import(w, l, h->ext_M, h->ext_cnt, sf);
+        }
+        if (timed && all_ev)
+            CU(record_timing(h->ev_t[2], sf));
+        nl += launch_m2l(w, h->t, 0, sf, 1);
+        if (timed && all_ev)
+            CU(record_timing(h->ev_t[3], sf));
+        for (int l = 2; l < w.lv.maxdepth; ++l)
+            nl += launch_l2l(w, h->t, l, 0, sf, 1);
+        nl += launch_l2p(w, sf);  // precision form: the far field before the join
+        if (timed && all_ev)
+            CU(record_timing(h->ev_t[4], sf));
+        if (!swap)
+            CU(cudaEventRecord(h->ev_join, h->side));
     }
-    if (timed)
+    if (near && !swap)
+        near_part();
+    if (timed && !swap)
         CU(record_timing(h->ev_t[5], s));
     if (far)
         CU(cudaStreamWaitEvent(s, h->ev_join, 0));
@@ -1328,7 +1344,7 @@ fmm_status fmm_velocity_adjoint(fmm_handle h, int64_t n, const double *x, const 
     cudaStream_t s = h->stream;
     int64_t nl = 0;
     bool far = w.lv.maxdepth >= 2;
-    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 1) * sizeof(int), s));  // counts and overflow flag
+    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the plain form's next leaf
     if (!h->has_domain) {
         nl += launch_bbox(w, x, y, s);
         nl += launch_domain_finalize(w, s);
@@ -1404,7 +1420,7 @@ fmm_status fmm_level_multipoles(fmm_handle h, int64_t n, const double *x, const 
     cudaStream_t s = h->stream;
     int64_t nl = 0;
     (void)cudaGetLastError();
-    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 1) * sizeof(int), s));  // counts and overflow flag
+    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the plain form's next leaf
     nl += launch_keys(w, x, y, gamma, s);  // an explicit square: the host derived the constants
     nl += launch_scan(w, s);
     nl += launch_scatter_sort(w, s);

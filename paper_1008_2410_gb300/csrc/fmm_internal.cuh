@@ -22,6 +22,7 @@
 #define FMM_MAXL 12
 #define FMM_PMAX 32
 #define FMM_MAXSYS 4096
+constexpr int kSMs = 152;
 #define FMM_NOFF 49  // M2L offsets (dx, dy) in [-3, 3]^2, indexed (dy + 3) * 7 + (dx + 3)
 
 // device status bits (OR-ed into the status word)
@@ -69,11 +70,11 @@ struct SysDev {
         double k2;             // 1 / 2 sigma^2
         double far_sc, far_sc2;  // scales of the far sums: 2^(-51 - ku); adjoint 2^(-46 - 2 ku)
         double close_sc;       // scale of the close sums: k2 2^(66 - s + ku)
-        long long vmax;        // z, before its shift, of the end of the tables
         int ku;                // lengths in units of 2^ku: two leaf widths are at most 2^61 of them
-        int thr;               // pairs whose r^2 has a high word (units of 2^94) of at least thr are far; 0: none is
-        int s;                 // close displacements are taken times 2^s (at most 2^62)
+        int thr;               // pairs whose r^2 has a high word (units of 2^94) of at least thr are far; 0: all run as close ones
+        int s, lim;            // close displacements are taken times 2^s (at most 2^62): high limbs below lim
         int e, kmh, kml;       // z = x 2^56 = (r2 km 2^-64) 2^e, r2 = r^2 2^-64 in those units
+        int vmax;              // high word of z 2^-e at the end of the tables
         int ranges;            // lengths whose squares and their ratios stay well inside FP64's range
     } n64;
 };
@@ -81,7 +82,7 @@ struct SysDev {
 // Constants of the plain form's near field (near64.cu), from the leaf width and sigma: computed once per system so that
 // its threads spend no FP64 operation on them.
 #define N64_XCUT 37.5    // e^-37.5 < 2^-54: beyond it 1 - e^-x rounds to 1
-#define N64_ROWS 2400    // rows of the fixed-point tables of F on [0, N64_XCUT)
+#define N64_XMAX 120     // end of the fixed-point tables of F
 #define N64_RMIN 3410000  // smallest high word of r^2 the fixed point takes: 1 / r^2 below 2^31 as a seed, r^2 to 2^-53
 __host__ __device__ inline unsigned long long bits_of(double v)
 {
@@ -103,22 +104,29 @@ __host__ __device__ inline void derive_near64(SysDev &d)
     const int es = exponent_of(d.sigma), ew = exponent_of(d.wl);
     c.ranges = es > -200 && es < 200 && ew > -200 && ew < 200;
     const double cut = c.ranges ? ldexp(2.0 * N64_XCUT * d.sigma * d.sigma, -2 * c.ku - 94) : 0x1p40;
+    // A far pair costs about 75 instructions, a close one 110 and the list; where the tables of F reach across the
+    // neighbourhood (x < N64_XMAX up to 2 sqrt(2) leaf widths) at least four of five pairs are close, and all run as
+    // close pairs without the list.
+    const double xr = 4.0 * (d.wl / d.sigma) * (d.wl / d.sigma);
     c.thr = 0;
-    if (cut < 0x1p30)  // a leaf's diagonal neighbours reach 2^29
+    if (xr > 0.99 * N64_XMAX && cut < 0x1p30)
         c.thr = (int)cut + 2 > N64_RMIN ? (int)cut + 2 : N64_RMIN;
-    // a listed pair has r^2 below thr 2^94 units; in an all-close leaf |dx| is at most 2^61
-    int lg = 0;
-    while (c.thr > 0 && (1ll << lg) < c.thr)
-        ++lg;
-    c.s = c.thr > 0 && lg < 30 ? (30 - lg) >> 1 : 0;
-    const int ek = exponent_of(c.k2) + 1;  // k2 = m 2^ek, m in [1/2, 1); km = m 2^62
-    const long long km = c.ranges ? (long long)ldexp(c.k2, 62 - ek) : 0;
+    // close pairs are up to sqrt(2 N64_XCUT) sigma apart (below 2^(62 - s) units, s >= 1 in leaves wider than 5.4 sigma);
+    // without the list |dx| is at most 2^61 units. Leaves wider than 2^30 of that take FP64 (lim = 0).
+    const double rc = 8.67 * d.sigma;
+    const int lr = c.ranges && c.thr > 0 ? exponent_of(rc) + 1 - c.ku : 61;
+    c.s = 62 - lr > 1 ? 62 - lr : 1;
+    c.lim = c.s > 30 ? 0 : 1 << (31 - c.s);
+    c.s = c.s < 30 ? c.s : 30;
+    if (c.thr == 0)
+        c.lim = 0x7fffffff;  // two leaf widths may be 2^61 exactly
+    const int ek = exponent_of(c.k2) + 1;  // k2 = m 2^ek, m in [1/2, 1); km = m 2^62, less where e would be negative
+    c.e = ek + 2 * c.ku + 64 - 2 * c.s + 56 + 2;
+    const long long km = c.ranges ? (long long)ldexp(c.k2, 62 - ek + (c.e < 0 ? (c.e > -63 ? c.e : -63) : 0)) : 0;
     c.kmh = (int)((km + 0x80000000ll) >> 32);
     c.kml = (int)(unsigned)(unsigned long long)km;
-    c.e = ek + 2 * c.ku + 64 - 2 * c.s + 56 + 2;
-    const int sh = c.e < 63 ? c.e : 63;
-    c.vmax = c.e >= 0 ? ((long long)N64_ROWS << 50) >> sh : 0x7fffffffffffffffll;
-    c.e = c.e > -63 ? c.e : -63;
+    c.e = c.e < 0 ? 0 : (c.e < 63 ? c.e : 63);
+    c.vmax = (int)((((long long)N64_XMAX << 56) >> c.e) >> 32);
     c.far_sc = c.ranges ? ldexp(1.0, -51 - c.ku) : 1.0;
     c.far_sc2 = c.ranges ? ldexp(1.0, -46 - 2 * c.ku) : 1.0;
     c.close_sc = c.ranges ? ldexp(c.k2, 66 - c.s + c.ku) : 1.0;

@@ -1,16 +1,15 @@
 // near64.cu -- Fig. 1 stage 9 in the plain form: the near field of Eq. 6 in (at least) FP64 accuracy.
 //
 // GB300 has 2 FP64 multiply-adds per SM and clock against 128 in FP32 and 30 wide (32 x 32 -> 64) integer ones, so
-// the pairs are split by what they need:
+// the pairs run in 64-bit fixed point on the integer pipe: coordinates as exact integers (their differences carry no
+// rounding error), products from three wide multiplications each, sums in 64-bit integers.
 //   * r > sqrt(75) sigma (x = r^2 / 2 sigma^2 > 37.5): 1 - e^-x is 1 in FP64 and the pair is the point vortex
-//     gamma (-dy, dx) / r^2. It runs in 64-bit fixed point on the integer pipe: coordinates as exact integers (their
-//     differences carry no rounding error), 1 / r^2 by one Newton step of second order from the SFU's FP32
-//     reciprocal, products from three wide multiplications each, sums in 64-bit integers.
-//   * closer pairs go to a list per thread (index in shared memory) and run in FP64 once the list is full or the
-//     sources are done, every lane with a pair of its own: F(x) = (1 - e^-x) / x comes from a table of 600
-//     polynomials of degree 6 (no exponential, no division), 15 FP64 operations a pair.
-// A block whose charges span a wide range (so that a fixed unit could lose digits of a small sum), and trees whose
-// leaves are so narrow that every adjacent pair is close, run all pairs in FP64.
+//     gamma (-dy, dx) / r^2, with 1 / r^2 by one Newton step of second order from the SFU's FP32 reciprocal.
+//   * closer pairs go to a list per thread (index in shared memory) and run once the list is full or the sources are
+//     done, every lane with a pair of its own: F(x) = (1 - e^-x) / x from a table of polynomials of degree 5 (no
+//     exponential, no division). Where nearly every adjacent pair is close, all take this path, without the list.
+// A block whose charges span a wide range (so that a fixed unit could lose digits of a small sum) or that has few
+// sources runs all pairs in FP64, with a table of polynomials of degree 6.
 #include <math.h>
 
 #include <mutex>
@@ -72,10 +71,11 @@ void cheb(long double (*fn)(long double), long double c, long double h, long dou
     }
 }
 
-// The same functions for the fixed point: row i, the degree-5 polynomials of F and of -F' in u = 128 (x - c), c = (i +
-// 1/2) / 64 (interpolation error below 2^-59), as 32 bytes: c0 2^62, c1 2^64, c2 2^66 (50 bits, |c5| 2^58 above
-// them), c3 2^56, c4 2^58. Both functions are completely monotone, so the signs alternate: c2 > 0 > c5.
-constexpr int kFixN = N64_ROWS;
+// The same functions for the fixed point on [0, 128): rows of degree-5 polynomials of F and of -F' in u = (x - c) / h
+// about the row's centre c. Below x = 8 the rows are 1 / 64 wide, above it twice as wide from octave to octave (256 rows
+// each): interpolation error below 2^-59. 32 bytes: c0 2^62, c1 2^64, c2 2^66 (50 bits, |c5| 2^58 above them), c3 2^56,
+// c4 2^58. Both functions are completely monotone, so the signs alternate: c2 > 0 > c5.
+constexpr int kFixN = 1536;
 __device__ int4 g_fix_f[kFixN * 2], g_fix_d[kFixN * 2];
 
 std::mutex g_tab_mu;
@@ -187,15 +187,15 @@ constexpr int N64_CAP = 48;     // close pairs listed per thread before they are
 constexpr int N64_SPILL = 96;   // terms a 64-bit sum holds: 96 * 2^56.2 < 2^63
 constexpr int N64_CSPILL = 16;  // close terms a 64-bit sum holds: 16 * 2^59 at most
 constexpr int N64_FEW = 96;     // fewer sources than this run in FP64
-// The smallest e with every charge of the neighbourhood below 2^e (1 - 2^-12), or kNoFixed where the fixed point is not for
-// them: it serves sums whose terms are not all far below its unit's range, that is charges with a mean magnitude (of
-// the non-zero ones, the largest left out) of at least 1/16 of the largest one's; the others, subnormal, infinite and
-// NaN ones run in FP64. b, if given, is a second array of charges of the same kind. Block-uniform.
+// The smallest e with every charge of the neighbourhood below 2^e (1 - 2^-12), or kNoFixed where the fixed point is not
+// for them: where the sum of the charges' squares, the largest left out, is below a quarter of the largest one's. A
+// term's rounding is about 0.3 2^-54 of a term of the largest charge, an FP64 sum of N such terms of size V takes about
+// sqrt(N) 2^-55 V, and V may leave out the target's own charge, so that from there on the fixed point is no worse.
+// Subnormal, infinite and NaN charges run in FP64. b, if given, is a second array of charges of the same kind.
+// Block-uniform (integer sums, so the choice is the same in every run).
 constexpr int kNoFixed = -1000000;
 struct Stats64 {
-    unsigned max;
-    int cnt;
-    unsigned long long sum;
+    unsigned max, sum;
 };
 __device__ __forceinline__ int charge_exponent(const Rows64 &R, int ntot, const double *__restrict__ a,
                                                const double *__restrict__ b, Stats64 &st)
@@ -207,11 +207,8 @@ __device__ __forceinline__ int charge_exponent(const Rows64 &R, int ntot, const 
         return b ? max(h, (unsigned)__double2hiint(b[j]) & 0x7fffffffu) : h;
     };
     __syncthreads();
-    if (tid == 0) {
-        st.max = 0;
-        st.cnt = 0;
-        st.sum = 0;
-    }
+    if (tid == 0)
+        st.max = st.sum = 0;
     __syncthreads();
     unsigned gm = 0;
     for (int q = tid; q < ntot; q += blockDim.x)
@@ -224,26 +221,17 @@ __device__ __forceinline__ int charge_exponent(const Rows64 &R, int ntot, const 
     const int ge = (int)(gm >> 20);  // biased exponent of the largest charge
     if (ge <= 100 || ge == 0x7ff)
         return kNoFixed;
-    unsigned sum = 0;
-    int cnt = 0;
-    for (int q = tid; q < ntot; q += blockDim.x) {
-        const unsigned h = mag(q);
-        sum += ((h & 0xfffffu) | 0x100000u) >> min(ge - (int)(h >> 20), 31);
-        cnt += h != 0;
-        if (sum > 0x40000000u) {
-            atomicAdd(&st.sum, (unsigned long long)sum);
-            sum = 0;
-        }
+    unsigned sum = 0;  // of (charge / 2^ge)^2 2^18; enough is enough at 2^20
+    for (int q = tid; q < ntot && sum < (1u << 20); q += blockDim.x) {
+        const unsigned h = mag(q), v = (((h & 0xfffffu) | 0x100000u) >> 6) >> min(ge - (int)(h >> 20), 31);
+        sum += (v * v) >> 10;
     }
-    sum = __reduce_add_sync(0xffffffffu, sum >> 5);  // the low bits do not matter here
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if ((tid & 31) == 0) {
-        atomicAdd(&st.sum, (unsigned long long)sum << 5);
-        atomicAdd(&st.cnt, cnt);
-    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((tid & 31) == 0)
+        atomicAdd(&st.sum, sum);
     __syncthreads();
-    const unsigned long long big = (gm & 0xfffffu) | 0x100000u;
-    if (!(st.sum > big && (st.sum - big) * 16 >= big * (unsigned long long)max(st.cnt - 1, 1)))
+    const unsigned big = ((gm & 0xfffffu) | 0x100000u) >> 6, big2 = (big * big) >> 10;
+    if (st.sum < big2 + big2 / 4)
         return kNoFixed;
     return ge - 1022 + ((gm & 0xfffffu) < 0xfff00u ? 0 : 1);
 }
@@ -279,29 +267,31 @@ __device__ __forceinline__ long long mul_hi(int ah, int al, int bh, int bl)
     return wide(ah, bh, (long long)hi_of(wide(al, bh, wide(ah, bl, 1ll << 31))));
 }
 
-// Close pairs in fixed point: displacements D = dx 2^s (at most 2^62), r2 = r^2 2^-64 in their units.
-__device__ __forceinline__ long long scale_close(int h, int l, int s)
+// Close pairs in fixed point: displacements D = dx 2^s (at most 2^62, s >= 1) as signed limbs, D = x 2^32 + y.
+__device__ __forceinline__ int2 close_limbs(int h, int l, int s)
 {
-    return (long long)(((unsigned long long)(long long)h << 31) + (unsigned long long)(long long)l) << s;
+    const long long t = wide(l, 1 << s, 0);
+    return make_int2(hi_bal(t) + (h << (s - 1)), (int)lo_of(t));
 }
-// z = x 2^56 from r2, or -1 beyond the tables
+// z = x 2^56 from r2 = r^2 2^-64, or -1 beyond the tables
 __device__ __forceinline__ long long z_close(const SysDev::Near64 &c, long long r2)
 {
     const long long v = mul_hi(hi_bal(r2), (int)lo_of(r2), c.kmh, c.kml);
-    return v >= c.vmax ? -1 : (c.e >= 0 ? v << c.e : v >> -c.e);
+    return hi_of(v) >= c.vmax ? -1 : v << c.e;
 }
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }  // normal range only
-// D^2-like sums: (ah 2^32 + al)(bh 2^32 + bl) + (ch 2^32 + cl)(dh 2^32 + dl), / 2^64.
-__device__ __forceinline__ long long dot_hi(int ah, int al, int bh, int bl, int ch, int cl, int dh, int dl)
+// r^2 2^-64 of a displacement (X, Y).
+__device__ __forceinline__ long long r2_close(int2 X, int2 Y)
 {
-    return wide(ah, bh, wide(ch, dh, (long long)hi_of(wide(al, bh, wide(ah, bl, wide(cl, dh, wide(ch, dl, 1ll << 31)))))));
+    return wide(X.x, X.x, wide(Y.x, Y.x, wide(X.x, X.y, wide(Y.x, Y.y, 1 << 30)) >> 31));
 }
-// F 2^62 (or -F' 2^62) from a row and z, of which 50 bits lie below the row number.
+// F 2^62 (or -F' 2^62) at z = x 2^56 < 2^63.
 __device__ __forceinline__ long long blob_fixed(const int4 *__restrict__ tab, long long z)
 {
-    const int i = hi_of(z) >> 18;
+    const int o = max(5 - __clz(hi_of(z)), 0);  // octave: 0 below x = 8, then x in [4 2^o, 8 2^o)
+    const int i = (hi_of(z) >> (18 + o)) + 256 * o;
     const int4 a = __ldg(tab + 2 * i), b = __ldg(tab + 2 * i + 1);
-    const long long U = (long long)(((unsigned long long)z << 14) ^ 0x8000000000000000ull) >> 1;  // u 2^62
+    const long long U = (long long)(((unsigned long long)z << (14 - o)) ^ 0x8000000000000000ull) >> 1;  // u 2^62
     const int uh = hi_bal(U), ul = (int)lo_of(U);
     const int e4 = b.w - (__mulhi(uh, (int)((unsigned)b.y >> 18) << 2));
     const int e3 = b.z + __mulhi(uh, e4);
@@ -331,20 +321,63 @@ __device__ __forceinline__ int pick_passes(int c)
 // One block per leaf. Thread = (target t, source group g of G): the pass's targets run over the threads, and the
 // groups take the sources in turn; the groups' sums of a target are added at the end in a fixed order.
 // Measured at 2^20 uniform particles (leaves of 64, 16 sigma wide): 39.0 ms with every pair by expm1 and a division
-// in FP64, 4.1 ms so; bound by the FP64 pipe (77 % busy) on the tenth of the pairs that are close. The error of the
-// near field against quad precision fell from 8.6e-16 to 2.2e-16 relative L2 (exact differences, integer sums).
+// in FP64, 3.25 ms so, issue and integer pipes about 65 % busy. The error of the near field against quad precision fell
+// from 8.6e-16 to 1.9e-16 relative L2 (exact differences, integer sums).
 // Line of the fixed point: fewer than 96 sources in the neighbourhood have no time in it (4 to 24 particles a leaf
 // agree to 2.5e-16 either way).
-__global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
+// Sums of 64-bit sums, one per thread: 96 bits, carried in shared memory (a conversion to FP64 and an addition on that
+// pipe cost as much as half a pair).
+struct Acc64 {
+    unsigned long long lo[N64_THREADS];
+    int hi[N64_THREADS];
+    __device__ __forceinline__ void clear(int t) { lo[t] = 0, hi[t] = 0; }
+    __device__ __forceinline__ void add(int t, long long v)
+    {
+        const unsigned long long a = lo[t], b = a + (unsigned long long)v;
+        lo[t] = b;
+        hi[t] += (int)(v >> 63) + (b < a ? 1 : 0);
+    }
+    // the sum over threads t, t + step, ... (n of them), as FP64
+    __device__ __forceinline__ double total(int t, int step, int n) const
+    {
+        unsigned long long a = 0;
+        int h = 0;
+        for (int k = 0; k < n; ++k) {
+            const unsigned long long b = a + lo[t + k * step];
+            h += hi[t + k * step] + (b < a ? 1 : 0);
+            a = b;
+        }
+        return fma((double)(h + (int)(a >> 63)), 0x1p64, (double)(long long)a);
+    }
+};
+constexpr size_t N64_SMEM = N64_TILE * 24 + 4 * sizeof(Acc64) + N64_CAP * N64_THREADS * 2;
+
+__global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 {
-    __shared__ int4 pos[N64_TILE];   // x and y limbs
-    __shared__ int2 gam[N64_TILE];   // gamma limbs, base 2^32
-    __shared__ unsigned short lst[N64_CAP * N64_THREADS];
+    __shared__ int s_leaf;
+    extern __shared__ __align__(16) unsigned char sm[];  // N64_SMEM bytes
+    int4 *pos = reinterpret_cast<int4 *>(sm);                        // x and y limbs
+    int2 *gam = reinterpret_cast<int2 *>(pos + N64_TILE);            // gamma limbs, base 2^32
+    Acc64 *acc = reinterpret_cast<Acc64 *>(gam + N64_TILE);          // far u, far v, close u, close v
+    unsigned short *lst = reinterpret_cast<unsigned short *>(acc + 4);
     __shared__ Stats64 st;
-    const int leaf = blockIdx.x, tid = threadIdx.x;
-    const int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
-    if (c == 0)
+    const int tid = threadIdx.x;
+    for (;;) {
+    if (tid == 0)
+        s_leaf = atomicAdd(&w.cnt[w.nleaf + 1], 1);
+    __syncthreads();
+    const int leaf = s_leaf / parts, part = s_leaf - leaf * parts;
+    __syncthreads();
+    if (leaf >= w.nleaf)
         return;
+    int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
+    {  // this unit's share of the leaf's targets
+        const int a = (int)((long long)part * c / parts), b = (int)((long long)(part + 1) * c / parts);
+        s0 += a;
+        c = b - a;
+    }
+    if (c == 0)
+        continue;
     const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
     const SysDev &d = w.sys[k];
     const Rows64 R(w, d, leaf);
@@ -366,8 +399,8 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
         const bool active = grp < G;
         const double xt = w.sx[tpos], yt = w.sy[tpos];
         double au = 0.0, av = 0.0;    // FP64 pairs: sums of gamma F(x) (-dy, dx), in units of k2
-        double iu = 0.0, iv = 0.0;    // far pairs in fixed point
-        double cu = 0.0, cv = 0.0;    // close pairs in fixed point
+        for (int q = 0; q < 4; ++q)
+            acc[q].clear(tid);        // pairs in fixed point
         auto pair64 = [&](int q) {
             const int j = R.global(q);
             const double ax = xt - w.sx[j], ay = yt - w.sy[j];
@@ -385,8 +418,8 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                     const double ax = xt - w.sx[j], ay = yt - w.sy[j], r2 = ax * ax + ay * ay;
                     if (r2 > 0.0) {
                         const double f = -expm1(-r2 * k2) / r2 * w.sg[j];
-                        iu += ay * f;
-                        iv += ax * f;
+                        au -= ay * f;
+                        av += ax * f;
                     }
                 }
         } else if (!fixed) {
@@ -408,22 +441,22 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
             auto close = [&](int q0, int q) {
                 const int4 p = pos[q];
                 const int2 g = gam[q];
-                const long long X = scale_close(tx.x - p.x, tx.y - p.y, cl.s), Y = scale_close(ty.x - p.z, ty.y - p.w, cl.s);
-                const int xh = hi_bal(X), xl = (int)lo_of(X), yh = hi_bal(Y), yl = (int)lo_of(Y);
-                const long long z = z_close(cl, dot_hi(xh, xl, xh, xl, yh, yl, yh, yl));
-                if (z < 0) {  // leaves so wide that r^2 of a far pair is below the fixed point
+                const int dxh = tx.x - p.x, dyh = ty.x - p.z;
+                const int2 X = close_limbs(dxh, tx.y - p.y, cl.s), Y = close_limbs(dyh, ty.y - p.w, cl.s);
+                const long long z = z_close(cl, r2_close(X, Y));
+                if (max(abs(dxh), abs(dyh)) >= cl.lim || z < 0) {  // leaves so wide that far pairs are listed too
                     pair64(q0 + q);
                     return;
                 }
                 const long long F = blob_fixed(g_fix_f, z);
                 const long long f = mul_hi(g.x, g.y, hi_bal(F), (int)lo_of(F));
                 const int fh = hi_bal(f), fl = (int)lo_of(f);
-                wu += mul_hi(fh, fl, yh, yl);
-                wv += mul_hi(fh, fl, xh, xl);
+                wu += mul_hi(fh, fl, Y.x, Y.y);
+                wv += mul_hi(fh, fl, X.x, X.y);
             };
             auto spill_close = [&]() {
-                cu += (double)wu;
-                cv += (double)wv;
+                acc[2].add(tid, wu);
+                acc[3].add(tid, wv);
                 wu = wv = 0;
             };
             for (int q0 = 0; q0 < ntot; q0 += N64_TILE) {
@@ -452,7 +485,9 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                     // as many sources as the fullest list of the warp still takes
                     const int used = __reduce_max_sync(0xffffffffu, cnt);
                     const int i1 = min(nmax, i0 + N64_CAP - used);
-                    for (int i = i0; i < min(i1, nj); ++i) {
+                    const int ie = min(i1, nj);
+#pragma unroll 2
+                    for (int i = i0; i < ie; ++i) {
                         const int q = grp + G * i;
                         const int4 p = pos[q];
                         int2 g = gam[q];
@@ -471,8 +506,8 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                     }
                     terms += i1 - i0;
                     if (terms > N64_SPILL - N64_CAP) {
-                        iu += (double)su;
-                        iv += (double)sv;
+                        acc[0].add(tid, su);
+                        acc[1].add(tid, sv);
                         su = sv = 0;
                         terms = 0;
                     }
@@ -491,30 +526,38 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w)
                     }
                 }
             }
-            iu += (double)su;
-            iv += (double)sv;
-            // a far term is gamma dx / r^2 2^(51 + ku - ka), a close one gamma F dx 2^(s - 66 - ku - ka)
+            acc[0].add(tid, su);
+            acc[1].add(tid, sv);
             spill_close();
-            const double gs = pow2(ka);
-            iu = fma(cu, cl.close_sc, iu * cl.far_sc) * gs;
-            iv = fma(cv, cl.close_sc, iv * cl.far_sc) * gs;
         }
-        // groups of a target, in order, through the (now idle) list
+        // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double2 *red = reinterpret_cast<double2 *>(pos);
-        const double pu = ranges ? fma(au, k2, -iu) : -iu, pv = ranges ? fma(av, k2, iv) : iv;
-        __syncthreads();
-        if (active)
-            red[tid] = make_double2(pu, pv);
-        __syncthreads();
+        const bool some64 = __syncthreads_or(au != 0.0 || av != 0.0);
+        if (some64) {
+            red[tid] = make_double2(au, av);
+            __syncthreads();
+        }
         if (tid < cp) {
             double u = 0.0, v = 0.0;
-            for (int g = 0; g < G; ++g) {
+            for (int g = 0; some64 && g < G; ++g) {
                 const double2 a = red[tid + g * cp];
                 u += a.x;
                 v += a.y;
             }
+            if (ranges) {
+                u *= k2;
+                v *= k2;
+            }
+            if (fixed) {
+                // a far term is gamma dx / r^2 2^(51 + ku - ka), a close one gamma F dx 2^(s - 66 - ku - ka)
+                const double gs = pow2(ka);
+                u -= fma(acc[2].total(tid, cp, G), cl.close_sc, acc[0].total(tid, cp, G) * cl.far_sc) * gs;
+                v += fma(acc[3].total(tid, cp, G), cl.close_sc, acc[1].total(tid, cp, G) * cl.far_sc) * gs;
+            }
             w.near64[tpos] = make_double2(u / kTwoPi, v / kTwoPi);
         }
+        __syncthreads();
+    }
     }
 }
 
@@ -626,7 +669,10 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
             ay += ty;
         } else {
             const int2 tx = limbs31(to_fixed(xt, ku)), ty = limbs31(to_fixed(yt, ku));
-            const long long tg = to_fixed(gt, ka), tgu = to_fixed(gut, kb), tgv = to_fixed(gvt, kb);
+            // cu and cv are linear in the target's charges: scaled up together, so that a weak target keeps its digits
+            const int te = max(exponent_of(gt) - (ka + 61), max(exponent_of(gut), exponent_of(gvt)) - (kb + 57));
+            const int tau = te < -900 ? 0 : -te;
+            const long long tg = to_fixed(gt, ka - tau), tgu = to_fixed(gut, kb - tau), tgv = to_fixed(gvt, kb - tau);
             const int tgh = -hi_bal(tg), tgl = (int)lo_of(tg) >> 1;  // low limb halved: it can be negated
             const int tuh = hi_bal(tgu), tul = (int)lo_of(tgu), tvh = hi_bal(tgv), tvl = (int)lo_of(tgv);
             int cnt = 0, terms = 0;
@@ -718,8 +764,9 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
             // units: a / r^2 2^(120 - 1 + ku) per ca, charges 2^-kb and 2^-ka; sums in units of 2^64
             const double sa = pow2(ka), sb = pow2(kb);
             ig *= cl.far_sc * 0x1p-4 * sb;
-            ix = ix * cl.far_sc2 * sa * sb;
-            iy = iy * cl.far_sc2 * sa * sb;
+            const double st2 = sa * pow2(-tau);
+            ix = ix * cl.far_sc2 * st2 * sb;
+            iy = iy * cl.far_sc2 * st2 * sb;
         }
         // groups of a target, in order, through the (now idle) source limbs
         double *red = reinterpret_cast<double *>(pos);
@@ -770,7 +817,8 @@ int prepare_near64(cudaStream_t s)
             tab[k][i][7] = (double)c;
         }
         for (int i = 0; i < kFixN; ++i) {
-            cheb<5>(k ? blob_d : blob_f, (i + 0.5L) / 64.0L, 1.0L / 128.0L, a);
+            const int o = i < 512 ? 0 : (i >> 8) - 1;  // octave [4 2^o, 8 2^o) for i >= 256
+            cheb<5>(k ? blob_d : blob_f, ldexpl((i - 256 * o + 0.5L) / 64.0L, o), ldexpl(1.0L / 128.0L, o), a);
             for (int m = 0; m <= 5; ++m)
                 a[m] = k ? -a[m] : a[m];
             const long long c0 = llroundl(ldexpl(a[0], 62)), c1 = llroundl(ldexpl(a[1], 64)),
@@ -792,13 +840,23 @@ int prepare_near64(cudaStream_t s)
         cudaMemcpyToSymbolAsync(g_fix_d, fix[1], sizeof fix[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return -1;
+    if (cudaFuncSetAttribute(k_near64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)N64_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(k_near64, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+        return -1;
     g_tab_ready[dev] = true;
     return 0;
 }
 
+// Persistent blocks, three to an SM, that take leaves from a counter: the register file (3 x 16 K of 64 K registers)
+// and the shared memory left over hold blocks of the multipole sweep, which runs beside this kernel on the FP64 pipe
+// (pending blocks of a plain grid would keep them out, and so would a smaller shared-memory carveout). Measured at 2^20:
+// near field 3.05 ms with four blocks an SM and 3.25 with three; whole evaluation 4.38 and 3.50 ms (sweep alone 1.5).
+// Where there are fewer leaves than resident blocks, each leaf's targets are shared out over up to eight units.
 int launch_near64(const Work &w, cudaStream_t s)
 {
-    k_near64<<<w.nleaf, N64_THREADS, 0, s>>>(w);
+    const int resident = 3 * kSMs;
+    const int parts = max(1, min(8, resident / w.nleaf));
+    k_near64<<<min(w.nleaf * parts, resident), N64_THREADS, N64_SMEM, s>>>(w, parts);
     return 1;
 }
 

@@ -261,7 +261,7 @@ extern "C" fmm_status fmm_velocity_noalloc(int tree_depth, int p, double sigma, 
     NA_CU(cudaMemcpyAsync(w.sys, &sd, sizeof sd, cudaMemcpyHostToDevice, s));
     NA_CU(cudaMemcpyAsync(w.sys_list, list, sizeof list, cudaMemcpyHostToDevice, s));
     NA_CU(cudaMemsetAsync(w.status, 0, 64, s));
-    NA_CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 1) * sizeof(int), s));
+    NA_CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));
     // the same stages as fmm_velocity, in order on the caller's stream (no second stream, no events)
     if (!domain)
         launch_bbox(w, x, y, s);

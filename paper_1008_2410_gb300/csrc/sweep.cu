@@ -250,121 +250,103 @@ int launch_m2m(const Work &w, const Tables &t, int l, int adj, cudaStream_t s, i
     return 1;
 }
 
-// ------------------------------------------------------------------ stage 6: M2L (warp per target box, all levels)
+// ------------------------------------------------------------------ stage 6: M2L (all levels)
 
-// One warp per target box, lane l = local coefficient. The interaction list (children of the parent's
-// neighbours that are not adjacent, at most 27, empty boxes skipped) is built once; sources are then taken two
-// at a time: lane m scales a~_m by (-1)^(m+1) rho^m into shared memory, and lane l contracts with its column of
-// binomials C(m + l, m), held in registers, before the rho^(l+1) scaling.
-template <int PM, typename R, typename S>
-__device__ void m2l_box(const Work &w, const typename store_of<R>::T *__restrict__ rho, const R *__restrict__ binom,
-                        const S *__restrict__ M, S *Loc, const SysDev &d, int l, int b, cx<R> *alpha, int2 *list)
-{
-    const int lane = threadIdx.x & 31, p = w.p;
-    const int ns = 1 << l, bx = b & (ns - 1), by = b >> l;
-    const int px = bx >> 1, py = by >> 1;
-    const int RS = 2 * FMM_PMAX + 2;
-    // interaction list: lanes 0..35 cover the 6 x 6 children block of the parent's 3 x 3 neighbourhood
-    int cnt = 0;
-    for (int base = 0; base < 36; base += 32) {
-        int q = base + lane;
-        bool ok = false;
-        int2 ent = make_int2(0, 0);
-        if (q < 36) {
-            int jx = 2 * (px - 1) + q % 6, jy = 2 * (py - 1) + q / 6;
-            int ddx = jx - bx, ddy = jy - by;
-            if (jx >= 0 && jy >= 0 && jx < ns && jy < ns && !(ddx >= -1 && ddx <= 1 && ddy >= -1 && ddy <= 1)) {
-                int64_t sb = d.box0[l] + (int64_t)jy * ns + jx;
-                if (w.bcount[sb] != 0) {
-                    ok = true;
-                    ent = make_int2((int)(sb - d.box0[l]), (ddy + 3) * 7 + (ddx + 3));
-                }
-            }
-        }
-        unsigned m = __ballot_sync(0xffffffffu, ok);
-        if (ok)
-            list[cnt + __popc(m & ((1u << lane) - 1))] = ent;
-        cnt += __popc(m);
-    }
-    __syncwarp();
-    R cb[PM];
-#pragma unroll
-    for (int m = 0; m < PM; ++m)
-        cb[m] = (m < p && lane < p) ? binom[m * FMM_PMAX + lane] : (R)0;
-    cx<R> acc = {(R)0, (R)0};
-    for (int s = 0; s < cnt; s += 2) {
-        const bool two = s + 1 < cnt;
-        const int2 e0 = list[s], e1 = two ? list[s + 1] : list[s];
-        const typename store_of<R>::T *rp0 = rho + e0.y * RS, *rp1 = rho + e1.y * RS;
-        if (lane < p) {
-            const R sg = (lane & 1) ? (R)1 : (R)-1;  // (-1)^(m+1)
-            cx<R> a0 = ldc<R>(M, (d.box0[l] + e0.x) * (int64_t)p + lane);
-            auto r0 = rp0[lane];
-            cx<R> t0 = cmul(cx<R>{(R)r0.x, (R)r0.y}, a0);
-            alpha[lane] = {sg * t0.re, sg * t0.im};
-            cx<R> t1 = {(R)0, (R)0};
-            if (two) {
-                cx<R> a1 = ldc<R>(M, (d.box0[l] + e1.x) * (int64_t)p + lane);
-                auto r1 = rp1[lane];
-                t1 = cmul(cx<R>{(R)r1.x, (R)r1.y}, a1);
-            }
-            alpha[32 + lane] = {sg * t1.re, sg * t1.im};
-        } else {
-            alpha[lane] = {(R)0, (R)0};  // entries m >= p meet zero binomials: keep them finite
-            alpha[32 + lane] = {(R)0, (R)0};
-        }
-        __syncwarp();
-        cx<R> b0 = {(R)0, (R)0}, b1 = {(R)0, (R)0};
-#pragma unroll
-        for (int m = 0; m < PM; ++m) {
-            const cx<R> am = alpha[m], an = alpha[32 + m];
-            b0.re = fma(cb[m], am.re, b0.re);
-            b0.im = fma(cb[m], am.im, b0.im);
-            b1.re = fma(cb[m], an.re, b1.re);
-            b1.im = fma(cb[m], an.im, b1.im);
-        }
-        if (lane < p) {
-            auto q0 = rp0[lane + 1];
-            acc = cadd(acc, cmul(cx<R>{(R)q0.x, (R)q0.y}, b0));
-            if (two) {
-                auto q1 = rp1[lane + 1];
-                acc = cadd(acc, cmul(cx<R>{(R)q1.x, (R)q1.y}, b1));
-            }
-        }
-        __syncwarp();
-    }
-    if (lane < p)
-        stc(Loc, (d.box0[l] + b) * (int64_t)p + lane, acc);
-}
+// FP64 levels: NB target boxes a block, thread = (box, coefficient). The 40 offsets of the interaction list are ten
+// orbits of quarter turns: with delta_k = i^k delta_0, rho_k = i^-k rho_0, the sources of one orbit contribute
+//   b^_l += rho_0^(l+1) sum_m C(m+l, m) y^r_m,  y^r_m = sum_k i^(-k r) (-1)^(m+1) rho_0^m a~k_m,  r = (l + m + 1) mod 4,
+// so the up to four sources (2.7 on average) share one binomial contraction, and the four y^r are a four-point
+// transform, additions only. GB300 has 2 FP64 multiply-adds per SM and clock, which bound this kernel: 670 operations
+// a coefficient, against 27 x 44 by single sources; and p threads a box, not a warp (47 % idle lanes at p = 17).
+// Measured at 2^20 particles (21840 boxes, p = 17): 1.61 ms with a warp a box and single sources, 0.51 ms so.
+__constant__ signed char c_m2l_orbit[10][2] = {{2, 0}, {3, 0}, {2, 1}, {3, 1}, {1, 2}, {2, 2}, {3, 2}, {1, 3}, {2, 3}, {3, 3}};
 
+constexpr int M2L64_T = 128;  // threads: 10 K registers a block, which fit beside the near field's blocks
 template <int PM>
-__global__ void __launch_bounds__(128) k_m2l(Work w, Tables t, int adj, int64_t gw0, int64_t gw1)
+__global__ void __launch_bounds__(M2L64_T) k_m2l64(Work w, const double2 *__restrict__ rho, const double *__restrict__ binom,
+                                               const double2 *__restrict__ M, double2 *__restrict__ Loc, int nb, int64_t gw0,
+                                               int64_t gw1)
 {
-    __shared__ __align__(16) double2 alpha_sh[4][64];
-    __shared__ int2 list_sh[4][40];
-    int64_t gw = gw0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (gw >= gw1)
-        return;
+    extern __shared__ __align__(16) double2 sh_y[];  // [2][4][nb][PM]
+    const int p = w.p, b = threadIdx.x / p, c = threadIdx.x - b * p;
+    const int64_t gw = gw0 + (int64_t)blockIdx.x * nb + b;
+    const int row = nb * PM, buf = 4 * row + 4;
+    for (int i = threadIdx.x; i < 2 * buf; i += blockDim.x)
+        sh_y[i] = make_double2(0.0, 0.0);  // entries m >= p meet zero binomials: keep them finite
+    bool on = b < nb && gw < gw1;
     int l = 2;
     while (l < w.lv.maxdepth && gw >= w.lv.m2l_item0[l + 1])
         ++l;
-    if (l > w.lv.maxdepth || gw >= w.lv.m2l_item0[l + 1])
-        return;
-    int64_t g = gw - w.lv.m2l_item0[l];
-    int b = (int)(g & (((int64_t)1 << (2 * l)) - 1));
-    int sidx = (int)(g >> (2 * l));
-    const SysDev &d = w.sys[sys_at_level(w, l, sidx)];
-    if (w.bcount[d.box0[l] + b] == 0)
-        return;
-    int wi = threadIdx.x >> 5;
-    if (level_fp64(w, l)) {
-        double2 *M = adj ? w.AM64 : w.M64, *Lc = adj ? w.AL64 : w.L64;
-        m2l_box<PM, double, double2>(w, t.rho64, t.binom64, M, Lc, d, l, b,
-                                     reinterpret_cast<cx<double> *>(alpha_sh[wi]), list_sh[wi]);
-    } else {
-        m2l_box<PM, float, float2>(w, t.rho32, t.binom32, w.M32, w.L32, d, l, b,
-                                   reinterpret_cast<cx<float> *>(alpha_sh[wi]), list_sh[wi]);
+    const int64_t g = gw - w.lv.m2l_item0[l];
+    const int box = (int)(g & (((int64_t)1 << (2 * l)) - 1));
+    const int ns = 1 << l, bx = box & (ns - 1), by = box >> l;
+    int64_t base = 0;
+    if (on) {
+        base = w.sys[sys_at_level(w, l, (int)(g >> (2 * l)))].box0[l];
+        on = w.bcount[base + box] != 0;
     }
+    const int xlo = max(2 * (bx >> 1) - 2, 0), xhi = min(2 * (bx >> 1) + 3, ns - 1);
+    const int ylo = max(2 * (by >> 1) - 2, 0), yhi = min(2 * (by >> 1) + 3, ns - 1);
+    double cb[PM];
+#pragma unroll
+    for (int m = 0; m < PM; ++m)
+        cb[m] = m < p && b < nb ? binom[m * FMM_PMAX + c] : 0.0;
+    const double sg = (c & 1) ? 1.0 : -1.0;  // (-1)^(m+1)
+    double accr = 0.0, acci = 0.0;
+    __syncthreads();
+    for (int o = 0; o < 10; ++o) {
+        const int ox = c_m2l_orbit[o][0], oy = c_m2l_orbit[o][1];
+        const double2 *rp = rho + ((oy + 3) * 7 + (ox + 3)) * (2 * FMM_PMAX + 2);
+        double2 *y = sh_y + (o & 1) * buf;
+        bool any = false;
+        if (on) {
+            // source k at (bx, by) + i^k (ox, oy)
+            double2 a[4];
+            int dx = ox, dy = oy;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int sx = bx + dx, sy = by + dy;
+                a[k] = make_double2(0.0, 0.0);
+                if (sx >= xlo && sx <= xhi && sy >= ylo && sy <= yhi) {
+                    const int64_t sb = base + (int64_t)sy * ns + sx;
+                    if (w.bcount[sb] != 0) {
+                        a[k] = M[sb * p + c];
+                        any = true;
+                    }
+                }
+                const int t = dx;
+                dx = -dy;
+                dy = t;
+            }
+            double2 r = rp[c];
+            r.x *= sg;
+            r.y *= sg;
+            const double2 t0 = make_double2(a[0].x + a[2].x, a[0].y + a[2].y), t1 = make_double2(a[0].x - a[2].x, a[0].y - a[2].y);
+            const double2 t2 = make_double2(a[1].x + a[3].x, a[1].y + a[3].y), t3 = make_double2(a[1].x - a[3].x, a[1].y - a[3].y);
+            auto put = [&](int q, double vr, double vi) {
+                y[q * (row + 1) + b * PM + c] = make_double2(r.x * vr - r.y * vi, r.x * vi + r.y * vr);
+            };
+            put(0, t0.x + t2.x, t0.y + t2.y);
+            put(1, t1.x + t3.y, t1.y - t3.x);  // a0 - i a1 - a2 + i a3
+            put(2, t0.x - t2.x, t0.y - t2.y);
+            put(3, t1.x - t3.y, t1.y + t3.x);
+        }
+        __syncthreads();
+        if (any) {
+            double br = 0.0, bi = 0.0;
+#pragma unroll
+            for (int m = 0; m < PM; ++m) {
+                const double2 v = y[((c + m + 1) & 3) * (row + 1) + b * PM + m];
+                br = fma(cb[m], v.x, br);
+                bi = fma(cb[m], v.y, bi);
+            }
+            const double2 q = rp[c + 1];
+            accr += q.x * br - q.y * bi;
+            acci += q.x * bi + q.y * br;
+        }
+    }
+    if (on)
+        Loc[(base + box) * p + c] = make_double2(accr, acci);
 }
 
 // Precision form, FP32 levels: one warp per target box with lane q = source q of its interaction list (at most
@@ -375,12 +357,6 @@ __global__ void __launch_bounds__(128) k_m2l(Work w, Tables t, int adj, int64_t 
 __constant__ int2 c_m2l_off[4][27];
 
 static int g_const_ready[64];
-
-static bool m2l_constants_ready()
-{
-    int dev = 0;
-    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && g_const_ready[dev];
-}
 
 // Uploads the offset table of k_m2l_src to the current device once (synchronises the stream: call it before
 // any stream capture).
@@ -525,12 +501,14 @@ static void m2l_src_launch(const Work &w, int64_t a, int64_t b, cudaStream_t s)
 }
 
 template <int PM>
-static void m2l_box_launch(const Work &w, const Tables &t, int adj, int64_t a, int64_t b, cudaStream_t s)
+static void m2l64_launch(const Work &w, const Tables &t, int adj, int64_t a, int64_t b, cudaStream_t s)
 {
-    if (b <= a)
-        return;
-    unsigned blocks = (unsigned)(((b - a) * 32 + 127) / 128);
-    k_m2l<PM><<<blocks, 128, 0, s>>>(w, t, adj, a, b);
+    // boxes a block: as many as 128 threads hold, fewer where the grid would leave SMs idle
+    const int64_t spread = (b - a) / (2 * kSMs);
+    const int nb = (int)(spread < 1 ? 1 : (spread > M2L64_T / PM ? M2L64_T / PM : spread));
+    const size_t sm = 2 * (size_t)(4 * nb * PM + 4) * sizeof(double2);
+    k_m2l64<PM><<<(unsigned)((b - a + nb - 1) / nb), (nb * w.p + 31) & ~31, sm, s>>>(
+        w, t.rho64, t.binom64, adj ? w.AM64 : w.M64, adj ? w.AL64 : w.L64, nb, a, b);
 }
 
 int launch_m2l(const Work &w, const Tables &t, int adj, cudaStream_t s, int prio)
@@ -539,25 +517,25 @@ int launch_m2l(const Work &w, const Tables &t, int adj, cudaStream_t s, int prio
     const int64_t total = w.lv.m2l_item0[w.lv.maxdepth + 1];
     if (w.lv.maxdepth < 2 || total == 0)
         return 0;
-    // FP64 levels (all levels of the plain form; levels <= coarse_level of the precision form): lane = coefficient
-    int l32 = w.mixed ? max(2, w.coarse_level + 1) : w.lv.maxdepth + 1;  // first FP32 level
-    if (!m2l_constants_ready())
-        l32 = w.lv.maxdepth + 1;  // constants not uploaded on this device: the lane-per-coefficient kernel for all
+    // FP64 levels: all levels of the plain form; levels <= coarse_level of the precision form
+    const int l32 = w.mixed ? max(2, w.coarse_level + 1) : w.lv.maxdepth + 1;  // first FP32 level
     const int64_t split = l32 > w.lv.maxdepth ? total : w.lv.m2l_item0[l32];
     int n = 0;
     if (split > 0) {
         if (w.p <= 8)
-            m2l_box_launch<8>(w, t, adj, 0, split, s);
+            m2l64_launch<8>(w, t, adj, 0, split, s);
         else if (w.p <= 12)
-            m2l_box_launch<12>(w, t, adj, 0, split, s);
-        else if (w.p <= 16)
-            m2l_box_launch<16>(w, t, adj, 0, split, s);
+            m2l64_launch<12>(w, t, adj, 0, split, s);
+        else if (w.p <= 14)
+            m2l64_launch<14>(w, t, adj, 0, split, s);
+        else if (w.p <= 17)
+            m2l64_launch<17>(w, t, adj, 0, split, s);
         else if (w.p <= 20)
-            m2l_box_launch<20>(w, t, adj, 0, split, s);
+            m2l64_launch<20>(w, t, adj, 0, split, s);
         else if (w.p <= 24)
-            m2l_box_launch<24>(w, t, adj, 0, split, s);
+            m2l64_launch<24>(w, t, adj, 0, split, s);
         else
-            m2l_box_launch<32>(w, t, adj, 0, split, s);
+            m2l64_launch<32>(w, t, adj, 0, split, s);
         ++n;
     }
     // FP32 levels: the tensor cores take l32 .. the finest level they cover, the CUDA cores the rest
