@@ -1353,23 +1353,25 @@ fmm_status fmm_velocity_adjoint(fmm_handle h, int64_t n, const double *x, const 
     nl += launch_scan(w, s);
     nl += launch_scatter_sort(w, s);
     nl += launch_gather(w, x, y, gamma, gu, gv, s);
+    // near field written to the outputs first, on the priority stream; the sweeps run beside it on the caller's stream
+    // (see enqueue_forward), and the far part is added after the join
+    cudaStream_t sn = far ? h->side : s;
     if (far) {
         CU(cudaEventRecord(h->ev_fork, s));
         CU(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-        for (int adj = 0; adj < 2; ++adj) {
-            nl += launch_p2m(w, h->t, adj, h->side);
-            for (int l = w.lv.maxdepth - 1; l >= 2; --l)
-                nl += launch_m2m(w, h->t, l, adj, h->side, 1);
-            nl += launch_m2l(w, h->t, adj, h->side, 1);
-            for (int l = 2; l < w.lv.maxdepth; ++l)
-                nl += launch_l2l(w, h->t, l, adj, h->side, 1);
-        }
-        nl += launch_adjoint_far(w, h->side);
-        CU(cudaEventRecord(h->ev_join, h->side));
     }
-    // near field written to the outputs first; the far part is added after the join
-    nl += launch_adjoint_p2p(w, dgamma, dx, dy, h->adj_fp32, s);
+    nl += launch_adjoint_p2p(w, dgamma, dx, dy, h->adj_fp32, sn);
     if (far) {
+        CU(cudaEventRecord(h->ev_join, h->side));
+        for (int adj = 0; adj < 2; ++adj) {
+            nl += launch_p2m(w, h->t, adj, s);
+            for (int l = w.lv.maxdepth - 1; l >= 2; --l)
+                nl += launch_m2m(w, h->t, l, adj, s, 1);
+            nl += launch_m2l(w, h->t, adj, s, 1);
+            for (int l = 2; l < w.lv.maxdepth; ++l)
+                nl += launch_l2l(w, h->t, l, adj, s, 1);
+        }
+        nl += launch_adjoint_far(w, s);
         CU(cudaStreamWaitEvent(s, h->ev_join, 0));
         nl += launch_adjoint_combine(w, dgamma, dx, dy, s);
     }

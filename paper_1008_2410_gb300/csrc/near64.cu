@@ -285,6 +285,22 @@ __device__ __forceinline__ long long r2_close(int2 X, int2 Y)
 {
     return wide(X.x, X.x, wide(Y.x, Y.x, wide(X.x, X.y, wide(Y.x, Y.y, 1 << 30)) >> 31));
 }
+__device__ __forceinline__ long long square_hi(int2 X)
+{
+    return wide(X.x, X.x, wide(X.x, X.y, 1 << 30) >> 31);
+}
+// v (h 2^32 + l) / 2^55, to its last bit.
+__device__ __forceinline__ long long mul_55(long long v, int h, int l)
+{
+    const int vh = hi_bal(v), vl = (int)lo_of(v);
+    return (wide(vh, h, 0) << 9) + (wide(vl, h, wide(vh, l, (long long)__mulhi(vl, l) + (1 << 22))) >> 23);
+}
+// The share of z that a part of r2 gives (a square or a product of displacements), to its last bit (e < 32).
+__device__ __forceinline__ long long scale_z(const SysDev::Near64 &c, long long v)
+{
+    const int h = hi_bal(v), l = (int)lo_of(v);
+    return (wide(h, c.kmh, 0) << c.e) + (wide(l, c.kmh, wide(h, c.kml, (long long)__mulhi(l, c.kml))) >> (32 - c.e));
+}
 // F 2^62 (or -F' 2^62) at z = x 2^56 < 2^63.
 __device__ __forceinline__ long long blob_fixed(const int4 *__restrict__ tab, long long z)
 {
@@ -336,6 +352,12 @@ struct Acc64 {
         const unsigned long long a = lo[t], b = a + (unsigned long long)v;
         lo[t] = b;
         hi[t] += (int)(v >> 63) + (b < a ? 1 : 0);
+    }
+    __device__ __forceinline__ void add(int t, long long h, long long l)  // h 2^24 + l
+    {
+        const unsigned long long a = lo[t], b = a + ((unsigned long long)h << 24), d = b + (unsigned long long)l;
+        lo[t] = d;
+        hi[t] += (int)(h >> 40) + (b < a ? 1 : 0) + (int)(l >> 63) + (d < b ? 1 : 0);
     }
     // the sum over threads t, t + step, ... (n of them), as FP64
     __device__ __forceinline__ double total(int t, int step, int n) const
@@ -569,36 +591,58 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 //   dy_k     += cu dKu/db + cv dKv/db,  cv = gamma_m gv_k - gamma_k gv_m
 // (K is odd and its Jacobian even in z). The same split as the forward kernel's. A far pair has f = 1 / r^2 and, with
 // P = 2 a b / r^4 and Q = (b^2 - a^2) / r^4, contributes cu P + cv Q to dx and cu Q - cv P to dy: 54 wide integer
-// multiplications in fixed point (22 operations in FP64, three times the time); sums in two 64-bit parts, high products
-// and cross terms. A close one takes F and F' from their tables, 37 FP64 operations. Measured at 2^20 uniform particles
-// (leaves of 64, 16 sigma wide): 103 ms with exp, expm1 and divisions in FP64 for every pair, 12.0 ms so, bound by the
-// FP64 pipe (63 % busy) on the close pairs; no further from quad precision on either side of the split.
+// multiplications in fixed point (22 operations in FP64, several times the time); sums in two 64-bit parts, high
+// products and cross terms. A close one takes F and -F' from their tables, 86 wide multiplications (37 operations in
+// FP64). Measured at 2^20 uniform particles (leaves of 64, 16 sigma wide): 103 ms with exp, expm1 and divisions in FP64
+// for every pair; the whole adjoint (near field beside both sweeps) 108 ms then, 8.9 ms now. 112 or 128 registers keep
+// the sweeps' blocks out (11.6 to 12.0 ms), 80 spill (10.9). Errors against quad precision are below the former ones.
 // Writes the near part in caller order (the far part is added later).
-constexpr int A64_TILE = 512;
-__global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, double *__restrict__ odg,
-                                                                   double *__restrict__ odx, double *__restrict__ ody,
-                                                                   int skip_plain)
+constexpr int A64_REGS = 96, A64_B = 2;  // registers a thread, blocks an SM: room for the sweep's blocks beside them
+constexpr int A64_TILE = 640;
+constexpr int A64_CAP = 48;  // terms between two hand-overs to the 96-bit sums
+constexpr size_t A64_SMEM = A64_TILE * 40 + 6 * sizeof(Acc64) + A64_CAP * N64_THREADS * 2;
+__global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double *__restrict__ odg,
+                                                                                double *__restrict__ odx,
+                                                                                double *__restrict__ ody, int skip_plain)
 {
-    __shared__ int4 pos[A64_TILE];   // x and y limbs
-    __shared__ int2 gam[A64_TILE];   // gamma limbs, base 2^32
-    __shared__ int4 ggr[A64_TILE];   // gu and gv limbs
-    __shared__ unsigned short lst[N64_CAP * N64_THREADS];
+    extern __shared__ __align__(16) unsigned char sm[];  // A64_SMEM bytes
+    int4 *pos = reinterpret_cast<int4 *>(sm);                // x and y limbs
+    int4 *ggr = pos + A64_TILE;                              // gu and gv limbs
+    int2 *gam = reinterpret_cast<int2 *>(ggr + A64_TILE);    // gamma limbs, base 2^32
+    Acc64 *acc = reinterpret_cast<Acc64 *>(gam + A64_TILE);  // dgamma, dx, dy of the far pairs, of the close ones
+    unsigned short *lst = reinterpret_cast<unsigned short *>(acc + 6);
     __shared__ Stats64 st;
-    const int leaf = blockIdx.x, tid = threadIdx.x;
-    const int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
-    if (c == 0)
+    __shared__ int s_leaf;
+    const int tid = threadIdx.x;
+    if (skip_plain && w.nsys == 1 && !(w.sys[0].s_unit > P2P_SPLIT_S))
+        return;  // the only system's near field is the FP32 kernel's
+    for (;;) {
+    if (tid == 0)
+        s_leaf = atomicAdd(&w.cnt[w.nleaf + 1], 1);
+    __syncthreads();
+    const int leaf = s_leaf / parts, part = s_leaf - leaf * parts;
+    __syncthreads();
+    if (leaf >= w.nleaf)
         return;
+    int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
+    {  // this unit's share of the leaf's targets
+        const int a = (int)((long long)part * c / parts), b = (int)((long long)(part + 1) * c / parts);
+        s0 += a;
+        c = b - a;
+    }
+    if (c == 0)
+        continue;
     const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
     const SysDev &d = w.sys[k];
     if (skip_plain && !(d.s_unit > P2P_SPLIT_S))
-        return;  // this system's near field is the FP32 kernel's
+        continue;  // this system's near field is the FP32 kernel's
     const Rows64 R(w, d, leaf);
     const int ntot = R.pre[3];
     const SysDev::Near64 cl = d.n64;
     const double k2 = cl.k2;
     const int ku = cl.ku, thr = cl.thr;
     const bool ranges = cl.ranges;
-    bool fixed = thr > 0 && ntot >= N64_FEW;
+    bool fixed = ranges && ntot >= N64_FEW;
     int ka = 0, kb = 0;  // units 2^ka of gamma (below 2^62), 2^kb of gu and gv (below 2^58)
     if (fixed) {
         const int ea = charge_exponent(R, ntot, w.sg, nullptr, st);
@@ -614,8 +658,10 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
         const int grp = tid / cp, tpos = s0 + t0 + (tid - grp * cp);
         const bool active = grp < G;
         const double xt = w.sx[tpos], yt = w.sy[tpos], gt = w.sg[tpos], gut = w.sgu[tpos], gvt = w.sgv[tpos];
+        for (int q = 0; q < 6; ++q)
+            acc[q].clear(tid);
+        int tau = 0;
         double ag = 0.0, ax = 0.0, ay = 0.0;  // FP64 pairs: dgamma in units of k2, dx and dy in units of k2
-        double ig = 0.0, ix = 0.0, iy = 0.0;  // fixed-point pairs
         auto pair64 = [&](int q) {
             const int j = R.global(q);
             const double a = xt - w.sx[j], b = yt - w.sy[j];
@@ -649,9 +695,9 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
                     const double e = exp(-s * k2), om = -expm1(-s * k2);
                     const double f = om / s, fp = (k2 * e * s - om) / (s * s);
                     const double cu = w.sg[j] * gut - gt * w.sgu[j], cv = w.sg[j] * gvt - gt * w.sgv[j];
-                    ig += f * (w.sgu[j] * b - w.sgv[j] * a);
-                    ix += cv * (f + 2.0 * a * a * fp) - cu * (2.0 * a * b * fp);
-                    iy += cv * (2.0 * a * b * fp) - cu * (f + 2.0 * b * b * fp);
+                    ag += f * (w.sgu[j] * b - w.sgv[j] * a);
+                    ax += cv * (f + 2.0 * a * a * fp) - cu * (2.0 * a * b * fp);
+                    ay += cv * (2.0 * a * b * fp) - cu * (f + 2.0 * b * b * fp);
                 }
         } else if (!fixed) {
             double tg = 0.0, tx = 0.0, ty = 0.0;
@@ -671,18 +717,60 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
             const int2 tx = limbs31(to_fixed(xt, ku)), ty = limbs31(to_fixed(yt, ku));
             // cu and cv are linear in the target's charges: scaled up together, so that a weak target keeps its digits
             const int te = max(exponent_of(gt) - (ka + 61), max(exponent_of(gut), exponent_of(gvt)) - (kb + 57));
-            const int tau = te < -900 ? 0 : -te;
+            tau = te < -900 ? 0 : -te;
             const long long tg = to_fixed(gt, ka - tau), tgu = to_fixed(gut, kb - tau), tgv = to_fixed(gvt, kb - tau);
             const int tgh = -hi_bal(tg), tgl = (int)lo_of(tg) >> 1;  // low limb halved: it can be negated
             const int tuh = hi_bal(tgu), tul = (int)lo_of(tgu), tvh = hi_bal(tgv), tvl = (int)lo_of(tgv);
-            int cnt = 0, terms = 0;
+            int cnt = 0;
             long long hg = 0, lg = 0, hx = 0, lx = 0, hy = 0, ly = 0;  // high products, cross terms / 2^8
-            auto spill = [&]() {
-                ig += fma((double)lg, 0x1p-24, (double)hg);
-                ix += fma((double)lx, 0x1p-24, (double)hx);
-                iy += fma((double)ly, 0x1p-24, (double)hy);
+            auto spill = [&](Acc64 *a) {  // units of 2^40
+                a[0].add(tid, hg, lg);
+                a[1].add(tid, hx, lx);
+                a[2].add(tid, hy, ly);
                 hg = lg = hx = lx = hy = ly = 0;
-                terms = 0;
+            };
+            // listed pairs beyond x = 40 in FP64: J falls as 1 / x, and few closer ones may be there to outweigh it
+            const int vmax = (thr ? cl.vmax / 3 : cl.vmax) - 2;
+            // cu, cv / 2^64 of a source: gamma_m gu_k - gamma_k gu_m; the target's negated limbs are (tgh, -2 tgl)
+            auto cross = [&](int2 g, int gh, int gl, int th, int tl) {
+                return wide(g.x, th, wide(tgh, gh, (long long)hi_of(wide(g.y, th, wide(g.x, tl, 1ll << 31)) +
+                                                                    wide(tgh, gl, -2 * wide(tgl, gh, 0)))));
+            };
+            // dx += cu A + cv B, dy += cu C + cv D, with the low halves' products (the range of the terms takes up
+            // most of the high ones)
+            auto grad = [&](long long cu, long long cv, long long A, long long B, long long C, long long D) {
+                const int cuh = hi_bal(cu), cul = (int)lo_of(cu), cvh = hi_bal(cv), cvl = (int)lo_of(cv);
+                const int Ah = hi_bal(A), Al = (int)lo_of(A), Bh = hi_bal(B), Bl = (int)lo_of(B);
+                hx = wide(cuh, Ah, wide(cvh, Bh, hx));
+                lx += wide(cuh, Al, wide(cul, Ah, wide(cvh, Bl, wide(cvl, Bh, (long long)__mulhi(cul, Al) + __mulhi(cvl, Bl))))) >> 8;
+                const int Ch = hi_bal(C), Cl = (int)lo_of(C), Dh = hi_bal(D), Dl = (int)lo_of(D);
+                hy = wide(cuh, Ch, wide(cvh, Dh, hy));
+                ly += wide(cuh, Cl, wide(cul, Ch, wide(cvh, Dl, wide(cvl, Dh, (long long)__mulhi(cul, Cl) + __mulhi(cvl, Dl))))) >> 8;
+            };
+            // a close pair: with alpha^2 = a^2 k2 and so on, in units of k2,
+            //   J = dKv/da = F - 2 alpha^2 H, -dKu/db = F - 2 beta^2 H, dKv/db = -dKu/da = -2 alpha beta H, H = -F'
+            auto close = [&](int q0, int q) {
+                const int4 p = pos[q];
+                const int dxh = tx.x - p.x, dyh = ty.x - p.z;
+                const int2 X = close_limbs(dxh, tx.y - p.y, cl.s), Y = close_limbs(dyh, ty.y - p.w, cl.s);
+                const long long sxx = square_hi(X), syy = square_hi(Y), sxy = mul_hi(X.x, X.y, Y.x, Y.y);
+                if (max(abs(dxh), abs(dyh)) >= cl.lim || __mulhi(hi_bal(sxx + syy), cl.kmh) >= vmax) {
+                    pair64(q0 + q);  // leaves so wide that far pairs are listed too
+                    return;
+                }
+                const long long zx = scale_z(cl, sxx), zy = scale_z(cl, syy), zxy = scale_z(cl, sxy);
+                const long long F = blob_fixed(g_fix_f, zx + zy), H = blob_fixed(g_fix_d, zx + zy);
+                const int hh = hi_bal(H), hl = (int)lo_of(H);
+                const long long Pxx = mul_55(zx, hh, hl), Pyy = mul_55(zy, hh, hl), Pxy = mul_55(zxy, hh, hl);
+                const int2 g = gam[q];
+                const int4 gg = ggr[q];
+                // dgamma: (gu_m b - gv_m a) F
+                const long long t = wide(gg.x, Y.x, wide(-gg.z, X.x, (long long)hi_of(wide(gg.y, Y.x, wide(gg.x, Y.y, 1ll << 31)) -
+                                                                                      wide(gg.w, X.x, wide(gg.z, X.y, 0)))));
+                const int th = hi_bal(t), tl = (int)lo_of(t), fh = hi_bal(F), fl = (int)lo_of(F);
+                hg = wide(th, fh, hg);
+                lg += wide(th, fl, wide(tl, fh, (long long)__mulhi(tl, fl))) >> 8;
+                grad(cross(g, gg.x, gg.y, tuh, tul), cross(g, gg.z, gg.w, tvh, tvl), Pxy, F - Pxx, Pyy - F, -Pxy);
             };
             for (int q0 = 0; q0 < ntot; q0 += A64_TILE) {
                 const int m = min(A64_TILE, ntot - q0);
@@ -698,9 +786,18 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
                 __syncthreads();
                 const int nj = active ? (m - grp + G - 1) / G : 0;  // this thread's sources: grp, grp + G, ...
                 const int nmax = __reduce_max_sync(0xffffffffu, nj);
+                if (thr == 0) {  // every pair is close
+                    for (int i = 0; i < nj; ++i) {
+                        close(q0, grp + G * i);
+                        if (i % A64_CAP == A64_CAP - 1)
+                            spill(acc + 3);
+                    }
+                    spill(acc + 3);
+                    continue;
+                }
                 for (int i0 = 0; i0 < nmax;) {
                     const int used = __reduce_max_sync(0xffffffffu, cnt);
-                    const int i1 = min(nmax, i0 + N64_CAP - used);
+                    const int i1 = min(nmax, i0 + A64_CAP - used);
                     for (int i = i0; i < min(i1, nj); ++i) {
                         const int q = grp + G * i;
                         const int4 p = pos[q];
@@ -723,75 +820,62 @@ __global__ void __launch_bounds__(N64_THREADS, 2) k_adjoint_near64(Work w, doubl
                         const long long Q = mul_hi(hi_bal(cs), (int)lo_of(cs), hi_bal(cd), (int)lo_of(cd));
                         const int2 g = gam[q];
                         const int4 gg = ggr[q];
-                        // cu, cv / 2^64: gamma_m gu_k - gamma_k gu_m; the target's negated limbs are (tgh, -2 tgl)
-                        const long long cu =
-                            wide(g.x, tuh,
-                                 wide(tgh, gg.x,
-                                      (long long)hi_of(wide(g.y, tuh, wide(g.x, tul, 1ll << 31)) +
-                                                       wide(tgh, gg.y, -2 * wide(tgl, gg.x, 0)))));
-                        const long long cv =
-                            wide(g.x, tvh,
-                                 wide(tgh, gg.z,
-                                      (long long)hi_of(wide(g.y, tvh, wide(g.x, tvl, 1ll << 31)) +
-                                                       wide(tgh, gg.w, -2 * wide(tgl, gg.z, 0)))));
                         // dgamma: gu_m b - gv_m a
                         hg = wide(gg.x, cbh, wide(-gg.z, cah, hg));
                         lg += (wide(gg.y, cbh, wide(gg.x, cbl, 0)) - wide(gg.w, cah, wide(gg.z, cal, 0))) >> 8;
-                        // dx: cu P + cv Q, dy: cu Q - cv P, with the low halves' products (the range of the terms
-                        // takes up most of the high ones)
-                        const int cuh = hi_bal(cu), cul = (int)lo_of(cu), cvh = hi_bal(cv), cvl = (int)lo_of(cv);
-                        const int Ph = hi_bal(P), Pl = (int)lo_of(P), Qh = hi_bal(Q), Ql = (int)lo_of(Q);
-                        hx = wide(cuh, Ph, wide(cvh, Qh, hx));
-                        lx += wide(cuh, Pl, wide(cul, Ph, wide(cvh, Ql, wide(cvl, Qh, (long long)__mulhi(cul, Pl) + __mulhi(cvl, Ql))))) >> 8;
-                        hy = wide(cuh, Qh, wide(-cvh, Ph, hy));
-                        ly += (wide(cuh, Ql, wide(cul, Qh, (long long)__mulhi(cul, Ql) - __mulhi(cvl, Pl))) -
-                               wide(cvh, Pl, wide(cvl, Ph, 0))) >> 8;
+                        grad(cross(g, gg.x, gg.y, tuh, tul), cross(g, gg.z, gg.w, tvh, tvl), P, Q, Q, -P);
                     }
-                    terms += i1 - i0;
-                    if (terms > N64_SPILL - N64_CAP)
-                        spill();
+                    spill(acc);
                     i0 = i1;
                     const int full = __reduce_max_sync(0xffffffffu, cnt);
-                    if (full > N64_CAP - 12 || (i0 >= nmax && full > 0)) {
+                    if (full > A64_CAP - 12 || (i0 >= nmax && full > 0)) {
                         for (int e = 0; e < full; ++e)
                             if (e < cnt)
-                                pair64(q0 + lst[e * N64_THREADS + tid]);
+                                close(q0, lst[e * N64_THREADS + tid]);
+                        spill(acc + 3);
                         cnt = 0;
                     }
                 }
             }
-            spill();
-            // units: a / r^2 2^(120 - 1 + ku) per ca, charges 2^-kb and 2^-ka; sums in units of 2^64
-            const double sa = pow2(ka), sb = pow2(kb);
-            ig *= cl.far_sc * 0x1p-4 * sb;
-            const double st2 = sa * pow2(-tau);
-            ix = ix * cl.far_sc2 * st2 * sb;
-            iy = iy * cl.far_sc2 * st2 * sb;
         }
-        // groups of a target, in order, through the (now idle) source limbs
+        // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double *red = reinterpret_cast<double *>(pos);
-        __syncthreads();
-        if (active) {
-            red[tid] = ranges ? fma(ag, k2, ig) : ig;
-            red[N64_THREADS + tid] = ranges ? fma(ax, k2, ix) : ix;
-            red[2 * N64_THREADS + tid] = ranges ? fma(ay, k2, iy) : iy;
+        const bool some64 = __syncthreads_or(ag != 0.0 || ax != 0.0 || ay != 0.0);
+        if (some64) {
+            red[tid] = ag;
+            red[N64_THREADS + tid] = ax;
+            red[2 * N64_THREADS + tid] = ay;
+            __syncthreads();
         }
-        __syncthreads();
         if (tid < cp) {
-            double sg = 0.0, sx = 0.0, sy = 0.0;
-            for (int g = 0; g < G; ++g) {
-                sg += red[tid + g * cp];
-                sx += red[N64_THREADS + tid + g * cp];
-                sy += red[2 * N64_THREADS + tid + g * cp];
+            double out[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                for (int g = 0; some64 && g < G; ++g)
+                    out[q] += red[q * N64_THREADS + tid + g * cp];
+                if (ranges)
+                    out[q] *= k2;
+            }
+            if (fixed) {
+                // sums in units of 2^40: far a / r^2 2^(119 + ku) per ca, close F 2^62 in units of k2, a 2^(s - ku);
+                // charges 2^-ka and 2^-kb, the target's 2^tau up
+                const double sa = pow2(ka) * pow2(-tau), sb = pow2(kb);
+                out[0] += fma(acc[3].total(tid, cp, G), cl.close_sc * 0x1p-24, acc[0].total(tid, cp, G) * (cl.far_sc * 0x1p-28)) * sb;
+#pragma unroll
+                for (int q = 1; q < 3; ++q)
+                    out[q] += fma(acc[3 + q].total(tid, cp, G), k2 * 0x1p42,
+                                  acc[q].total(tid, cp, G) * (cl.far_sc2 * 0x1p-24)) * sa * sb;
             }
             const int i = w.perm[tpos];
             if (odg)
-                odg[i] = sg / kTwoPi;
+                odg[i] = out[0] / kTwoPi;
             if (odx)
-                odx[i] = sx / kTwoPi;
+                odx[i] = out[1] / kTwoPi;
             if (ody)
-                ody[i] = sy / kTwoPi;
+                ody[i] = out[2] / kTwoPi;
         }
+        __syncthreads();
+    }
     }
 }
 
@@ -840,7 +924,10 @@ int prepare_near64(cudaStream_t s)
         cudaMemcpyToSymbolAsync(g_fix_d, fix[1], sizeof fix[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return -1;
-    if (cudaFuncSetAttribute(k_near64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)N64_SMEM) != cudaSuccess ||
+    if (cudaFuncSetAttribute(k_adjoint_near64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A64_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(k_adjoint_near64, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(k_near64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)N64_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(k_near64, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return -1;
     g_tab_ready[dev] = true;
@@ -862,7 +949,9 @@ int launch_near64(const Work &w, cudaStream_t s)
 
 int launch_adjoint_near64(const Work &w, double *dg, double *dx, double *dy, int skip_plain, cudaStream_t s)
 {
-    k_adjoint_near64<<<w.nleaf, N64_THREADS, 0, s>>>(w, dg, dx, dy, skip_plain);
+    const int resident = A64_B * kSMs;
+    const int parts = max(1, min(8, resident / w.nleaf));
+    k_adjoint_near64<<<min(w.nleaf * parts, resident), N64_THREADS, A64_SMEM, s>>>(w, parts, dg, dx, dy, skip_plain);
     return 1;
 }
 
