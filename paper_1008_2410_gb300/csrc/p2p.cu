@@ -197,7 +197,7 @@ __device__ __forceinline__ void two_sum2(f2 &s, f2 &c, f2 x)
 // them); the others lie more than 6 sigma from every target (outside the band of their leaf that faces the
 // targets' leaf), where 1 - exp(-r^2 / 2 sigma^2) is 1 in FP32, and run without either: [t1, ja) and [jb, j1)
 // first, then the band.
-template <int KT, bool SELF, bool SPLIT>
+template <int KT, bool SELF, bool SPLIT, int UN = kP2PUnroll>
 __device__ __forceinline__ void p2p_segment(const Work &w, const float4 *__restrict__ EH,
                                             const float4 *__restrict__ EL, const float4 *__restrict__ EG, int j0,
                                             int j1, int t1, int ja, int jb, float sdx, float sdy,
@@ -301,7 +301,7 @@ __device__ __forceinline__ void p2p_segment(const Work &w, const float4 *__restr
         int lo = t1, hi = ja;
 #pragma unroll 1
         for (int ph = 0; ph < 2; ++ph) {
-#pragma unroll(kP2PUnroll)
+#pragma unroll(UN)
             for (int j = lo; j < hi; ++j)
                 source(j, std::false_type{});
             lo = jb;
@@ -311,7 +311,7 @@ __device__ __forceinline__ void p2p_segment(const Work &w, const float4 *__restr
     int lo = j0, hi = t1;
 #pragma unroll 1
     for (int ph = 0; ph < 2; ++ph) {
-#pragma unroll(kP2PUnroll)
+#pragma unroll(UN == 1 ? 1 : 2)
         for (int j = lo; j < hi; ++j)
             source(j, std::true_type{});
         lo = ja;
@@ -663,6 +663,258 @@ __global__ void __launch_bounds__(P2PBounds<LPB, KTM>::threads, P2PBounds<LPB, K
     }
 }
 
+// ------------------------------------------------------------------ precision form, one warp per leaf and source row
+
+// The target-side near field where k_p2p32 would leave the GPU idle (few leaves): one block per leaf, one warp for each
+// of the three source rows, each with a tile buffer and a barrier of its own, and the source loop unrolled (few warps
+// an SM, so registers are free and latency is what counts). The sums are those of k_p2p32 with lpb leaves a block, to
+// the last bit: the same tile boundaries (the row of the block's lpb + 2 columns cut every `tile` sources), plain FP32
+// sums within a tile, kept per row and tile in shared memory and added by TwoSum in the same order at the end. A leaf
+// with more tiles in a row than P2PW_TILES (dense) goes row by row through the first warp. Latency bound; 4096 uniform
+// particles (64 leaves): 73 us with k_p2p32 (32 blocks), 14 us so.
+#define P2PW_TILES 4
+#define P2PW_UNROLL 4
+template <int KTM>
+__global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t bars[3];
+    __shared__ int4 segtab[3][3];
+    __shared__ int segt1[3][3];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int full_pass = KTM == 4 ? 128 : 64, NPR = KTM == 4 ? 2 : 1, RI = KTM == 4 ? 1 : 0;
+    float4 *TT = reinterpret_cast<float4 *>(smem_raw);            // the pass's targets: x hi, x lo, y hi, y lo
+    f2 *part = reinterpret_cast<f2 *>(TT + full_pass);            // [3][P2PW_TILES][2 NPR][32] sums of a tile
+    const int nbuf = w.p2p_all_plain ? 2 : 3;
+    float4 *EH = reinterpret_cast<float4 *>(part + 3 * P2PW_TILES * 2 * NPR * 32) + (size_t)warp * tile * nbuf;
+    float4 *EG = EH + tile, *EL = EG + tile;
+    const int leaf = blockIdx.x;
+    const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
+    const SysDev &d = w.sys[k];
+    const int L = d.depth, ns = 1 << L, local = leaf - (int)d.leaf0;
+    const int ix = local & (ns - 1), iy = local >> L;
+    const int my_s0 = w.start[leaf], my_c = w.start[leaf + 1] - my_s0;
+    if (my_c == 0)
+        return;
+    const int ca = max((ix & ~(lpb - 1)) - 1, 0), cz = min((ix & ~(lpb - 1)) + lpb, ns - 1);  // the block's columns
+    const bool split = d.s_unit > P2P_SPLIT_S, rem_form = !split;
+    const bool bands = w.cls_off != nullptr && d.bnd_ok;
+    const int per_pass = rem_form ? full_pass : 64;
+    const int my_np = (my_c + per_pass - 1) / per_pass;
+    const float s = d.s_unit;
+    bool dense = false;
+    for (int dyr = -1; dyr <= 1; ++dyr) {
+        const int row = iy + dyr;
+        if (row >= 0 && row < ns) {
+            const int rl = (int)d.leaf0 + row * ns;
+            dense |= w.start[rl + cz + 1] - w.start[rl + ca] > P2PW_TILES * tile;
+        }
+    }
+    uint64_t &bar = bars[warp];
+    if (lane == 0) {
+        mbar_init(&bar, 1);
+        fence_proxy_async();
+    }
+    __syncwarp();
+    uint32_t phase = 0;
+    for (int pass = 0; pass < my_np; ++pass) {
+        int t_lo, t_cnt;
+        if (rem_form) {  // full passes, the rest in the last
+            t_lo = full_pass * pass;
+            t_cnt = min(full_pass, my_c - t_lo);
+        } else {  // balanced passes
+            t_lo = (int)((int64_t)pass * my_c / my_np);
+            t_cnt = (int)((int64_t)(pass + 1) * my_c / my_np) - t_lo;
+        }
+        const int tbase = my_s0 + t_lo;
+        for (int e = threadIdx.x; e < full_pass; e += 96) {
+            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (e < t_cnt) {
+                const float4 th = w.eh[tbase + e], tl = w.el[tbase + e];
+                t = make_float4(th.x, tl.x, th.z, tl.z);
+            }
+            TT[e] = t;
+        }
+        __syncthreads();
+        const bool kt4 = KTM == 4 && rem_form && t_cnt > 96;
+        const int n_main = !rem_form || kt4 ? t_cnt : (t_cnt >= 64 ? 64 : (t_cnt > 32 ? t_cnt : 0));
+        const int r = t_cnt - n_main;
+        f2 SU[2] = {0ull, 0ull}, CU[2] = {0ull, 0ull}, SV[2] = {0ull, 0ull}, CV[2] = {0ull, 0ull};
+        bool ok = true;
+        for (int dyr = dense ? (warp == 0 ? -1 : 2) : warp - 1; dyr <= (dense ? 1 : warp - 1); ++dyr) {
+            const int row = iy + dyr;
+            if (row < 0 || row >= ns)
+                continue;
+            const int rowleaf = (int)d.leaf0 + row * ns;
+            const int r0 = w.start[rowleaf + ca], r1 = w.start[rowleaf + cz + 1];
+            __syncwarp();
+            if (lane < 3) {  // the row's three source leaves (see k_p2p32)
+                const int col = ix - 1 + lane;
+                int4 t = make_int4(0, 0, 0, 0);
+                int t1 = 0;
+                if (col >= 0 && col < ns) {
+                    t.x = w.start[rowleaf + col];
+                    t.y = w.start[rowleaf + col + 1];
+                    t.z = t.x;
+                    t.w = t.y;
+                    t1 = t.x;
+                    if (bands && !(lane == 1 && dyr == 0)) {
+                        const int *o = w.cls_off + (int64_t)(rowleaf + col) * 8;
+                        const int dir = (dyr + 1) * 3 + lane;
+                        const int ka = (int)((0x066004224ull >> (4 * dir)) & 15ull);
+                        const int kb = (int)((0x187307355ull >> (4 * dir)) & 15ull);
+                        t.z = ka == 0 ? t.x : o[ka - 1];
+                        t.w = o[kb - 1];
+                        if (dir == 7)
+                            t1 = o[0];
+                    }
+                }
+                segtab[warp][lane] = t;
+                segt1[warp][lane] = t1;
+            }
+            __syncwarp();
+            for (int q0 = r0, it = 0; q0 < r1; q0 += tile, ++it) {
+                const int m = min(tile, r1 - q0);
+                __syncwarp();  // the warp is done with the previous tile
+                if (lane == 0) {
+                    fence_proxy_async();
+                    mbar_expect_tx(&bar, (uint32_t)m * (split ? 48u : 32u));
+                    bulk_g2s(EH, w.eh + q0, (uint32_t)m * 16u, &bar);
+                    bulk_g2s(EG, w.eg + q0, (uint32_t)m * 16u, &bar);
+                    if (split)
+                        bulk_g2s(EL, w.el + q0, (uint32_t)m * 16u, &bar);
+                }
+                if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar, phase, w.status))) {
+                    mbar_wait_bounded(&bar, phase, w.status);  // let a late copy land before exiting
+                    ok = false;
+                    break;
+                }
+                phase ^= 1;
+                f2 PU[2] = {0ull, 0ull}, PV[2] = {0ull, 0ull};
+#pragma unroll 1
+                for (int k3 = 0; k3 < 3; ++k3) {
+                    const int4 sg = segtab[warp][k3];
+                    const int j0 = max(q0, sg.x) - q0, j1 = min(q0 + m, sg.y) - q0;
+                    if (j0 >= j1)
+                        continue;
+                    const float sdx = (float)(k3 - 1) * s, sdy = (float)dyr * s;
+                    const bool self = k3 == 1 && dyr == 0;
+                    const int t1 = min(max(segt1[warp][k3] - q0, j0), j1);
+                    const int ja = min(max(sg.z - q0, t1), j1), jb = max(min(sg.w - q0, j1), ja);
+#define P2P_SEG(KT, SELF, SPLIT) \
+    p2p_segment<KT, SELF, SPLIT, P2PW_UNROLL>(w, EH, EL, EG, j0, j1, t1, ja, jb, sdx, sdy, TT, n_main, PU, PV)
+                    if (KTM == 4 && kt4) {
+                        if (self)
+                            P2P_SEG(KTM, true, false);
+                        else
+                            P2P_SEG(KTM, false, false);
+                    } else if (n_main > 0) {
+                        if (split) {
+                            if (self)
+                                P2P_SEG(2, true, true);
+                            else
+                                P2P_SEG(2, false, true);
+                        } else {
+                            if (self)
+                                P2P_SEG(2, true, false);
+                            else
+                                P2P_SEG(2, false, false);
+                        }
+                    }
+#undef P2P_SEG
+                    if (r > 0) {
+                        if (self)
+                            p2p_segment_rem<true>(EH, EG, j0, j1, sdx, sdy, TT, n_main, r, PU[RI], PV[RI]);
+                        else
+                            p2p_segment_rem<false>(EH, EG, j0, j1, sdx, sdy, TT, n_main, r, PU[RI], PV[RI]);
+                    }
+                }
+#pragma unroll
+                for (int pr = 0; pr < NPR; ++pr) {
+                    if (dense) {
+                        two_sum2(SU[pr], CU[pr], PU[pr]);
+                        two_sum2(SV[pr], CV[pr], PV[pr]);
+                    } else {
+                        f2 *q = part + ((size_t)(warp * P2PW_TILES + it) * 2 * NPR + 2 * pr) * 32 + lane;
+                        q[0] = PU[pr];
+                        q[32] = PV[pr];
+                    }
+                }
+            }
+            if (!ok)
+                break;
+        }
+        if (!__syncthreads_and(ok))
+            return;
+        if (warp == 0) {
+            if (!dense)
+                for (int dyr = -1; dyr <= 1; ++dyr) {
+                    const int row = iy + dyr;
+                    if (row < 0 || row >= ns)
+                        continue;
+                    const int rowleaf = (int)d.leaf0 + row * ns;
+                    const int nt = (w.start[rowleaf + cz + 1] - w.start[rowleaf + ca] + tile - 1) / tile;
+                    for (int it = 0; it < nt; ++it)
+#pragma unroll
+                        for (int pr = 0; pr < NPR; ++pr) {
+                            const f2 *q = part + ((size_t)((dyr + 1) * P2PW_TILES + it) * 2 * NPR + 2 * pr) * 32 + lane;
+                            two_sum2(SU[pr], CU[pr], q[0]);
+                            two_sum2(SV[pr], CV[pr], q[32]);
+                        }
+                }
+            const float snear = d.snear;
+#pragma unroll
+            for (int pr = 0; pr < NPR; ++pr) {  // main group: targets lane + 32 (2 pr + h); pr = 1 only with kt4
+                if ((pr == 1 && !kt4) || n_main == 0)
+                    break;
+                float su[2], cu[2], sv[2], cv[2];
+                up2(SU[pr], su[0], su[1]);
+                up2(CU[pr], cu[0], cu[1]);
+                up2(SV[pr], sv[0], sv[1]);
+                up2(CV[pr], cv[0], cv[1]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int e = lane + 32 * (2 * pr + h);
+                    if (e < n_main)
+                        w.near32[(int64_t)(tbase + e) * w.nf_stride] =
+                            make_float2(-(su[h] + cu[h]) * snear, (sv[h] + cv[h]) * snear);
+                }
+            }
+            if (r > 0) {  // remainder: the G partial sums of each target, added in FP64
+                float2 *red = reinterpret_cast<float2 *>(EH);
+                float su[2], cu[2], sv[2], cv[2];
+                up2(SU[RI], su[0], su[1]);
+                up2(CU[RI], cu[0], cu[1]);
+                up2(SV[RI], sv[0], sv[1]);
+                up2(CV[RI], cv[0], cv[1]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    red[lane + 32 * h] = make_float2(su[h] + cu[h], sv[h] + cv[h]);
+                __syncwarp();
+                const int G = 64 / r;
+                for (int t = lane; t < r; t += 32) {
+                    double au = 0.0, av = 0.0;
+                    for (int gq = 0; gq < G; ++gq) {
+                        const float2 p = red[t + gq * r];
+                        au += (double)p.x;
+                        av += (double)p.y;
+                    }
+                    w.near32[(int64_t)(tbase + n_main + t) * w.nf_stride] =
+                        make_float2(-(float)au * snear, (float)av * snear);
+                }
+            }
+        }
+        __syncthreads();  // targets, sums and the first tile buffer are free again
+    }
+}
+
+template <int KTM>
+static size_t p2pw_smem(const Work &w, int tile)
+{
+    return (KTM == 4 ? 128 : 64) * sizeof(float4) + 3 * P2PW_TILES * 2 * (KTM == 4 ? 2 : 1) * 32 * sizeof(f2) +
+           (size_t)3 * tile * (w.p2p_all_plain ? 32 : 48);
+}
+
 // ------------------------------------------------------------------ precision form, symmetric near field
 
 // Each unordered pair of particles in adjacent leaves is evaluated once and acts on both (the kernel is odd:
@@ -948,7 +1200,11 @@ int prepare_p2p()
     if (cudaFuncSetAttribute(k_p2p32<1, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
         cudaFuncSetAttribute(k_p2p32<2, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
         cudaFuncSetAttribute(k_p2p32<1, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-        cudaFuncSetAttribute(k_p2p32<2, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess)
+        cudaFuncSetAttribute(k_p2p32<2, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
+        cudaFuncSetAttribute(k_p2p32w<2>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
+        cudaFuncSetAttribute(k_p2p32w<4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
+        cudaFuncSetAttribute(k_p2p32w<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(k_p2p32w<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess)
         return -1;
     g_p2p_ready[dev] = 1;
     return 0;
@@ -980,7 +1236,19 @@ int launch_p2p(const Work &w, int threads, int kt, cudaStream_t s)
     const int tile = ktmax == 4 ? 256 : (w.p2p_all_plain ? P2P_TILE2 : 192);
     // plus the staged targets of a pass, 16 bytes each for up to 32 ktmax targets per warp (two warps)
     const size_t sm = (size_t)tile * (w.p2p_all_plain ? 32 : 48) + (size_t)2 * 32 * ktmax * 16;
-    if (threads == 256 && w.lv.nsys_at[2] == w.nsys) {
+    const bool pairs1 = w.lv.nsys_at[1] == w.nsys, quads = threads == 256 && w.lv.nsys_at[2] == w.nsys;
+    // few leaves: the same sums, a warp per leaf and source row. Evaluation in a graph, k_p2p32 / k_p2p32w: 64 leaves
+    // of 64 particles 89 / 43 us, 256 of 64 101 / 55, 1024 of 98 327 / 109, 4096 of 98 353 / 292, 4096 of 64 190 / 185,
+    // but 4096 of 39 108 / 138 (two per lane leave a third of the slots empty, and a row's tile is copied per leaf)
+    if (threads != 192 && (w.nleaf <= 1024 || (w.nleaf <= 4096 && w.n / 64 >= w.nleaf))) {
+        const int tl = quads ? (w.p2p_all_plain ? P2P_TILE4 : 288) : tile, lpb = quads ? 4 : ((threads == 64 || threads == 256) && pairs1 ? 2 : 1);
+        if (ktmax == 4)
+            k_p2p32w<4><<<w.nleaf, 96, p2pw_smem<4>(w, tl), s>>>(w, tl, lpb);
+        else
+            k_p2p32w<2><<<w.nleaf, 96, p2pw_smem<2>(w, tl), s>>>(w, tl, lpb);
+        return 1;
+    }
+    if (quads) {
         // four leaves per block (every system at least 4 leaves wide): a 3 x 6 source neighbourhood for four
         // target leaves, twice the warps per block at the same per-warp register budget
         const int tile4 = w.p2p_all_plain ? P2P_TILE4 : 288;
