@@ -47,7 +47,7 @@ struct SysDev {
     double sigma;
     int depth;
     int explicit_domain;
-    int pad[2];
+    int n64_kmh, n64_kml;           // plain form's near field (near64.cu), packed by derive_near64
     // derived once per evaluation by k_domain_finalize (so no per-particle kernel divides in FP64)
     double scale;                   // 2^L / S
     double xe, ye;                  // x0 + S, y0 + S
@@ -57,26 +57,14 @@ struct SysDev {
                                     // width, so that exp(-r^2 / 2 sigma^2) = 2^-(r')^2 with r' = s r / w_L
     float inv_s;                    // 1 / s
     float snear;                    // s / (2 pi w_L): scale of the near-field sum in these units
-    float pad_f;
+    int n64_thr;
     double iu;                      // adaptive tree's precision form: 1 / u, u = sigma sqrt(2 / log2 e)
     // boundary bands of the precision form's near field: a particle whose leaf-relative position zeta (in leaf
     // widths, |zeta| <= 1/2) has |zeta_x| * 2^52 > fbnd lies within delta = sigma (1 + 2^-8) of its leaf's left or
     // right side (likewise y); bnd_ok = 0 when the bands would overlap (leaf narrower than 2 delta)
     long long fbnd;
     int bnd_ok;
-    int pad_b;
-    // plain form's near field (near64.cu), see derive_near64
-    struct Near64 {
-        double k2;             // 1 / 2 sigma^2
-        double far_sc, far_sc2;  // scales of the far sums: 2^(-51 - ku); adjoint 2^(-46 - 2 ku)
-        double close_sc;       // scale of the close sums: k2 2^(66 - s + ku)
-        int ku;                // lengths in units of 2^ku: two leaf widths are at most 2^61 of them
-        int thr;               // pairs whose r^2 has a high word (units of 2^94) of at least thr are far; 0: all run as close ones
-        int s, lim;            // close displacements are taken times 2^s (at most 2^62): high limbs below lim
-        int e, kmh, kml;       // z = x 2^56 = (r2 km 2^-64) 2^e, r2 = r^2 2^-64 in those units
-        int vmax;              // high word of z 2^-e at the end of the tables
-        int ranges;            // lengths whose squares and their ratios stay well inside FP64's range
-    } n64;
+    int n64_pack;
 };
 
 // Constants of the plain form's near field (near64.cu), from the leaf width and sigma: computed once per system so that
@@ -84,6 +72,15 @@ struct SysDev {
 #define N64_XCUT 37.5    // e^-37.5 < 2^-54: beyond it 1 - e^-x rounds to 1
 #define N64_XMAX 120     // end of the fixed-point tables of F
 #define N64_RMIN 3410000  // smallest high word of r^2 the fixed point takes: 1 / r^2 below 2^31 as a seed, r^2 to 2^-53
+struct Near64 {
+    double k2;         // 1 / 2 sigma^2
+    int ku;            // lengths in units of 2^ku: two leaf widths are at most 2^61 of them
+    int thr;           // pairs whose r^2 has a high word (units of 2^94) of at least thr are far; 0: all run as close ones
+    int s, lim;        // close displacements are taken times 2^s (at most 2^62): high limbs below lim
+    int e, kmh, kml;   // z = x 2^56 = (r2 km 2^-64) 2^e, r2 = r^2 2^-64 in those units
+    int vmax;          // high word of z 2^-e at the end of the tables
+    bool ranges;       // lengths whose squares and their ratios stay well inside FP64's range
+};
 __host__ __device__ inline unsigned long long bits_of(double v)
 {
 #ifdef __CUDA_ARCH__
@@ -95,41 +92,64 @@ __host__ __device__ inline unsigned long long bits_of(double v)
 #endif
 }
 __host__ __device__ inline int exponent_of(double v) { return (int)((bits_of(v) >> 52) & 0x7ff) - 1023; }
+__host__ __device__ inline int near64_unit(double wl)  // ku
+{
+    const double w2 = 2.0 * wl;
+    return exponent_of(w2) + ((bits_of(w2) & 0xfffffffffffffull) ? 1 : 0) - 61;
+}
 __host__ __device__ inline void derive_near64(SysDev &d)
 {
-    SysDev::Near64 &c = d.n64;
-    c.k2 = 1.0 / (2.0 * d.sigma * d.sigma);
-    const double w2 = 2.0 * d.wl;
-    c.ku = exponent_of(w2) + ((bits_of(w2) & 0xfffffffffffffull) ? 1 : 0) - 61;
-    const int es = exponent_of(d.sigma), ew = exponent_of(d.wl);
-    c.ranges = es > -200 && es < 200 && ew > -200 && ew < 200;
-    const double cut = c.ranges ? ldexp(2.0 * N64_XCUT * d.sigma * d.sigma, -2 * c.ku - 94) : 0x1p40;
+    const double k2 = 1.0 / (2.0 * d.sigma * d.sigma);
+    const int ku = near64_unit(d.wl), es = exponent_of(d.sigma), ew = exponent_of(d.wl);
+    d.n64_thr = -1;
+    d.n64_kmh = d.n64_kml = d.n64_pack = 0;
+    if (!(es > -200 && es < 200 && ew > -200 && ew < 200))
+        return;
+    const double cut = ldexp(2.0 * N64_XCUT * d.sigma * d.sigma, -2 * ku - 94);
     // A far pair costs about 75 instructions, a close one 110 and the list; where the tables of F reach across the
     // neighbourhood (x < N64_XMAX up to 2 sqrt(2) leaf widths) at least four of five pairs are close, and all run as
     // close pairs without the list.
     const double xr = 4.0 * (d.wl / d.sigma) * (d.wl / d.sigma);
-    c.thr = 0;
+    d.n64_thr = 0;
     if (xr > 0.99 * N64_XMAX && cut < 0x1p30)
-        c.thr = (int)cut + 2 > N64_RMIN ? (int)cut + 2 : N64_RMIN;
+        d.n64_thr = (int)cut + 2 > N64_RMIN ? (int)cut + 2 : N64_RMIN;
     // close pairs are up to sqrt(2 N64_XCUT) sigma apart (below 2^(62 - s) units, s >= 1 in leaves wider than 5.4 sigma);
-    // without the list |dx| is at most 2^61 units. Leaves wider than 2^30 of that take FP64 (lim = 0).
-    const double rc = 8.67 * d.sigma;
-    const int lr = c.ranges && c.thr > 0 ? exponent_of(rc) + 1 - c.ku : 61;
-    c.s = 62 - lr > 1 ? 62 - lr : 1;
+    // without the list |dx| is at most 2^61 units. Leaves wider than 2^30 of that take FP64 (s = 31).
+    const int lr = d.n64_thr > 0 ? exponent_of(8.67 * d.sigma) + 1 - ku : 61;
+    int s = 62 - lr > 1 ? 62 - lr : 1;
+    s = s > 30 ? 31 : s;
+    const int ek = exponent_of(k2) + 1;  // k2 = m 2^ek, m in [1/2, 1); km = m 2^62
+    const long long km = (long long)ldexp(k2, 62 - ek);
+    d.n64_kmh = (int)(km >> 32);
+    d.n64_kml = (int)(unsigned)(unsigned long long)km;
+    int e = ek + 2 * ku + 64 - 2 * s + 56 + 2;
+    e = e < -63 ? -63 : (e > 31 ? 31 : e);
+    d.n64_pack = ek * 65536 + (e + 64) * 256 + s;
+}
+__device__ __forceinline__ Near64 near64_of(const SysDev &d)
+{
+    Near64 c;
+    c.ranges = d.n64_thr >= 0;
+    c.thr = d.n64_thr;
+    c.ku = near64_unit(d.wl);
+    c.s = d.n64_pack & 0xff;
     c.lim = c.s > 30 ? 0 : 1 << (31 - c.s);
     c.s = c.s < 30 ? c.s : 30;
     if (c.thr == 0)
         c.lim = 0x7fffffff;  // two leaf widths may be 2^61 exactly
-    const int ek = exponent_of(c.k2) + 1;  // k2 = m 2^ek, m in [1/2, 1); km = m 2^62, less where e would be negative
-    c.e = ek + 2 * c.ku + 64 - 2 * c.s + 56 + 2;
-    const long long km = c.ranges ? (long long)ldexp(c.k2, 62 - ek + (c.e < 0 ? (c.e > -63 ? c.e : -63) : 0)) : 0;
-    c.kmh = (int)((km + 0x80000000ll) >> 32);
-    c.kml = (int)(unsigned)(unsigned long long)km;
-    c.e = c.e < 0 ? 0 : (c.e < 63 ? c.e : 63);
+    // k2 from its mantissa (53 of km's 62 bits) and exponent; km gives way where e is negative (x is tiny there)
+    const unsigned long long km = ((unsigned long long)(unsigned)d.n64_kmh << 32) | (unsigned)d.n64_kml;
+    const int ek = d.n64_pack >> 16;
+    c.k2 = __longlong_as_double((long long)(((km >> 9) & 0xfffffffffffffull) | ((unsigned long long)(ek + 1022) << 52)));
+    if (!c.ranges)
+        c.k2 = 1.0 / (2.0 * d.sigma * d.sigma);
+    c.e = ((d.n64_pack >> 8) & 0xff) - 64;
+    const long long kr = (long long)(c.e < 0 ? km >> -c.e : km);
+    c.e = c.e > 0 ? c.e : 0;
+    c.kmh = (int)((kr + 0x80000000ll) >> 32);
+    c.kml = (int)(unsigned)(unsigned long long)kr;
     c.vmax = (int)((((long long)N64_XMAX << 56) >> c.e) >> 32);
-    c.far_sc = c.ranges ? ldexp(1.0, -51 - c.ku) : 1.0;
-    c.far_sc2 = c.ranges ? ldexp(1.0, -46 - 2 * c.ku) : 1.0;
-    c.close_sc = c.ranges ? ldexp(c.k2, 66 - c.s + c.ku) : 1.0;
+    return c;
 }
 
 // Per-level work lists for the tree sweeps, computed on the host and passed by value. The systems that have

@@ -274,7 +274,7 @@ __device__ __forceinline__ int2 close_limbs(int h, int l, int s)
     return make_int2(hi_bal(t) + (h << (s - 1)), (int)lo_of(t));
 }
 // z = x 2^56 from r2 = r^2 2^-64, or -1 beyond the tables
-__device__ __forceinline__ long long z_close(const SysDev::Near64 &c, long long r2)
+__device__ __forceinline__ long long z_close(const Near64 &c, long long r2)
 {
     const long long v = mul_hi(hi_bal(r2), (int)lo_of(r2), c.kmh, c.kml);
     return hi_of(v) >= c.vmax ? -1 : v << c.e;
@@ -296,7 +296,7 @@ __device__ __forceinline__ long long mul_55(long long v, int h, int l)
     return (wide(vh, h, 0) << 9) + (wide(vl, h, wide(vh, l, (long long)__mulhi(vl, l) + (1 << 22))) >> 23);
 }
 // The share of z that a part of r2 gives (a square or a product of displacements), to its last bit (e < 32).
-__device__ __forceinline__ long long scale_z(const SysDev::Near64 &c, long long v)
+__device__ __forceinline__ long long scale_z(const Near64 &c, long long v)
 {
     const int h = hi_bal(v), l = (int)lo_of(v);
     return (wide(h, c.kmh, 0) << c.e) + (wide(l, c.kmh, wide(h, c.kml, (long long)__mulhi(l, c.kml))) >> (32 - c.e));
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
     const SysDev &d = w.sys[k];
     const Rows64 R(w, d, leaf);
     const int ntot = R.pre[3];
-    const SysDev::Near64 cl = d.n64;
+    const Near64 cl = near64_of(d);
     const double k2 = cl.k2;
     const int ku = cl.ku, thr = cl.thr;
     const bool ranges = cl.ranges;
@@ -572,9 +572,9 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             }
             if (fixed) {
                 // a far term is gamma dx / r^2 2^(51 + ku - ka), a close one gamma F dx 2^(s - 66 - ku - ka)
-                const double gs = pow2(ka);
-                u -= fma(acc[2].total(tid, cp, G), cl.close_sc, acc[0].total(tid, cp, G) * cl.far_sc) * gs;
-                v += fma(acc[3].total(tid, cp, G), cl.close_sc, acc[1].total(tid, cp, G) * cl.far_sc) * gs;
+                const double gs = pow2(ka), fs = pow2(-51 - ku), cs = k2 * pow2(66 - cl.s + ku);
+                u -= fma(acc[2].total(tid, cp, G), cs, acc[0].total(tid, cp, G) * fs) * gs;
+                v += fma(acc[3].total(tid, cp, G), cs, acc[1].total(tid, cp, G) * fs) * gs;
             }
             w.near64[tpos] = make_double2(u / kTwoPi, v / kTwoPi);
         }
@@ -638,7 +638,7 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
         continue;  // this system's near field is the FP32 kernel's
     const Rows64 R(w, d, leaf);
     const int ntot = R.pre[3];
-    const SysDev::Near64 cl = d.n64;
+    const Near64 cl = near64_of(d);
     const double k2 = cl.k2;
     const int ku = cl.ku, thr = cl.thr;
     const bool ranges = cl.ranges;
@@ -860,11 +860,11 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
                 // sums in units of 2^40: far a / r^2 2^(119 + ku) per ca, close F 2^62 in units of k2, a 2^(s - ku);
                 // charges 2^-ka and 2^-kb, the target's 2^tau up
                 const double sa = pow2(ka) * pow2(-tau), sb = pow2(kb);
-                out[0] += fma(acc[3].total(tid, cp, G), cl.close_sc * 0x1p-24, acc[0].total(tid, cp, G) * (cl.far_sc * 0x1p-28)) * sb;
+                out[0] += fma(acc[3].total(tid, cp, G), k2 * pow2(42 - cl.s + ku), acc[0].total(tid, cp, G) * pow2(-79 - ku)) * sb;
 #pragma unroll
                 for (int q = 1; q < 3; ++q)
                     out[q] += fma(acc[3 + q].total(tid, cp, G), k2 * 0x1p42,
-                                  acc[q].total(tid, cp, G) * (cl.far_sc2 * 0x1p-24)) * sa * sb;
+                                  acc[q].total(tid, cp, G) * pow2(-70 - 2 * ku)) * sa * sb;
             }
             const int i = w.perm[tpos];
             if (odg)
