@@ -39,7 +39,7 @@ def _stale(target: str, deps: list[str]) -> bool:
 def build(force: bool = False, verbose: bool = False, extra_flags=(), out_dir: str | None = None) -> str:
     out = out_dir or OUT_DIR
     os.makedirs(out, exist_ok=True)
-    headers = [os.path.join(CSRC, "fmm_internal.cuh"), os.path.join(ROOT, "include", "fmm2d.h")]
+    headers = [os.path.join(CSRC, "fmm_internal.cuh"), os.path.join(CSRC, "near64.cuh"), os.path.join(ROOT, "include", "fmm2d.h")]
     objs = []
     jobs = []
     for src in SOURCES:

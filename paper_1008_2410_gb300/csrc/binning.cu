@@ -599,8 +599,15 @@ __device__ __forceinline__ void place_particle(const Work &w, int v, int pos, in
             const SysDev &d = w.sys[0];
             const double X = (xv - d.x0) * d.iu, Y = (yv - d.y0) * d.iu;
             const float hx = (float)X, hy = (float)Y;
-            w.eh[pos] = make_float4(hx, hy, (float)(X - (double)hx), (float)(Y - (double)hy));
-            w.eg[pos].x = (float)gv0;
+            // two particles a record, so that the near field loads packed pairs: (x hi of the even, of the odd one,
+            // y hi, y hi), the lo parts alike, the charges
+            float *h = reinterpret_cast<float *>(w.eh + (pos >> 1)) + (pos & 1);
+            float *l = reinterpret_cast<float *>(w.el + (pos >> 1)) + (pos & 1);
+            h[0] = hx;
+            h[2] = hy;
+            l[0] = (float)(X - (double)hx);
+            l[2] = (float)(Y - (double)hy);
+            reinterpret_cast<float *>(w.eg)[pos] = (float)gv0;
         }
     }
 }

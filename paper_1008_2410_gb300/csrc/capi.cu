@@ -364,7 +364,7 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     sizes[i++] = np * 4;                                      // 27 iperm
     sizes[i++] = adjoint ? np * 24 : 0;                       // 28 adj_far
     sizes[i++] = h->adaptive_cap ? (size_t)nbox * 4 + 16 : 0;   // 29 ad_list
-    sizes[i++] = h->adaptive_cap ? (FMM_MAXL + 2) * 4 : 0;      // 30 ad_cnt
+    sizes[i++] = h->adaptive_cap ? (FMM_MAXL + 3) * 4 : 0;      // 30 ad_cnt
     sizes[i++] = (size_t)(n / 129 + 2) * 4;                    // 31 big (leaves of more than 128 particles)
     sizes[i++] = mixed ? (size_t)nleaf * 32 + 16 : 0;          // 32 cls_off (boundary classes of each leaf)
     sizes[i++] = mixed ? np : 0;                              // 33 cls8 (boundary class of each particle)
@@ -377,6 +377,10 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     sizes[i++] = mixed ? m2l_tc_layout_bytes(h->lv, p) : 0;     // 35 mtc (tensor-core M2L windows)
     sizes[i++] = mixed ? m2l_tc_part_bytes(h->lv, p) : 0;       // 36 m2l_part (its partial locals)
     sizes[i++] = mixed ? m2l_tc_count_bytes(h->lv, p) : 0;      // 37 m2l_cnt (its tile counters)
+    // 38, 39 the adaptive leaves' U and W lists: room for leaves an eighth full on average
+    const int ad_cap = h->adaptive_cap ? (int)std::min<int64_t>(n, n * 8 / h->adaptive_cap + 1024) : 0;
+    sizes[i++] = h->adaptive_cap ? np * 4 : 0;                              // ad_leaf
+    sizes[i++] = (size_t)ad_cap * sizeof(AdLeaf);                           // ad_lists
     int count = i;
     Layout lay;
     size_t total = 0;
@@ -467,6 +471,10 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     w.adj_far = sizes[28] ? (double *)(b + lay.off[28]) : nullptr;
     w.ad_list = sizes[29] ? (int *)(b + lay.off[29]) : nullptr;
     w.ad_cnt = sizes[30] ? (int *)(b + lay.off[30]) : nullptr;
+    w.ad_leaf = sizes[38] ? (int *)(b + lay.off[38]) : nullptr;
+    w.ad_lists = sizes[39] ? (AdLeaf *)(b + lay.off[39]) : nullptr;
+    w.ad_cap = ad_cap;
+    w.blob_f = near64_table();
     w.big = (int *)(b + lay.off[31]);
     w.cls_off = sizes[32] ? (int *)(b + lay.off[32]) : nullptr;
     w.cls8 = sizes[33] ? (unsigned char *)(b + lay.off[33]) : nullptr;
@@ -547,8 +555,14 @@ static fmm_status enqueue_adaptive(fmm_handle h, cudaStream_t s, int mode, const
     const bool count = near && h->count_pairs;
     if (count)
         CU(cudaMemsetAsync(w.pair_count, 0, sizeof(unsigned long long), s));
-    if (sweep)
-        CU(cudaMemsetAsync(w.ad_cnt, 0, (FMM_MAXL + 2) * sizeof(int), s));
+    const bool lists = w.maxdepth >= 2;
+    if (lists) {
+        CU(cudaMemsetAsync(w.ad_cnt, 0, (FMM_MAXL + 3) * sizeof(int), s));
+        CU(cudaMemsetAsync(w.ad_leaf, 0xff, (size_t)w.n * sizeof(int), s));
+        nl += launch_adaptive_boxes(w, s);
+    } else {
+        w.ad_leaf = nullptr;  // no lists
+    }
     if (timed)
         CU(record_timing(h->ev_t[1], s));
     if (sweep) {
@@ -561,8 +575,11 @@ static fmm_status enqueue_adaptive(fmm_handle h, cudaStream_t s, int mode, const
         if (timed)
             CU(record_timing(h->ev_t[3], h->side));
         CU(cudaEventRecord(h->ev_join, h->side));
-        CU(cudaStreamWaitEvent(s, h->ev_join, 0));
     }
+    if (lists)
+        nl += launch_adaptive_lists(w, s);
+    if (sweep)
+        CU(cudaStreamWaitEvent(s, h->ev_join, 0));
     if (timed)
         CU(record_timing(h->ev_t[6], s));
     // the walk reads the W multipoles and the leaf's local expansion

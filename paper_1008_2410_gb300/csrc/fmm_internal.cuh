@@ -23,6 +23,8 @@
 #define FMM_PMAX 32
 #define FMM_MAXSYS 4096
 constexpr int kSMs = 152;
+#define AD_UCAP 24  // entries of an adaptive leaf's U and W lists (a leaf with more is walked by each particle)
+#define AD_WCAP 24
 #define FMM_NOFF 49  // M2L offsets (dx, dy) in [-3, 3]^2, indexed (dy + 3) * 7 + (dx + 3)
 
 // device status bits (OR-ed into the status word)
@@ -152,6 +154,17 @@ __device__ __forceinline__ Near64 near64_of(const SysDev &d)
     return c;
 }
 
+// U and W lists of an adaptive leaf (adaptive.cu).
+struct AdLeaf {
+    int box, nu, nw, pad;   // packed box; numbers of entries
+    double2 c;              // centre
+    int2 u[AD_UCAP];        // particle ranges
+    struct W {
+        double2 c;          // centre
+        int box, pad[3];
+    } w[AD_WCAP];
+};
+
 // Per-level work lists for the tree sweeps, computed on the host and passed by value. The systems that have
 // level l (depth >= l) are sys_list[first_at[l] .. first_at[l] + nsys_at[l]) (device array, ascending).
 struct LevelInfo {
@@ -203,7 +216,12 @@ struct Work {
     int adapt_cap;            // adaptive tree: a box holding more than this many particles is split (0: uniform)
     int ad_mixed;             // adaptive tree in the precision form (FP32 expansions and near field)
     int *ad_list;             // adaptive tree: Morton indices of the existing boxes of level l at [box0[l], ...)
-    int *ad_cnt;              // [FMM_MAXL + 2] adaptive tree: number of existing boxes per level
+    int *ad_cnt;              // [FMM_MAXL + 2] adaptive tree: number of existing boxes per level; then the number of
+                              // leaves in the lists below
+    int *ad_leaf;             // adaptive tree: [n] the list number of each sorted particle's leaf, -1: none (walked)
+    struct AdLeaf *ad_lists;  // adaptive tree: [ad_cap] the leaves' U and W lists
+    int ad_cap;
+    const double2 *blob_f;    // FP64 table of F (near64_table)
     // arrays
     int *key, *slot, *cnt, *start, *scan_tmp, *perm, *sleaf;
     int2 *tmp;                // [n] leaf order before the in-leaf ranking: (caller index, leaf) at the arrival slot;
@@ -338,6 +356,8 @@ int launch_far_tail(const Work &w, int rings, cudaStream_t s);
 // M2M), then the downward pass (per level L2L + M2L over V). Main stream, after the sweep, one kernel per target:
 // a walk of U and W, exact K_sigma over U if use_near, the multipoles of W and the leaf's local if use_far,
 // written in the caller's order.
+int launch_adaptive_boxes(const Work &w, cudaStream_t s);  // box lists: before the fork
+int launch_adaptive_lists(const Work &w, cudaStream_t s);  // the leaves' U and W lists, from the box lists
 int launch_adaptive_up(const Work &w, const Tables &t, cudaStream_t s);
 int launch_adaptive_down(const Work &w, const Tables &t, cudaStream_t s);
 int launch_adaptive_near(const Work &w, unsigned long long *pairs, int use_near, int use_far, double *u, double *v,
@@ -358,6 +378,7 @@ int m2l_tc_max_level();
 int prepare_m2l_tc();
 int launch_near64(const Work &w, cudaStream_t s);  // plain form's near field (near64.cu) into near64
 int launch_adjoint_near64(const Work &w, double *dg, double *dx, double *dy, int skip_plain, cudaStream_t s);
+const double2 *near64_table();  // its FP64 table of F on the current device, once prepared
 int prepare_near64(cudaStream_t s);  // its table, once per device before any stream capture; 0 on success
 int prepare_p2p();  // near-field kernel attributes, once per device before any stream capture; 0 on success
 int launch_m2l_tc(const Work &w, const Tables &t, int l_lo, int l_hi, cudaStream_t s);

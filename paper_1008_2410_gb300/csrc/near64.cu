@@ -14,7 +14,7 @@
 
 #include <mutex>
 
-#include "fmm_internal.cuh"
+#include "near64.cuh"
 
 namespace fmm {
 
@@ -80,37 +80,7 @@ __device__ int4 g_fix_f[kFixN * 2], g_fix_d[kFixN * 2];
 
 std::mutex g_tab_mu;
 bool g_tab_ready[64];
-
-// F(x) for 0 <= x < kXCut: the row from the bit pattern of x (integer operations), then one subtraction and six
-// multiply-adds.
-__device__ __forceinline__ int blob_row(double x)
-{
-    const int hi = __double2hiint(x);
-    const int e = (hi >> 20) - 1023;
-    return e >= -4 ? ((hi & 0xfffff) | 0x100000) >> (16 - e) : 0;
-}
-__device__ __forceinline__ double blob_poly(const double2 *__restrict__ tab, int i, double x)
-{
-    const double2 c01 = __ldg(tab + 4 * i), c23 = __ldg(tab + 4 * i + 1), c45 = __ldg(tab + 4 * i + 2),
-                  c6c = __ldg(tab + 4 * i + 3);
-    const double t = x - c6c.y;
-    double f = fma(c6c.x, t, c45.y);
-    f = fma(f, t, c45.x);
-    f = fma(f, t, c23.y);
-    f = fma(f, t, c23.x);
-    f = fma(f, t, c01.y);
-    return fma(f, t, c01.x);
-}
-
-// 1 / x to FP64 rounding for a normal x > 0: the SFU's seed (relative error below 2^-20) and one Newton step of third
-// order, y (1 + e + e^2) with e = 1 - x y.
-__device__ __forceinline__ double recip64(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
+const double2 *g_tab_f[64];  // device address of g_blob_f
 
 // ------------------------------------------------------------------ fixed point
 
@@ -930,8 +900,18 @@ int prepare_near64(cudaStream_t s)
         cudaFuncSetAttribute(k_near64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)N64_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(k_near64, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return -1;
+    void *f = nullptr;
+    if (cudaGetSymbolAddress(&f, g_blob_f) != cudaSuccess)
+        return -1;
+    g_tab_f[dev] = (const double2 *)f;
     g_tab_ready[dev] = true;
     return 0;
+}
+
+const double2 *near64_table()
+{
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? g_tab_f[dev] : nullptr;
 }
 
 // Persistent blocks, three to an SM, that take leaves from a counter: the register file (3 x 16 K of 64 K registers)
