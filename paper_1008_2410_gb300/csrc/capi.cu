@@ -315,7 +315,7 @@ static void build_system_layout(fmm_handle h, int64_t *nleaf_out, int64_t *nbox_
 }
 
 struct Layout {
-    size_t off[40];
+    size_t off[48];
     size_t total;
 };
 
@@ -332,7 +332,7 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     bool ad_mixed = h->mixed && !adjoint && h->adaptive_cap;  // ... and keeps FP32 expansions / split positions
     bool f64 = !mixed || adjoint;
     size_t np = (size_t)n + 8;
-    size_t sizes[40];
+    size_t sizes[48];
     int i = 0;
     sizes[i++] = np * 4;                                      // 0 key
     sizes[i++] = (size_t)nleaf * 4 + 16;                      // 1 cnt and the overflow flag
@@ -381,6 +381,8 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     const int ad_cap = h->adaptive_cap ? (int)std::min<int64_t>(n, n * 8 / h->adaptive_cap + 1024) : 0;
     sizes[i++] = h->adaptive_cap ? np * 4 : 0;                              // ad_leaf
     sizes[i++] = (size_t)ad_cap * sizeof(AdLeaf);                           // ad_lists
+    const bool sym = mixed && h->p2p_threads == 128;
+    sizes[i++] = sym ? (size_t)nleaf * 4 + 1024 + 256 : 0;                    // 40 order, order_cnt
     int count = i;
     Layout lay;
     size_t total = 0;
@@ -474,6 +476,8 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     w.ad_leaf = sizes[38] ? (int *)(b + lay.off[38]) : nullptr;
     w.ad_lists = sizes[39] ? (AdLeaf *)(b + lay.off[39]) : nullptr;
     w.ad_cap = ad_cap;
+    w.order_cnt = sizes[40] ? (int *)(b + lay.off[40]) : nullptr;
+    w.order = sizes[40] ? w.order_cnt + 256 : nullptr;
     w.blob_f = near64_table();
     w.big = (int *)(b + lay.off[31]);
     w.cls_off = sizes[32] ? (int *)(b + lay.off[32]) : nullptr;

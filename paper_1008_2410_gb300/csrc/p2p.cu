@@ -937,8 +937,9 @@ __device__ __forceinline__ f2 shfl2(f2 v, int src)
 
 // One chunk of 32 sources (SH, SG in shared memory) against the lane's KT targets. SELF: the sources are the
 // targets' own leaf (r' = 0 occurs; no reaction). SYM: accumulate the reaction on the source in RU, RV and
-// rotate it with the source.
-template <int KT, bool SELF, bool SYM>
+// rotate it with the source. FAR: every source is farther than 6 sigma from every target, where 2^-(r'^2) < 2^-25 leaves
+// g (1 - e) at g in FP32, and nothing is close enough for the series.
+template <int KT, bool SELF, bool SYM, bool FAR = false>
 __device__ __forceinline__ void p2ps_chunk(const float4 *__restrict__ SH, const float4 *__restrict__ SG, int lane,
                                            const f2 *AX, const f2 *AY, const f2 *GT, const f2 *GTN, f2 *PU, f2 *PV,
                                            f2 &RU, f2 &RV)
@@ -959,17 +960,19 @@ __device__ __forceinline__ void p2ps_chunk(const float4 *__restrict__ SH, const 
             r2[pr] = fma2(dx[pr], dx[pr], mul2(dy[pr], dy[pr]));
             float ra, rb;
             up2(r2[pr], ra, rb);
-            e[pr] = pk2(ex2_approx(-ra), ex2_approx(-rb));
+            if (!FAR)
+                e[pr] = pk2(ex2_approx(-ra), ex2_approx(-rb));
             if (SELF) {
                 q[pr] = pk2(rcp_approx(fmaxf(ra, 1e-30f)), rcp_approx(fmaxf(rb, 1e-30f)));
                 rmin = __uint_as_float(min(__float_as_uint(rmin), min(__float_as_uint(ra) - 1u, __float_as_uint(rb) - 1u)));
             } else {
                 q[pr] = pk2(rcp_approx(ra), rcp_approx(rb));
-                rmin = fminf(rmin, fminf(ra, rb));
+                if (!FAR)
+                    rmin = fminf(rmin, fminf(ra, rb));
             }
         }
         // rare (0 < r < sigma): the series gives (1 - e) q directly; e := 0, q := series
-        if (__any_sync(0xffffffffu, SELF ? (__float_as_uint(rmin) < __float_as_uint(P2P_THR)) : (rmin < P2P_THR))) {
+        if (!FAR && __any_sync(0xffffffffu, SELF ? (__float_as_uint(rmin) < __float_as_uint(P2P_THR)) : (rmin < P2P_THR))) {
 #pragma unroll
             for (int pr = 0; pr < NP; ++pr) {
                 float ra, rb, qa, qb, ea, eb, sa, sb;
@@ -991,11 +994,11 @@ __device__ __forceinline__ void p2ps_chunk(const float4 *__restrict__ SH, const 
         }
 #pragma unroll
         for (int pr = 0; pr < NP; ++pr) {
-            const f2 gf = mul2(fma2(e[pr], gn, gp), q[pr]);  // gamma_s (1 - e) q
+            const f2 gf = mul2(FAR ? gp : fma2(e[pr], gn, gp), q[pr]);  // gamma_s (1 - e) q
             PU[pr] = fma2(dy[pr], gf, PU[pr]);                // u accumulates -dy g f: negated at the end
             PV[pr] = fma2(dx[pr], gf, PV[pr]);
             if (SYM) {
-                const f2 gr = mul2(fma2(e[pr], GTN[pr], GT[pr]), q[pr]);  // gamma_t (1 - e) q
+                const f2 gr = mul2(FAR ? GT[pr] : fma2(e[pr], GTN[pr], GT[pr]), q[pr]);  // gamma_t (1 - e) q
                 RU = fma2(dy[pr], gr, RU);  // reaction on the source: u += +dy g f, v += -dx g f
                 RV = fma2(dx[pr], gr, RV);
             }
@@ -1007,6 +1010,7 @@ __device__ __forceinline__ void p2ps_chunk(const float4 *__restrict__ SH, const 
     }
 }
 
+#define P2PS_FAR2 27.0f  // r'^2 past which e < 2^-25, with room for the rounding of the leaf frame
 #ifndef P2PS_MIN_BLOCKS
 #define P2PS_MIN_BLOCKS 6  // minimum resident 128-thread blocks per SM for the symmetric kernel (80 registers)
 #endif
@@ -1053,14 +1057,73 @@ __device__ __forceinline__ void stream_load(const Work &w, const SymStream &S, i
     }
 }
 
+// Leaves in order of falling work (passes over the targets times the sources of a pass): a warp per leaf takes from
+// microseconds to milliseconds on clustered particles, and the long ones must not start last. Classes of a quarter
+// octave, counted by the first kernel and filled by the second; the order within a class varies from run to run, which
+// only changes where a leaf runs. P2PS_ORDER_NOTE
+constexpr int kWorkClasses = 128;
+__device__ __forceinline__ int work_class(const Work &w, int A, int per_pass)
+{
+    const SysDev &d = w.sys[w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, A)];
+    const int ns = 1 << d.depth, local = A - (int)d.leaf0, ax = local & (ns - 1), ay = local >> d.depth;
+    const int c = w.start[A + 1] - w.start[A];
+    int src = c;
+#pragma unroll
+    for (int dd = 0; dd < 4; ++dd) {
+        const int bx = ax + c_p2p_fwd[dd].x, by = ay + c_p2p_fwd[dd].y;
+        if (bx >= 0 && bx < ns && by < ns) {
+            const int B = (int)d.leaf0 + by * ns + bx;
+            src += w.start[B + 1] - w.start[B];
+        }
+    }
+    const float work = (float)((c + per_pass - 1) / per_pass) * (float)src;
+    return work < 1.f ? kWorkClasses - 1 : max(0, kWorkClasses - 2 - (int)((__float_as_uint(work) >> 21) - 508u));
+}
+__global__ void __launch_bounds__(256) k_work_count(Work w, int per_pass)
+{
+    __shared__ int hist[kWorkClasses];
+    for (int i = threadIdx.x; i < kWorkClasses; i += blockDim.x)
+        hist[i] = 0;
+    __syncthreads();
+    const int A = blockIdx.x * blockDim.x + threadIdx.x;
+    if (A < w.nleaf)
+        atomicAdd(&hist[work_class(w, A, per_pass)], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kWorkClasses; i += blockDim.x)
+        if (hist[i])
+            atomicAdd(&w.order_cnt[i], hist[i]);
+}
+__global__ void __launch_bounds__(256) k_work_order(Work w, int per_pass)
+{
+    __shared__ int hist[kWorkClasses], base[kWorkClasses];
+    const int t = threadIdx.x;
+    if (t < kWorkClasses)
+        hist[t] = 0;
+    __syncthreads();
+    const int A = blockIdx.x * blockDim.x + t;
+    const int k = A < w.nleaf ? work_class(w, A, per_pass) : -1;
+    const int at = k >= 0 ? atomicAdd(&hist[k], 1) : 0;
+    __syncthreads();
+    if (t < kWorkClasses) {
+        int first = 0;
+        for (int i = 0; i < t; ++i)
+            first += w.order_cnt[i];
+        base[t] = first + (hist[t] ? atomicAdd(&w.order_cnt[kWorkClasses + t], hist[t]) : 0);
+    }
+    __syncthreads();
+    if (k >= 0)
+        w.order[base[k] + at] = A;
+}
+
 template <int LW>
-__global__ void __launch_bounds__(32 * LW, P2PS_MIN_BLOCKS) k_p2p32s(Work w, int ktmax)
+__global__ void __launch_bounds__(32 * LW, P2PS_MIN_BLOCKS) k_p2p32s(Work w, int ktmax, int ordered)
 {
     __shared__ float4 sh_h[LW][32], sh_g[LW][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int A = blockIdx.x * LW + warp;
-    if (A >= w.nleaf)
+    const int unit = blockIdx.x * LW + warp;
+    if (unit >= w.nleaf)
         return;  // warp-uniform; warps never synchronise with each other
+    const int A = ordered ? w.order[unit] : unit;
     const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, A);
     const SysDev &d = w.sys[k];
     if (d.s_unit > P2P_SPLIT_S)
@@ -1143,10 +1206,22 @@ __global__ void __launch_bounds__(32 * LW, P2PS_MIN_BLOCKS) k_p2p32s(Work w, int
                 else
                     p2ps_chunk<4, true, false>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
             } else {
-                if (kt == 2)
-                    p2ps_chunk<2, false, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-                else
-                    p2ps_chunk<4, false, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
+                // this lane's source's distance from A's square, past which a chunk runs without exponentials: leaves
+                // are ordered by boundary band, so that whole chunks lie on either side of it
+                const float4 hs = SH[lane];
+                const float ex = fmaxf(fabsf(hs.x) - 0.5f * s, 0.f), ey = fmaxf(fabsf(hs.z) - 0.5f * s, 0.f);
+                const bool away = __all_sync(0xffffffffu, ex * ex + ey * ey > P2PS_FAR2);
+                if (kt == 2) {
+                    if (away)
+                        p2ps_chunk<2, false, true, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
+                    else
+                        p2ps_chunk<2, false, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
+                } else {
+                    if (away)
+                        p2ps_chunk<4, false, true, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
+                    else
+                        p2ps_chunk<4, false, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
+                }
                 if (dir >= 0) {  // reaction on this lane's source (pass 0 writes, later passes add)
                     float ru0, ru1, rv0, rv1;
                     up2(RU, ru0, ru1);
@@ -1221,7 +1296,14 @@ int launch_p2p(const Work &w, int threads, int kt, cudaStream_t s)
     if (threads == 128 && w.p2p_sym) {
         // symmetric near field for the one-float systems; k_p2p32 only where a system may need split coordinates
         constexpr int LW = 4;
-        k_p2p32s<LW><<<(w.nleaf + LW - 1) / LW, 32 * LW, 0, s>>>(w, ktmax);
+        const int ordered = w.order && w.nleaf > kSMs * P2PS_MIN_BLOCKS * LW;  // fewer are all resident at once
+        if (ordered) {
+            cudaMemsetAsync(w.order_cnt, 0, 2 * kWorkClasses * sizeof(int), s);
+            k_work_count<<<(w.nleaf + 255) / 256, 256, 0, s>>>(w, 32 * ktmax);
+            k_work_order<<<(w.nleaf + 255) / 256, 256, 0, s>>>(w, 32 * ktmax);
+            nl += 2;
+        }
+        k_p2p32s<LW><<<(w.nleaf + LW - 1) / LW, 32 * LW, 0, s>>>(w, ktmax, ordered);
         ++nl;
         if (!w.p2p_all_plain) {
             const int tile = 192;
