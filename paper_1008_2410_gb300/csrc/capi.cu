@@ -381,8 +381,7 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     const int ad_cap = h->adaptive_cap ? (int)std::min<int64_t>(n, n * 8 / h->adaptive_cap + 1024) : 0;
     sizes[i++] = h->adaptive_cap ? np * 4 : 0;                              // ad_leaf
     sizes[i++] = (size_t)ad_cap * sizeof(AdLeaf);                           // ad_lists
-    const bool sym = mixed && h->p2p_threads == 128;
-    sizes[i++] = sym ? (size_t)nleaf * 4 + 1024 + 256 : 0;                    // 40 order, order_cnt
+    sizes[i++] = mixed ? (size_t)nleaf * 4 + 2048 : 0;                         // 40 order, order_cnt (any tile: it may change)
     int count = i;
     Layout lay;
     size_t total = 0;
@@ -477,7 +476,7 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     w.ad_lists = sizes[39] ? (AdLeaf *)(b + lay.off[39]) : nullptr;
     w.ad_cap = ad_cap;
     w.order_cnt = sizes[40] ? (int *)(b + lay.off[40]) : nullptr;
-    w.order = sizes[40] ? w.order_cnt + 256 : nullptr;
+    w.order = sizes[40] ? w.order_cnt + 512 : nullptr;
     w.blob_f = near64_table();
     w.big = (int *)(b + lay.off[31]);
     w.cls_off = sizes[32] ? (int *)(b + lay.off[32]) : nullptr;

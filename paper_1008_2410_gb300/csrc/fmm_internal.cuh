@@ -207,7 +207,7 @@ struct Work {
     unsigned int *status_host;  // page-locked copy of *status written by the final sum kernel, or null
     float2 *nearp;            // [4][n] leaf order: symmetric near field, reactions from the leaf at -P2P
                               // forward offset d (d = 0..3: (1,0), (1,1), (0,1), (-1,1)), or null
-    int *order, *order_cnt;   // symmetric near field: leaves by falling work, or null; the classes' counters [256]
+    int *order, *order_cnt;   // symmetric near field: leaves by falling work, or null; the classes' counters [512]
     int p2p_all_plain;        // host knows every system takes one-float near-field coordinates
     int p2p_sym;              // this evaluation's near field is the symmetric kernel (nearp holds reactions)
     int p2p_rows;             // this evaluation's near field comes per source row (nearp[0..2] hold the parts)

@@ -1011,10 +1011,6 @@ __device__ __forceinline__ void p2ps_chunk(const float4 *__restrict__ SH, const 
 }
 
 #define P2PS_FAR2 27.0f  // r'^2 past which e < 2^-25, with room for the rounding of the leaf frame
-#ifndef P2PS_MIN_BLOCKS
-#define P2PS_MIN_BLOCKS 6  // minimum resident 128-thread blocks per SM for the symmetric kernel (80 registers)
-#endif
-
 // Source stream of one target leaf A: A's own particles (padded to a multiple of 32), then the particles of
 // its forward neighbours in order d = 0..3, shifted into A's frame when they are staged. Stream position ->
 // (source index, forward direction d or -1 for A itself, or padding).
@@ -1057,10 +1053,10 @@ __device__ __forceinline__ void stream_load(const Work &w, const SymStream &S, i
     }
 }
 
-// Leaves in order of falling work (passes over the targets times the sources of a pass): a warp per leaf takes from
+// Leaves in order of falling work (passes over the targets times the sources of a pass): a leaf takes a warp from
 // microseconds to milliseconds on clustered particles, and the long ones must not start last. Classes of a quarter
 // octave, counted by the first kernel and filled by the second; the order within a class varies from run to run, which
-// only changes where a leaf runs. P2PS_ORDER_NOTE
+// only changes where a leaf runs. The two and the clearing take 10 us at 4096 leaves.
 constexpr int kWorkClasses = 128;
 __device__ __forceinline__ int work_class(const Work &w, int A, int per_pass)
 {
@@ -1078,6 +1074,10 @@ __device__ __forceinline__ int work_class(const Work &w, int A, int per_pass)
     }
     const float work = (float)((c + per_pass - 1) / per_pass) * (float)src;
     return work < 1.f ? kWorkClasses - 1 : max(0, kWorkClasses - 2 - (int)((__float_as_uint(work) >> 21) - 508u));
+}
+__device__ __forceinline__ float class_work(int c)  // the least work of a class below the last
+{
+    return __uint_as_float((unsigned)(kWorkClasses - 2 - c + 508) << 21);
 }
 __global__ void __launch_bounds__(256) k_work_count(Work w, int per_pass)
 {
@@ -1115,56 +1115,11 @@ __global__ void __launch_bounds__(256) k_work_order(Work w, int per_pass)
         w.order[base[k] + at] = A;
 }
 
-template <int LW>
-__global__ void __launch_bounds__(32 * LW, P2PS_MIN_BLOCKS) k_p2p32s(Work w, int ktmax, int ordered)
-{
-    __shared__ float4 sh_h[LW][32], sh_g[LW][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int unit = blockIdx.x * LW + warp;
-    if (unit >= w.nleaf)
-        return;  // warp-uniform; warps never synchronise with each other
-    const int A = ordered ? w.order[unit] : unit;
-    const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, A);
-    const SysDev &d = w.sys[k];
-    if (d.s_unit > P2P_SPLIT_S)
-        return;  // split-coordinate system: k_p2p32
-    const int L = d.depth, ns = 1 << L, local = A - (int)d.leaf0;
-    const int ax = local & (ns - 1), ay = local >> L;
-    SymStream S;
-    S.a0 = w.start[A];
-    S.ac = w.start[A + 1] - S.a0;
-    if (S.ac == 0)
-        return;
-    const float s = d.s_unit, snear = d.snear;
-    const int n = w.n;
-    S.selfpad = (S.ac + 31) & ~31;
-    S.fpre[0] = 0;
-#pragma unroll
-    for (int dd = 0; dd < 4; ++dd) {
-        const int2 o = c_p2p_fwd[dd];
-        const int bx = ax + o.x, by = ay + o.y;
-        int cnt = 0, b0 = 0;
-        if (bx >= 0 && bx < ns && by < ns) {
-            const int B = (int)d.leaf0 + by * ns + bx;
-            b0 = w.start[B];
-            cnt = w.start[B + 1] - b0;
-        }
-        S.fb0[dd] = b0;
-        S.fpre[dd + 1] = S.fpre[dd] + cnt;
-        S.fsx[dd] = (float)o.x * s;
-        S.fsy[dd] = (float)o.y * s;
-    }
-    S.total = S.selfpad + S.fpre[4];
-    float4 *SH = sh_h[warp], *SG = sh_g[warp];
-    const int per_pass = 32 * ktmax;
-    const int np = (S.ac + per_pass - 1) / per_pass;
-    for (int pass = 0; pass < np; ++pass) {
-        const int t_lo = (int)((int64_t)pass * S.ac / np);
-        const int t_cnt = (int)((int64_t)(pass + 1) * S.ac / np) - t_lo;
-        const int kt = t_cnt <= 64 ? 2 : 4;
-        const int tbase = S.a0 + t_lo;
-        // the lane's targets in A's frame, one float per coordinate; charges (and negated) per packed pair
-        f2 AX[2], AY[2], GT[2], GTN[2];
+// The lane's targets of a pass in A's frame, one float per coordinate; charges (and negated) per packed pair.
+struct SymTargets {
+    f2 AX[2], AY[2], GT[2], GTN[2];
+    __device__ __forceinline__ void load(const Work &w, int tbase, int t_cnt, int lane)
+    {
 #pragma unroll
         for (int pr = 0; pr < 2; ++pr) {
             float hx[2], hy[2], gv[2];
@@ -1187,74 +1142,224 @@ __global__ void __launch_bounds__(32 * LW, P2PS_MIN_BLOCKS) k_p2p32s(Work w, int
             GT[pr] = pk2(gv[0], gv[1]);
             GTN[pr] = pk2(-gv[0], -gv[1]);
         }
-        f2 SU[2] = {0ull, 0ull}, CU[2] = {0ull, 0ull}, SV[2] = {0ull, 0ull}, CV[2] = {0ull, 0ull};
-        float4 nh, ng;
-        int nsrc, ndir;
-        stream_load(w, S, lane, nh, ng, nsrc, ndir);
-        for (int c0 = 0; c0 < S.total; c0 += 32) {
-            const int src = nsrc, dir = ndir;
-            __syncwarp();  // the previous chunk is no longer read
-            SH[lane] = nh;
-            SG[lane] = ng;
-            __syncwarp();
-            if (c0 + 32 < S.total)
-                stream_load(w, S, c0 + 32 + lane, nh, ng, nsrc, ndir);  // next chunk, in flight meanwhile
-            f2 PU[2] = {0ull, 0ull}, PV[2] = {0ull, 0ull}, RU = 0ull, RV = 0ull;
-            if (c0 < S.selfpad) {
-                if (kt == 2)
-                    p2ps_chunk<2, true, false>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-                else
-                    p2ps_chunk<4, true, false>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-            } else {
-                // this lane's source's distance from A's square, past which a chunk runs without exponentials: leaves
-                // are ordered by boundary band, so that whole chunks lie on either side of it
-                const float4 hs = SH[lane];
-                const float ex = fmaxf(fabsf(hs.x) - 0.5f * s, 0.f), ey = fmaxf(fabsf(hs.z) - 0.5f * s, 0.f);
-                const bool away = __all_sync(0xffffffffu, ex * ex + ey * ey > P2PS_FAR2);
-                if (kt == 2) {
-                    if (away)
-                        p2ps_chunk<2, false, true, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-                    else
-                        p2ps_chunk<2, false, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-                } else {
-                    if (away)
-                        p2ps_chunk<4, false, true, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-                    else
-                        p2ps_chunk<4, false, true>(SH, SG, lane, AX, AY, GT, GTN, PU, PV, RU, RV);
-                }
-                if (dir >= 0) {  // reaction on this lane's source (pass 0 writes, later passes add)
-                    float ru0, ru1, rv0, rv1;
-                    up2(RU, ru0, ru1);
-                    up2(RV, rv0, rv1);
-                    float2 r = make_float2((ru0 + ru1) * snear, -(rv0 + rv1) * snear);
-                    float2 *dst = w.nearp + (int64_t)dir * n + src;
-                    if (pass > 0) {
-                        const float2 old = *dst;
-                        r.x += old.x;
-                        r.y += old.y;
-                    }
-                    *dst = r;
-                }
-            }
-#pragma unroll
-            for (int pr = 0; pr < 2; ++pr) {
-                two_sum2(SU[pr], CU[pr], PU[pr]);
-                two_sum2(SV[pr], CV[pr], PV[pr]);
-            }
+    }
+};
+
+// One chunk of 32 sources, staged in SH, SG (one per lane: `src`, `dir` of this lane's): the targets' sums PU, PV, and
+// the reactions to nearp (pass 0 writes, later passes add).
+__device__ __forceinline__ void sym_chunk(const Work &w, const SymTargets &T, const float4 *SH, const float4 *SG, bool self,
+                                          int kt, float s, float snear, int src, int dir, int pass, int lane, f2 *PU, f2 *PV)
+{
+    f2 RU = 0ull, RV = 0ull;
+    if (self) {
+        if (kt == 2)
+            p2ps_chunk<2, true, false>(SH, SG, lane, T.AX, T.AY, T.GT, T.GTN, PU, PV, RU, RV);
+        else
+            p2ps_chunk<4, true, false>(SH, SG, lane, T.AX, T.AY, T.GT, T.GTN, PU, PV, RU, RV);
+        return;
+    }
+    // this lane's source's distance from A's square, past which a chunk runs without exponentials: leaves are ordered by
+    // boundary band, so that whole chunks lie on either side of it
+    const float4 hs = SH[lane];
+    const float ex = fmaxf(fabsf(hs.x) - 0.5f * s, 0.f), ey = fmaxf(fabsf(hs.z) - 0.5f * s, 0.f);
+    const bool away = __all_sync(0xffffffffu, ex * ex + ey * ey > P2PS_FAR2);
+    if (kt == 2) {
+        if (away)
+            p2ps_chunk<2, false, true, true>(SH, SG, lane, T.AX, T.AY, T.GT, T.GTN, PU, PV, RU, RV);
+        else
+            p2ps_chunk<2, false, true>(SH, SG, lane, T.AX, T.AY, T.GT, T.GTN, PU, PV, RU, RV);
+    } else {
+        if (away)
+            p2ps_chunk<4, false, true, true>(SH, SG, lane, T.AX, T.AY, T.GT, T.GTN, PU, PV, RU, RV);
+        else
+            p2ps_chunk<4, false, true>(SH, SG, lane, T.AX, T.AY, T.GT, T.GTN, PU, PV, RU, RV);
+    }
+    if (dir >= 0) {
+        float ru0, ru1, rv0, rv1;
+        up2(RU, ru0, ru1);
+        up2(RV, rv0, rv1);
+        float2 r = make_float2((ru0 + ru1) * snear, -(rv0 + rv1) * snear);
+        float2 *dst = w.nearp + (int64_t)dir * w.n + src;
+        if (pass > 0) {
+            const float2 old = *dst;
+            r.x += old.x;
+            r.y += old.y;
         }
+        *dst = r;
+    }
+}
+
+__device__ __forceinline__ void sym_store(const Work &w, f2 su_cu, f2 sv_cv, int pr, int tbase, int t_cnt, int lane, float snear)
+{
+    float u[2], v[2];
+    up2(su_cu, u[0], u[1]);
+    up2(sv_cv, v[0], v[1]);
 #pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
-            float su[2], cu[2], svv[2], cv[2];
-            up2(SU[pr], su[0], su[1]);
-            up2(CU[pr], cu[0], cu[1]);
-            up2(SV[pr], svv[0], svv[1]);
-            up2(CV[pr], cv[0], cv[1]);
+    for (int hh = 0; hh < 2; ++hh) {
+        const int e = lane + 32 * (2 * pr + hh);
+        if (e < t_cnt)
+            w.near32[(int64_t)(tbase + e) * w.nf_stride] = make_float2(-u[hh] * snear, v[hh] * snear);
+    }
+}
+
+// A leaf on a block (coop): warp k runs chunks k, k + SYM_W, ... of a pass, and the chunks' sums are added by TwoSum in
+// the order of the stream, one accumulator to a warp, so the bits are those of a warp alone; the reactions of a source
+// come from the same lane in each pass.
+// ordered: persistent blocks take leaves from counters in the order of falling work. Those of more than a part of a
+// warp's share of all work (and of SYM_MIN_WORK) take a block each: the densest leaf would bound the kernel else. Then
+// each warp takes leaves of its own. Otherwise (few leaves) every leaf has a block of its own.
+// Issue bound where it is large (2^21 particles in 8 patches at depth 8: 66% of the issue slots; 64 registers with
+// spills around the chunks for 32 resident warps are 5% faster than 80 for 24). Evaluation in a graph, us, a warp per
+// leaf in leaf order / now: 8 patches of 2^24 particles at depth 9 28500 / 25600, 2^21 at depth 8 2920 / 2430, 2^20 at
+// depth 7 7800 / 2200, 300000 at depth 6 5990 / 1130; uniform 2^20 at depth 7 612 / 612, 2^18 at depth 6 198 / 201,
+// 65536 at depth 5 88 / 67, 4096 at depth 3 69 / 38; 16384 clustered at depth 4 47400 / 7400.
+constexpr float SYM_SHARE = 2.f;       // heavy: 1 / SYM_SHARE of a warp's share (2^24, 2^21 patches: 4 3% and 6% slower,
+constexpr float SYM_MIN_WORK = 1024.f; // 1 equal and 8%); a minimum of 4096 takes 50% longer on 300000 in patches
+template <int SYM_W, int SYM_SM, bool ordered>
+__global__ void __launch_bounds__(32 * SYM_W, SYM_SM / SYM_W) k_p2p32s(Work w, int ktmax)
+{
+    __shared__ float4 sh_h[SYM_W][32], sh_g[SYM_W][32];
+    __shared__ f2 part[2][SYM_W][4][32];
+    __shared__ int s_unit, s_heavy;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float4 *SH = sh_h[warp], *SG = sh_g[warp];
+    int heavy = 0;
+    if (ordered) {
+        if (warp == 0) {
+            // every warp's share of the work, from the classes' lower bounds; the number of leaves above a part of it
+            float work = 0.f;
+            for (int c = lane; c < kWorkClasses - 1; c += 32)
+                work += (float)w.order_cnt[c] * class_work(c);
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int e = lane + 32 * (2 * pr + hh);
-                if (e < t_cnt)
-                    w.near32[(int64_t)(tbase + e) * w.nf_stride] =
-                        make_float2(-(su[hh] + cu[hh]) * snear, (svv[hh] + cv[hh]) * snear);
+            for (int o = 16; o; o >>= 1)
+                work += __shfl_xor_sync(0xffffffffu, work, o);
+            const float limit = fmaxf(SYM_MIN_WORK, work / (SYM_SHARE * SYM_W * gridDim.x));
+            int nh = 0;
+            for (int c = lane; c < kWorkClasses - 1; c += 32)
+                nh += class_work(c) >= limit ? w.order_cnt[c] : 0;
+            nh = __reduce_add_sync(0xffffffffu, nh);
+            if (lane == 0)
+                s_heavy = nh;
+        }
+        __syncthreads();
+        heavy = s_heavy;
+    }
+    bool coop = true, first = true;
+    for (;;) {
+        int A = warp * gridDim.x + blockIdx.x;  // ordered: a first leaf for the warp alone, over all SMs
+        if (ordered) {
+            if (coop) {
+                __syncthreads();
+                if (threadIdx.x == 0)
+                    s_unit = atomicAdd(w.order_cnt + 2 * kWorkClasses, 1);
+                __syncthreads();
+                coop = s_unit < heavy;
+            }
+            if (coop) {
+                A = s_unit;
+            } else if (first) {
+                first = false;
+                A += heavy;
+            } else {
+                if (lane == 0)
+                    A = heavy + SYM_W * gridDim.x + atomicAdd(w.order_cnt + 2 * kWorkClasses + 1, 1);
+                A = __shfl_sync(0xffffffffu, A, 0);
+            }
+            if (A >= w.nleaf)
+                return;  // only once the block's heavy leaves are done
+            A = w.order[A];
+        } else {
+            if (!first)
+                return;
+            first = false;
+            A = blockIdx.x;
+        }
+        const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, A);
+        const SysDev &d = w.sys[k];
+        if (d.s_unit > P2P_SPLIT_S)
+            continue;  // split-coordinate system: k_p2p32
+        const int L = d.depth, ns = 1 << L, local = A - (int)d.leaf0;
+        const int ax = local & (ns - 1), ay = local >> L;
+        SymStream S;
+        S.a0 = w.start[A];
+        S.ac = w.start[A + 1] - S.a0;
+        if (S.ac == 0)
+            continue;
+        const float s = d.s_unit, snear = d.snear;
+        S.selfpad = (S.ac + 31) & ~31;
+        S.fpre[0] = 0;
+#pragma unroll
+        for (int dd = 0; dd < 4; ++dd) {
+            const int2 o = c_p2p_fwd[dd];
+            const int bx = ax + o.x, by = ay + o.y;
+            int cnt = 0, b0 = 0;
+            if (bx >= 0 && bx < ns && by < ns) {
+                const int B = (int)d.leaf0 + by * ns + bx;
+                b0 = w.start[B];
+                cnt = w.start[B + 1] - b0;
+            }
+            S.fb0[dd] = b0;
+            S.fpre[dd + 1] = S.fpre[dd] + cnt;
+            S.fsx[dd] = (float)o.x * s;
+            S.fsy[dd] = (float)o.y * s;
+        }
+        S.total = S.selfpad + S.fpre[4];
+        const int per_pass = 32 * ktmax;
+        const int np = (S.ac + per_pass - 1) / per_pass;
+        const int c_first = coop ? 32 * warp : 0, c_step = coop ? 32 * SYM_W : 32;
+        const int c_end = coop ? (S.total + 32 * SYM_W - 1) / (32 * SYM_W) * (32 * SYM_W) : S.total;  // whole rounds
+        for (int pass = 0; pass < np; ++pass) {
+            const int t_lo = (int)((int64_t)pass * S.ac / np);
+            const int t_cnt = (int)((int64_t)(pass + 1) * S.ac / np) - t_lo;
+            const int kt = t_cnt <= 64 ? 2 : 4;
+            const int tbase = S.a0 + t_lo;
+            SymTargets T;
+            T.load(w, tbase, t_cnt, lane);
+            f2 SU[2] = {0ull, 0ull}, CU[2] = {0ull, 0ull}, SV[2] = {0ull, 0ull}, CV[2] = {0ull, 0ull};
+            float4 nh4, ng4;
+            int nsrc, ndir, buf = 0;
+            stream_load(w, S, c_first + lane, nh4, ng4, nsrc, ndir);
+            for (int c0 = c_first; c0 < c_end; c0 += c_step, buf ^= 1) {
+                const int src = nsrc, dir = ndir;
+                __syncwarp();  // the previous chunk is no longer read
+                SH[lane] = nh4;
+                SG[lane] = ng4;
+                __syncwarp();
+                if (c0 + c_step < S.total)
+                    stream_load(w, S, c0 + c_step + lane, nh4, ng4, nsrc, ndir);  // next chunk, in flight meanwhile
+                f2 PU[2] = {0ull, 0ull}, PV[2] = {0ull, 0ull};
+                if (c0 < S.total)
+                    sym_chunk(w, T, SH, SG, c0 < S.selfpad, kt, s, snear, src, dir, pass, lane, PU, PV);
+                if (coop) {
+                    part[buf][warp][0][lane] = PU[0];
+                    part[buf][warp][1][lane] = PV[0];
+                    part[buf][warp][2][lane] = PU[1];
+                    part[buf][warp][3][lane] = PV[1];
+                    __syncthreads();
+                    if (warp < 4) {  // accumulator `warp` over the round's chunks, in the stream's order
+                        const int nc = min(SYM_W, (S.total - (c0 - 32 * warp) + 31) / 32);
+                        for (int q = 0; q < nc; ++q)
+                            two_sum2(SU[0], CU[0], part[buf][q][warp][lane]);
+                    }
+                } else {
+#pragma unroll
+                    for (int pr = 0; pr < 2; ++pr) {
+                        two_sum2(SU[pr], CU[pr], PU[pr]);
+                        two_sum2(SV[pr], CV[pr], PV[pr]);
+                    }
+                }
+            }
+            if (coop) {
+                __syncthreads();
+                if (warp < 4)
+                    part[0][0][warp][lane] = add2(SU[0], CU[0]);
+                __syncthreads();
+                if (warp < 2)
+                    sym_store(w, part[0][0][2 * warp][lane], part[0][0][2 * warp + 1][lane], warp, tbase, t_cnt, lane, snear);
+                __syncthreads();
+            } else {
+                sym_store(w, add2(SU[0], CU[0]), add2(SV[0], CV[0]), 0, tbase, t_cnt, lane, snear);
+                sym_store(w, add2(SU[1], CU[1]), add2(SV[1], CV[1]), 1, tbase, t_cnt, lane, snear);
             }
         }
     }
@@ -1295,15 +1400,20 @@ int launch_p2p(const Work &w, int threads, int kt, cudaStream_t s)
     int nl = 0;
     if (threads == 128 && w.p2p_sym) {
         // symmetric near field for the one-float systems; k_p2p32 only where a system may need split coordinates
-        constexpr int LW = 4;
-        const int ordered = w.order && w.nleaf > kSMs * P2PS_MIN_BLOCKS * LW;  // fewer are all resident at once
-        if (ordered) {
-            cudaMemsetAsync(w.order_cnt, 0, 2 * kWorkClasses * sizeof(int), s);
+        // few leaves: a block each, of 16 warps while two blocks an SM hold them all, else of 4. 1024 uniform leaves of
+        // 64 67 us (16 warps 88, persistent 97); at 4096 uniform leaves of 64 blocks of 4 would take 178 us, not 201,
+        // but 2^18 particles in patches 1660, not 1100
+        if (w.nleaf <= 2 * kSMs) {
+            k_p2p32s<16, 32, false><<<w.nleaf, 512, 0, s>>>(w, ktmax);
+        } else if (w.nleaf <= 1024) {
+            k_p2p32s<4, 28, false><<<w.nleaf, 128, 0, s>>>(w, ktmax);
+        } else {
+            cudaMemsetAsync(w.order_cnt, 0, (2 * kWorkClasses + 2) * sizeof(int), s);
             k_work_count<<<(w.nleaf + 255) / 256, 256, 0, s>>>(w, 32 * ktmax);
             k_work_order<<<(w.nleaf + 255) / 256, 256, 0, s>>>(w, 32 * ktmax);
+            k_p2p32s<16, 32, true><<<2 * kSMs, 512, 0, s>>>(w, ktmax);
             nl += 2;
         }
-        k_p2p32s<LW><<<(w.nleaf + LW - 1) / LW, 32 * LW, 0, s>>>(w, ktmax, ordered);
         ++nl;
         if (!w.p2p_all_plain) {
             const int tile = 192;
