@@ -549,7 +549,6 @@ static fmm_status enqueue_adaptive(fmm_handle h, cudaStream_t s, int mode, const
     CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the plain form's next leaf
     if (!h->has_domain) {
         nl += launch_bbox(w, x, y, s);
-        nl += launch_domain_finalize(w, s);
     }
     nl += launch_keys(w, x, y, g, s);
     nl += launch_scan(w, s);
@@ -637,7 +636,6 @@ static fmm_status enqueue_forward(fmm_handle h, cudaStream_t s, int mode, const 
         any_bbox |= !c.explicit_domain;
     if (any_bbox) {  // explicit squares: the host derived the constants
         nl += launch_bbox(w, x, y, s);
-        nl += launch_domain_finalize(w, s);
     }
     nl += launch_keys(w, x, y, g, s);
     nl += launch_scan(w, s);
@@ -1367,7 +1365,6 @@ fmm_status fmm_velocity_adjoint(fmm_handle h, int64_t n, const double *x, const 
     CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the plain form's next leaf
     if (!h->has_domain) {
         nl += launch_bbox(w, x, y, s);
-        nl += launch_domain_finalize(w, s);
     }
     nl += launch_keys(w, x, y, gamma, s);
     nl += launch_scan(w, s);

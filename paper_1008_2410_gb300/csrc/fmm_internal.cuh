@@ -321,8 +321,8 @@ __device__ inline int find_sys_by_leaf(const SysDev *sys, int nsys, int64_t leaf
 }
 
 // ---- launchers (each returns the number of kernels launched) ----
-int launch_bbox(const Work &w, const double *x, const double *y, cudaStream_t s);
-int launch_domain_finalize(const Work &w, cudaStream_t s);
+int launch_bbox(const Work &w, const double *x, const double *y, cudaStream_t s);  // squares and constants
+int launch_constants(const Work &w, cudaStream_t s);  // explicit squares
 __host__ __device__ void derive_constants(SysDev &d);  // binning.cu: per-system constants from square, depth, sigma
 int launch_keys(const Work &w, const double *x, const double *y, const double *g, cudaStream_t s);
 int launch_scan(const Work &w, cudaStream_t s);  // cnt -> start

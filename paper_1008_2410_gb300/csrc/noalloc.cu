@@ -265,7 +265,8 @@ extern "C" fmm_status fmm_velocity_noalloc(int tree_depth, int p, double sigma, 
     // the same stages as fmm_velocity, in order on the caller's stream (no second stream, no events)
     if (!domain)
         launch_bbox(w, x, y, s);
-    launch_domain_finalize(w, s);
+    else
+        launch_constants(w, s);
     launch_keys(w, x, y, gamma, s);
     launch_scan(w, s);
     launch_scatter_sort(w, s);
