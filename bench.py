@@ -276,7 +276,7 @@ def run_ours(args, rank: int, world: int, local_rank: int) -> dict | None:
             traffic = None
     out["roofline"] = {"bound": "alu", "kernel": (f"{kname} (near field, stage 9, tile {tuned['p2p_threads']}x"
                                                    f"{tuned['p2p_targets_per_thread']})") if args.precision == "mixed"
-                       else "k_p2p64 (near field, stage 9)",
+                       else "k_near64 (near field, stage 9)",
                        "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                        "frac": achieved / FP32_PEAK_TFLOPS if achieved else None, "traffic": traffic,
                        "pairs_per_launch": pairs, "avg_launch_ms": p2p_avg,

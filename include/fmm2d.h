@@ -11,9 +11,9 @@
  *   1 root square (given, or the bounding-box rule below)  2 particle binning into leaves
  *   3 interaction lists (implicit on the uniform tree)     4 P2M  5 M2M  6 M2L  7 L2L  8 L2P
  *   9 near-field direct sum (P2P)                          10 sum of near and far parts
- * Stage 9 runs on the caller's stream while stages 4-7 run concurrently on a second, high-priority stream
- * (Fig. 1: no dependency between {4,5,6,7} and {9}). Stage 8 runs on that second stream too in the precision
- * form (the far field is ready at the join); in the plain FP64 form it is fused into stage 10 after the join.
+ * Stages 9 and 4-7 run concurrently on the caller's stream and a second, high-priority stream (Fig. 1: no dependency
+ * between {4,5,6,7} and {9}). In the precision form stages 4-8 have the second stream (the far field is ready at the
+ * join); in the plain FP64 form stage 9 has it, and stage 8 is fused into stage 10 after the join.
  *
  * Conventions for every call:
  *   - Array arguments of fmm_velocity*, fmm_velocity_adjoint and fmm_velocity_batched are DEVICE pointers
@@ -56,7 +56,7 @@ typedef enum {
 } fmm_status;
 
 typedef enum {
-    FMM_FP64 = 0,  /* plain form: every stage in FP64 */
+    FMM_FP64 = 0,  /* plain form: FP64 accuracy in every stage (near field in 64-bit fixed point) */
     FMM_MIXED = 1  /* precision form: FP32 near field (leaf-relative split coordinates, small-r series,
                       compensated sums), FP32 expansions; FP64 binning (bit-exact leaves) and, optionally,
                       FP64 coarse levels (fmm_set_coarse_level) */

@@ -5,7 +5,8 @@
 //   caller stream : [1-2] bbox, keys, scan, scatter, in-leaf order, gather --fork-->  [9] P2P  --join--> [8+10]
 //   side stream   :                                                          [4] P2M [5] M2M [6] M2L [7] L2L
 // The side stream has the highest priority, so whenever near-field blocks retire the block scheduler issues
-// the (small, latency-bound) coarse-level sweep kernels first; the near-field work fills the rest of the GPU.
+// the (small, latency-bound) coarse-level sweep kernels first; the near-field work fills the rest of the GPU. The plain
+// form and the adjoint exchange the two: their near field is persistent and has the side stream (see enqueue_forward).
 #include <algorithm>
 #include <cerrno>
 #include <cmath>
@@ -62,7 +63,7 @@ struct fmm_ctx {
     const long long *ext_cnt = nullptr;
     cudaStream_t stream = nullptr;  // caller's stream
     cudaStream_t exec = nullptr;    // internal stream used for graph capture / replay
-    cudaStream_t side = nullptr;    // high-priority stream of the multipole sweep
+    cudaStream_t side = nullptr;    // high-priority stream: the sweep, or the plain form's near field
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_status = nullptr, ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t ev_t[8] = {};
     int timing = 0, count_pairs = 0, use_graph = 0;

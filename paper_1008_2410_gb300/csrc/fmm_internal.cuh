@@ -50,7 +50,7 @@ struct SysDev {
     int depth;
     int explicit_domain;
     int n64_kmh, n64_kml;           // plain form's near field (near64.cu), packed by derive_near64
-    // derived once per evaluation by k_domain_finalize (so no per-particle kernel divides in FP64)
+    // derived once per evaluation by the domain kernels (so no per-particle kernel divides in FP64)
     double scale;                   // 2^L / S
     double xe, ye;                  // x0 + S, y0 + S
     double wl;                      // S / 2^L, leaf width

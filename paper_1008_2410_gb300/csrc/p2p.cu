@@ -1208,7 +1208,7 @@ __device__ __forceinline__ void sym_store(const Work &w, f2 su_cu, f2 sv_cv, int
 // ordered: persistent blocks take leaves from counters in the order of falling work. Those of more than a part of a
 // warp's share of all work (and of SYM_MIN_WORK) take a block each: the densest leaf would bound the kernel else. Then
 // each warp takes leaves of its own. Otherwise (few leaves) every leaf has a block of its own.
-// Issue bound where it is large (2^21 particles in 8 patches at depth 8: 66% of the issue slots; 64 registers with
+// Issue bound where it is large (2^21 particles in 8 patches at depth 8: 63% of the issue slots; 64 registers with
 // spills around the chunks for 32 resident warps are 5% faster than 80 for 24). Evaluation in a graph, us, a warp per
 // leaf in leaf order / now: 8 patches of 2^24 particles at depth 9 28500 / 25600, 2^21 at depth 8 2920 / 2430, 2^20 at
 // depth 7 7800 / 2200, 300000 at depth 6 5990 / 1130; uniform 2^20 at depth 7 612 / 612, 2^18 at depth 6 198 / 201,
