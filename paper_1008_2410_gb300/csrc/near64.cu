@@ -635,9 +635,9 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
         auto pair64 = [&](int q) {
             const int j = R.global(q);
             const double a = xt - w.sx[j], b = yt - w.sy[j];
-            const double x = fma(a, a, b * b) * k2;
-            if (__double_as_longlong(x) == 0)
-                return;  // a particle and itself, or coincident ones
+            const double r2 = fma(a, a, b * b), x = r2 * k2;
+            if (__double_as_longlong(r2) == 0)
+                return;  // a particle and itself, or coincident ones: K and its Jacobian count as zero
             double f, h;     // f / k2 and 2 f' / k2
             if (x < kXCut) {
                 const int i = blob_row(x);
@@ -723,6 +723,12 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
                 const int4 p = pos[q];
                 const int dxh = tx.x - p.x, dyh = ty.x - p.z;
                 const int2 X = close_limbs(dxh, tx.y - p.y, cl.s), Y = close_limbs(dyh, ty.y - p.w, cl.s);
+                if ((X.x | X.y | Y.x | Y.y) == 0) {
+                    // the same fixed-point position: the Jacobian counts as zero where the FP64 positions are equal too
+                    if (R.global(q0 + q) != tpos)
+                        pair64(q0 + q);
+                    return;
+                }
                 const long long sxx = square_hi(X), syy = square_hi(Y), sxy = mul_hi(X.x, X.y, Y.x, Y.y);
                 if (max(abs(dxh), abs(dyh)) >= cl.lim || __mulhi(hi_bal(sxx + syy), cl.kmh) >= vmax) {
                     pair64(q0 + q);  // leaves so wide that far pairs are listed too
