@@ -78,7 +78,7 @@ struct Near64 {
     double k2;         // 1 / 2 sigma^2
     int ku;            // lengths in units of 2^ku: two leaf widths are at most 2^61 of them
     int thr;           // pairs whose r^2 has a high word (units of 2^94) of at least thr are far; 0: all run as close ones
-    int s, lim;        // close displacements are taken times 2^s (at most 2^62): high limbs below lim
+    int s, lim;        // close displacements are taken times 2^s (at most 2^62): high limbs below lim, 0: all in FP64
     int e, kmh, kml;   // z = x 2^56 = (r2 km 2^-64) 2^e, r2 = r^2 2^-64 in those units
     int vmax;          // high word of z 2^-e at the end of the tables
     bool ranges;       // lengths whose squares and their ratios stay well inside FP64's range
@@ -116,10 +116,12 @@ __host__ __device__ inline void derive_near64(SysDev &d)
     if (xr > 0.99 * N64_XMAX && cut < 0x1p30)
         d.n64_thr = (int)cut + 2 > N64_RMIN ? (int)cut + 2 : N64_RMIN;
     // close pairs are up to sqrt(2 N64_XCUT) sigma apart (below 2^(62 - s) units, s >= 1 in leaves wider than 5.4 sigma);
-    // without the list |dx| is at most 2^61 units. Leaves wider than 2^30 of that take FP64 (s = 31).
+    // without the list |dx| is at most 2^61 units. A displacement is exact to 2^s of its units at most (positions next
+    // to a coordinate axis have bits below them), which a product holds 2^3 of: in leaves wider than about 100 sigma
+    // (s > 4), where few pairs are close, those take FP64 (s = 31).
     const int lr = d.n64_thr > 0 ? exponent_of(8.67 * d.sigma) + 1 - ku : 61;
     int s = 62 - lr > 1 ? 62 - lr : 1;
-    s = s > 30 ? 31 : s;
+    s = s > 4 ? 31 : s;
     const int ek = exponent_of(k2) + 1;  // k2 = m 2^ek, m in [1/2, 1); km = m 2^62
     const long long km = (long long)ldexp(k2, 62 - ek);
     d.n64_kmh = (int)(km >> 32);

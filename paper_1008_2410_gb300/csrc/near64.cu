@@ -1,15 +1,18 @@
 // near64.cu -- Fig. 1 stage 9 in the plain form: the near field of Eq. 6 in (at least) FP64 accuracy.
 //
 // GB300 has 2 FP64 multiply-adds per SM and clock against 128 in FP32 and 30 wide (32 x 32 -> 64) integer ones, so
-// the pairs run in 64-bit fixed point on the integer pipe: coordinates as exact integers (their differences carry no
-// rounding error), products from three wide multiplications each, sums in 64-bit integers.
+// the pairs run in 64-bit fixed point on the integer pipe: coordinates as integers in units of 2^-60 of a leaf's width
+// (FP64 positions exactly, but for those within 2^-7 widths of a coordinate axis: differences carry no other rounding
+// error), products from three wide multiplications each, sums in 64-bit integers.
 //   * r > sqrt(75) sigma (x = r^2 / 2 sigma^2 > 37.5): 1 - e^-x is 1 in FP64 and the pair is the point vortex
 //     gamma (-dy, dx) / r^2, with 1 / r^2 by one Newton step of second order from the SFU's FP32 reciprocal.
 //   * closer pairs go to a list per thread (index in shared memory) and run once the list is full or the sources are
 //     done, every lane with a pair of its own: F(x) = (1 - e^-x) / x from a table of polynomials of degree 5 (no
 //     exponential, no division). Where nearly every adjacent pair is close, all take this path, without the list.
 // A block whose charges span a wide range (so that a fixed unit could lose digits of a small sum) or that has few
-// sources runs all pairs in FP64, with a table of polynomials of degree 6.
+// sources runs all pairs in FP64, with a table of polynomials of degree 6; so do close pairs in leaves wider than about
+// 100 sigma. A target whose sums turn out small against the fixed unit (its velocity is that of weak charges among strong
+// ones without weight there, or of particles much closer together than sigma) is summed in FP64 instead.
 #include <math.h>
 
 #include <mutex>
@@ -341,12 +344,55 @@ struct Acc64 {
         }
         return fma((double)(h + (int)(a >> 63)), 0x1p64, (double)(long long)a);
     }
+    // thread t's sum in magnitude, in units of 2^32 (to 2^-24 of it or 2^8); 0 only if it is zero
+    __device__ __forceinline__ float size(int t) const
+    {
+        const unsigned long long l = lo[t];
+        const int h = hi[t];
+        return fmaxf(fabsf(fmaf((float)h, 0x1p32f, (float)(unsigned)(l >> 32))), (l | (unsigned)h) != 0 ? 1.0f : 0.0f);
+    }
 };
 constexpr size_t N64_SMEM = N64_TILE * 24 + 4 * sizeof(Acc64) + N64_CAP * N64_THREADS * 2;
 
+// The line below which a target's far and near sums are too small: the larger of those of the kinds that take part.
+__device__ __forceinline__ float line_of(float far, float near, float far_line, float near_line)
+{
+    const bool none = far == 0.0f && near == 0.0f;
+    return fmaxf(far != 0.0f || none ? far_line : 0.0f, near != 0.0f || none ? near_line : 0.0f);
+}
+
+// Source j in FP64: au, av in units of k2.
+__device__ __forceinline__ void near_pair(const Work &w, int j, double xt, double yt, double k2, double &au, double &av)
+{
+    const double ax = xt - w.sx[j], ay = yt - w.sy[j];
+    const double x = fma(ax, ax, ay * ay) * k2;
+    double f = x < kXCut ? blob_poly(g_blob_f, blob_row(x), x) : recip64(x);
+    // a particle and itself, or coincident ones: nothing, whatever the charge
+    f = __double_as_longlong(x) != 0 ? f * w.sg[j] : 0.0;
+    au = fma(-ay, f, au);
+    av = fma(ax, f, av);
+}
+
+// The sum of v over the block, added in a fixed order; for thread 0. red: 2 x 8 values.
+__device__ __forceinline__ double block_sum(double v, double *red)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();  // red is free
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0.0;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < N64_THREADS / 32; ++i)
+            v += red[i];
+    return v;
+}
+
 __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 {
-    __shared__ int s_leaf;
+    __shared__ int s_leaf, s_weak;
     extern __shared__ __align__(16) unsigned char sm[];  // N64_SMEM bytes
     int4 *pos = reinterpret_cast<int4 *>(sm);                        // x and y limbs
     int2 *gam = reinterpret_cast<int2 *>(pos + N64_TILE);            // gamma limbs, base 2^32
@@ -393,16 +439,7 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
         double au = 0.0, av = 0.0;    // FP64 pairs: sums of gamma F(x) (-dy, dx), in units of k2
         for (int q = 0; q < 4; ++q)
             acc[q].clear(tid);        // pairs in fixed point
-        auto pair64 = [&](int q) {
-            const int j = R.global(q);
-            const double ax = xt - w.sx[j], ay = yt - w.sy[j];
-            const double x = fma(ax, ax, ay * ay) * k2;
-            double f = x < kXCut ? blob_poly(g_blob_f, blob_row(x), x) : recip64(x);
-            // a particle and itself, or coincident ones: nothing, whatever the charge
-            f = __double_as_longlong(x) != 0 ? f * w.sg[j] : 0.0;
-            au = fma(-ay, f, au);
-            av = fma(ax, f, av);
-        };
+        auto pair64 = [&](int q) { near_pair(w, R.global(q), xt, yt, k2, au, av); };
         if (!ranges) {
             if (active)
                 for (int q = grp; q < ntot; q += G) {
@@ -524,11 +561,16 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
         }
         // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double2 *red = reinterpret_cast<double2 *>(pos);
+        if (tid == 0)
+            s_weak = 0;
         const bool some64 = __syncthreads_or(au != 0.0 || av != 0.0);
-        if (some64) {
+        if (some64)
             red[tid] = make_double2(au, av);
-            __syncthreads();
-        }
+        float2 *sizes = reinterpret_cast<float2 *>(lst);
+        unsigned short *weak = lst + 4 * N64_THREADS;
+        if (fixed)
+            sizes[tid] = make_float2(fmaxf(acc[0].size(tid), acc[1].size(tid)), fmaxf(acc[2].size(tid), acc[3].size(tid)));
+        __syncthreads();
         if (tid < cp) {
             double u = 0.0, v = 0.0;
             for (int g = 0; some64 && g < G; ++g) {
@@ -543,10 +585,37 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             if (fixed) {
                 // a far term is gamma dx / r^2 2^(51 + ku - ka), a close one gamma F dx 2^(s - 66 - ku - ka)
                 const double gs = pow2(ka), fs = pow2(-51 - ku), cs = k2 * pow2(66 - cl.s + ku);
+                // A term's rounding is about 0.4 of its unit (fs or cs, times gs) however small the term is, in FP64 it is
+                // relative to it: a target whose sums are all small against the unit, because the strong sources have no
+                // weight there, is left to FP64 below. At this line the two errors are about the same; the sums of groups
+                // of sources stand for the terms, so that a velocity that is small by cancellation does not count.
+                float2 sz = sizes[tid];
+                for (int g = 1; g < G; ++g) {
+                    const float2 q = sizes[tid + g * cp];
+                    sz = make_float2(fmaxf(sz.x, q.x), fmaxf(sz.y, q.y));
+                }
+                // (next to a coordinate axis a position is short of 2^(s - 3) units as well)
+                const float ratio = cl.lim ? (float)(k2 * pow2(117 - cl.s + 2 * ku)) : 0.0f;  // cs / fs
+                const float line = line_of(sz.x, sz.y, 0x1p20f, ratio * (cl.s > 3 ? 0x1p21f : (thr ? 0x1p20f : 0x1p21f)));
+                if (fmaxf(sz.x, sz.y * ratio) < line && (!some64 || fmax(fabs(u), fabs(v)) < line * 0x1p32 * fs * gs))
+                    weak[atomicAdd(&s_weak, 1)] = (unsigned short)tid;
                 u -= fma(acc[2].total(tid, cp, G), cs, acc[0].total(tid, cp, G) * fs) * gs;
                 v += fma(acc[3].total(tid, cp, G), cs, acc[1].total(tid, cp, G) * fs) * gs;
             }
             w.near64[tpos] = make_double2(u / kTwoPi, v / kTwoPi);
+        }
+        __syncthreads();
+        const int nweak = s_weak;
+        for (int e = 0; e < nweak; ++e) {  // the whole block on each weak target
+            const int t = s0 + t0 + weak[e];
+            const double xw = w.sx[t], yw = w.sy[t];
+            double bu = 0.0, bv = 0.0;
+            for (int q = tid; q < ntot; q += N64_THREADS)
+                near_pair(w, R.global(q), xw, yw, k2, bu, bv);
+            bu = block_sum(bu, &red->x);
+            bv = block_sum(bv, &red->x);
+            if (tid == 0)
+                w.near64[t] = make_double2(bu * k2 / kTwoPi, bv * k2 / kTwoPi);
         }
         __syncthreads();
     }

@@ -40,3 +40,92 @@ def test_adjoint_of_coincident_particles(lib, oracle, sigma, copies):
     for a, b in zip(got, ref):
         a, b = a.cpu().numpy()[same.ravel()], b[same.ravel()]
         assert np.linalg.norm(a - b) < 1e-11 * np.linalg.norm(b)
+
+
+# ---------------------------------------------------------------- each particle against direct sums in long double
+
+Q = np.longdouble
+TWO_PI = 2 * Q("3.14159265358979323846264338327950288")
+
+
+def blob(x):
+    """F(x) = (1 - e^-x) / x and F'(x): Taylor series below 1, the formulas from there on."""
+    F, D = np.zeros_like(x), np.zeros_like(x)
+    m = x < 1
+    t = np.ones_like(x[m])  # (-x)^k / (k + 1)!
+    for k in range(40):
+        F[m] += t
+        D[m] -= t * (k + 1) / (k + 2)
+        t = t * -x[m] / (k + 2)
+    X = x[~m]
+    F[~m] = (1 - np.exp(-X)) / X
+    D[~m] = ((1 + X) * np.exp(-X) - 1) / (X * X)
+    return F, D
+
+
+def pairs(w):
+    """Displacements, F k2 and 2 F' k2^2 of every pair (targets by rows); zero for coincident ones. Depth 1: all near."""
+    x, y = w.x.astype(Q), w.y.astype(Q)
+    a, b = x[:, None] - x[None, :], y[:, None] - y[None, :]
+    k2 = 1 / (2 * Q(w.sigma) ** 2)
+    F, D = blob(((a * a + b * b) * k2).ravel())
+    F, D = F.reshape(a.shape) * k2, D.reshape(a.shape) * 2 * k2 * k2
+    same = (a == 0) & (b == 0)
+    F[same] = D[same] = 0
+    return a, b, F, D
+
+
+def bound(n):
+    """An FP64 sum of n terms, each within a few 2^-53 of its size, is off by less than (n + 8) 2^-53 sum |terms|."""
+    return (n + 8) * 2.0 ** -53 / (2 * np.pi)
+
+
+def close_to_axes(ratio, spread):
+    """300 particles within a few spread * sigma of the origin, leaves of width 1 / 8 = sigma / ratio."""
+    r = fi.rng(142)
+    w = fi.uniform(300, seed_index=143, depth=1, p=4, sigma=0.125 * ratio)
+    w.x, w.y = (spread * w.sigma * r.standard_normal(w.n) for _ in range(2))
+    w.domain = (-0.125, -0.125, 0.25)
+    return w
+
+
+def weak_around_strong(weak, apart, sigma=1 / 32):
+    """Two particles of charge 1, apart * sigma from each other, among 574 of the order of weak."""
+    w = fi.uniform(576, seed_index=144, depth=1, p=4, sigma=sigma)
+    w.gamma = weak * fi.rng(145).standard_normal(w.n)
+    w.gamma[:2] = 1.0
+    w.x[1], w.y[1] = w.x[0] + apart * w.sigma, w.y[0]
+    return w
+
+
+EXACT = [
+    ("uniform", lambda: fi.uniform(1500, seed_index=146, depth=1, p=4)),
+    ("axes_16", lambda: close_to_axes(1 / 16, 2.0)),
+    ("axes_16_tight", lambda: close_to_axes(1 / 16, 1e-4)),
+    ("axes_60", lambda: close_to_axes(1 / 60, 2.0)),
+    ("axes_60_tight", lambda: close_to_axes(1 / 60, 1e-2)),
+    ("axes_500", lambda: close_to_axes(2e-3, 2.0)),
+    ("axes_1e5", lambda: close_to_axes(1e-5, 2.0)),
+    ("axes_1e7", lambda: close_to_axes(1e-7, 2.0)),
+    ("axes_1e9", lambda: close_to_axes(1e-9, 2.0)),
+    ("weak_1e-9", lambda: weak_around_strong(1e-9, 0.0)),
+    ("weak_1e-12", lambda: weak_around_strong(1e-12, 0.0)),
+    ("weak_1e-12_apart", lambda: weak_around_strong(1e-12, 1e-8)),
+    ("weak_1e-9_narrow", lambda: weak_around_strong(1e-9, 0.0, sigma=0.2)),
+]
+
+
+@pytest.mark.parametrize("name,make", EXACT, ids=[c[0] for c in EXACT])
+def test_each_velocity(lib, name, make):
+    w = make()
+    f = lib.FMM(w.depth, w.p, w.sigma, precision="fp64", domain=w.domain)
+    u, v = (t.cpu().numpy() for t in f.velocity_near(dev(w.x), dev(w.y), dev(w.gamma)))
+    f.sync()
+    a, b, F, _ = pairs(w)
+    g = w.gamma.astype(Q)
+    tu, tv = -b * F * g, a * F * g
+    err = np.maximum(abs(u - tu.sum(1) / (TWO_PI)), abs(v - tv.sum(1) / (TWO_PI)))
+    size = np.maximum(abs(tu).sum(1), abs(tv).sum(1))
+    worst = float((err / size).max())
+    print(f"{name}: {worst / bound(w.n):.2e} of the bound")
+    assert worst < bound(w.n)
