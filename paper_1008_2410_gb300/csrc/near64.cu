@@ -87,15 +87,13 @@ const double2 *g_tab_f[64];  // device address of g_blob_f
 
 // ------------------------------------------------------------------ fixed point
 
-// round(v * 2^-k) modulo 2^64 (v = 0 for zeros and subnormals).
+// round(v * 2^-k) modulo 2^64.
 __device__ __forceinline__ long long to_fixed(double v, int k)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const int be = (int)((b >> 52) & 0x7ff);
-    if (be == 0)
-        return 0;
-    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
-    const int sh = be - 1075 - k;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (be ? 1ull << 52 : 0ull);
+    const int sh = max(be, 1) - 1075 - k;
     unsigned long long r;
     if (sh >= 0)
         r = sh < 64 ? m << sh : 0ull;
@@ -903,13 +901,12 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             }
             if (fixed) {
                 // sums in units of 2^40: far a / r^2 2^(119 + ku) per ca, close F 2^62 in units of k2, a 2^(s - ku);
-                // charges 2^-ka and 2^-kb, the target's 2^tau up
-                const double sa = pow2(ka) * pow2(-tau), sb = pow2(kb);
-                out[0] += fma(acc[3].total(tid, cp, G), k2 * pow2(42 - cl.s + ku), acc[0].total(tid, cp, G) * pow2(-79 - ku)) * sb;
+                // charges 2^-ka and 2^-kb, the target's 2^tau up (in one exponent: 2^(ka - tau) alone may be below FP64's range)
+                out[0] += ldexp(fma(acc[3].total(tid, cp, G), k2 * pow2(42 - cl.s + ku), acc[0].total(tid, cp, G) * pow2(-79 - ku)), kb);
 #pragma unroll
                 for (int q = 1; q < 3; ++q)
-                    out[q] += fma(acc[3 + q].total(tid, cp, G), k2 * 0x1p42,
-                                  acc[q].total(tid, cp, G) * pow2(-70 - 2 * ku)) * sa * sb;
+                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, G), k2 * 0x1p42, acc[q].total(tid, cp, G) * pow2(-70 - 2 * ku)),
+                                    ka + kb - tau);
             }
             const int i = w.perm[tpos];
             if (odg)

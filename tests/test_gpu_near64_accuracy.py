@@ -129,3 +129,27 @@ def test_each_velocity(lib, name, make):
     worst = float((err / size).max())
     print(f"{name}: {worst / bound(w.n):.2e} of the bound")
     assert worst < bound(w.n)
+
+
+def test_gradient_of_charges_far_from_one(lib):
+    """Charges of 1e-188 with gradients of 1e200; every tenth target 1e-119 times as strong in both (its charge times the
+    unit of the others' is below FP64's range, its gradient is not). Tolerance 1e-11 relative L2 over those, as for the
+    other adjoint tests (the same sums, scaled)."""
+    w = fi.uniform(1500, seed_index=148, depth=1, p=4)
+    r = fi.rng(149)
+    g, gu, gv = r.standard_normal((3, w.n))
+    s = np.ones(w.n)
+    s[::10] = 1e-119
+    f = lib.FMM(w.depth, w.p, w.sigma, precision="fp64", domain=w.domain)
+    got = [t.cpu().numpy() for t in f.adjoint(dev(w.x), dev(w.y), dev(g * s * 1e-188), dev(gu * s * 1e200), dev(gv * s * 1e200))]
+    f.sync()
+    a, b, F, D = pairs(w)
+    g, gu, gv = (t.astype(Q) * s for t in (g, gu, gv))
+    cu = g[None, :] * gu[:, None] - g[:, None] * gu[None, :]
+    cv = g[None, :] * gv[:, None] - g[:, None] * gv[None, :]
+    J1, J2, ab = F + b * b * D, F + a * a * D, a * b * D
+    ref = (F * (gu[None, :] * b - gv[None, :] * a)).sum(1), (cv * J2 - cu * ab).sum(1), (cv * ab - cu * J1).sum(1)
+    # in units of 1e200 (dgamma), 1e-188 1e200 1e-119 = 1e-107 (dx, dy of the weak targets)
+    for q, t, unit, strength in zip(got, ref, (1e200, 1e-107, 1e-107), (1.0, 1e-119, 1e-119)):
+        q, t = q[::10] / unit, t[::10] / strength / TWO_PI
+        assert np.linalg.norm((q - t).astype(float)) < 1e-11 * np.linalg.norm(t.astype(float))
