@@ -350,6 +350,13 @@ struct Acc64 {
         return fmaxf(fabsf(fmaf((float)h, 0x1p32f, (float)(unsigned)(l >> 32))), (l | (unsigned)h) != 0 ? 1.0f : 0.0f);
     }
 };
+// v, without the compiler's knowledge that it is the same in every pass: what is derived from it is not kept in registers
+// through the loops over the sources (in the adjoint 3% of the kernel).
+__device__ __forceinline__ int fresh(int v)
+{
+    asm volatile("" : "+r"(v));
+    return v;
+}
 constexpr size_t N64_SMEM = N64_TILE * 24 + 4 * sizeof(Acc64) + N64_CAP * N64_THREADS * 2;
 
 // The line below which a target's far and near sums are too small: the larger of those of the kinds that take part.
@@ -622,6 +629,42 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 
 // ------------------------------------------------------------------ adjoint
 
+__device__ __forceinline__ unsigned position_hash(double x, double y)  // the same for 0 and -0
+{
+    const unsigned long long a = (unsigned long long)__double_as_longlong(x), b = (unsigned long long)__double_as_longlong(y);
+    const unsigned ah = (a << 1) ? (unsigned)(a >> 32) : 0u, bh = (b << 1) ? (unsigned)(b >> 32) : 0u;
+    return (((unsigned)a * 0x9e3779b1u + ah) * 0x85ebca77u + (unsigned)b) * 0xc2b2ae3du + bh;
+}
+
+// A particle of the adjoint, and its pair with source j in FP64: g (dgamma), x and y (dx, dy) in units of k2.
+struct Adj64 {
+    double x, y, g, gu, gv;
+    __device__ __forceinline__ Adj64(const Work &w, int t) : x(w.sx[t]), y(w.sy[t]), g(w.sg[t]), gu(w.sgu[t]), gv(w.sgv[t]) {}
+    __device__ __forceinline__ void pair(const Work &w, int j, double k2, double &ag, double &ax, double &ay) const
+    {
+        const double a = x - w.sx[j], b = y - w.sy[j];
+        const double r2 = fma(a, a, b * b), xx = r2 * k2;
+        if (__double_as_longlong(r2) == 0)
+            return;  // a particle and itself, or coincident ones: K and its Jacobian count as zero
+        double f, h;     // f / k2 and 2 f' / k2
+        if (xx < kXCut) {
+            const int i = blob_row(xx);
+            f = blob_poly(g_blob_f, i, xx);
+            h = 2.0 * k2 * blob_poly(g_blob_d, i, xx);
+        } else {
+            f = recip64(xx);
+            h = -2.0 * k2 * (f * f);
+        }
+        const double gj = w.sg[j], guj = w.sgu[j], gvj = w.sgv[j];
+        const double ah = a * h, bh = b * h, ab = a * bh;
+        const double J2 = fma(a, ah, f), J1 = fma(b, bh, f);  // dKv/da, -dKu/db; dKv/db = -dKu/da = ab
+        const double cu = gj * gu - g * guj, cv = gj * gv - g * gvj;
+        ag = fma(f, guj * b - gvj * a, ag);
+        ax += fma(cv, J2, -cu * ab);  // one rounding at the size of the sum
+        ay += fma(cv, ab, -cu * J1);
+    }
+};
+
 // For target k and neighbour m (z = (a, b) = z_k - z_m), with K = (Ku, Kv) = (-b, a) f of Eq. 6 and its Jacobian J:
 //   dgamma_k += -(gu_m Ku + gv_m Kv) = f (gu_m b - gv_m a)
 //   dx_k     += cu dKu/da + cv dKv/da,  cu = gamma_m gu_k - gamma_k gu_m
@@ -633,11 +676,13 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 // FP64). Measured at 2^20 uniform particles (leaves of 64, 16 sigma wide): 103 ms with exp, expm1 and divisions in FP64
 // for every pair; the whole adjoint (near field beside both sweeps) 108 ms then, 8.9 ms now. 112 or 128 registers keep
 // the sweeps' blocks out (11.6 to 12.0 ms), 80 spill (10.9). Errors against quad precision are below the former ones.
-// Writes the near part in caller order (the far part is added later).
+// Writes the near part in caller order (the far part is added later). Targets for whom the fixed unit is too coarse, or
+// with coincident particles, are listed in slot (free after the binning) for k_adjoint_weak64.
 constexpr int A64_REGS = 96, A64_B = 2;  // registers a thread, blocks an SM: room for the sweep's blocks beside them
 constexpr int A64_TILE = 640;
 constexpr int A64_CAP = 48;  // terms between two hand-overs to the 96-bit sums
 constexpr size_t A64_SMEM = A64_TILE * 40 + 6 * sizeof(Acc64) + A64_CAP * N64_THREADS * 2;
+
 __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double *__restrict__ odg,
                                                                                 double *__restrict__ odx,
                                                                                 double *__restrict__ ody, int skip_plain)
@@ -650,6 +695,8 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
     unsigned short *lst = reinterpret_cast<unsigned short *>(acc + 6);
     __shared__ Stats64 st;
     __shared__ int s_leaf;
+    __shared__ float4 s_line;
+    __shared__ unsigned char s_same[N64_THREADS];  // whether the thread's target has a coincident particle
     const int tid = threadIdx.x;
     if (skip_plain && w.nsys == 1 && !(w.sys[0].s_unit > P2P_SPLIT_S))
         return;  // the only system's near field is the FP32 kernel's
@@ -687,6 +734,12 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
         fixed = eb != kNoFixed;
         ka = ea - 62;
         kb = eb - 58;
+        if (tid == 0) {  // cg / fg, the close sums' line, cx / fx, the line (see the sums' end)
+            const float axis = cl.s > 3 ? 2.0f : 1.0f;
+            const float rg = cl.lim ? (float)(k2 * pow2(121 - cl.s + 2 * ku)) : 0.0f;
+            const float rx = cl.lim ? (float)(k2 * pow2(112 + 2 * ku)) : 0.0f;
+            s_line = make_float4(rg, axis * rg * (thr ? 0x1p39f : 0x1p43f), rx, axis * rx * (thr ? 0x1p40f : 0x1p42f));
+        }
     }
     const int npass = pick_passes(c);
     for (int pass = 0; pass < npass; ++pass) {
@@ -694,34 +747,13 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
         const int G = N64_THREADS / cp;
         const int grp = tid / cp, tpos = s0 + t0 + (tid - grp * cp);
         const bool active = grp < G;
-        const double xt = w.sx[tpos], yt = w.sy[tpos], gt = w.sg[tpos], gut = w.sgu[tpos], gvt = w.sgv[tpos];
+        const Adj64 me(w, tpos);
+        const double xt = me.x, yt = me.y, gt = me.g, gut = me.gu, gvt = me.gv;
         for (int q = 0; q < 6; ++q)
             acc[q].clear(tid);
         int tau = 0;
         double ag = 0.0, ax = 0.0, ay = 0.0;  // FP64 pairs: dgamma in units of k2, dx and dy in units of k2
-        auto pair64 = [&](int q) {
-            const int j = R.global(q);
-            const double a = xt - w.sx[j], b = yt - w.sy[j];
-            const double r2 = fma(a, a, b * b), x = r2 * k2;
-            if (__double_as_longlong(r2) == 0)
-                return;  // a particle and itself, or coincident ones: K and its Jacobian count as zero
-            double f, h;     // f / k2 and 2 f' / k2
-            if (x < kXCut) {
-                const int i = blob_row(x);
-                f = blob_poly(g_blob_f, i, x);
-                h = 2.0 * k2 * blob_poly(g_blob_d, i, x);
-            } else {
-                f = recip64(x);
-                h = -2.0 * k2 * (f * f);
-            }
-            const double gj = w.sg[j], guj = w.sgu[j], gvj = w.sgv[j];
-            const double ah = a * h, bh = b * h, ab = a * bh;
-            const double J2 = fma(a, ah, f), J1 = fma(b, bh, f);  // dKv/da, -dKu/db; dKv/db = -dKu/da = ab
-            const double cu = gj * gut - gt * guj, cv = gj * gvt - gt * gvj;
-            ag = fma(f, guj * b - gvj * a, ag);
-            ax += fma(cv, J2, -cu * ab);  // one rounding at the size of the sum
-            ay += fma(cv, ab, -cu * J1);
-        };
+        auto pair64 = [&](int q) { me.pair(w, R.global(q), k2, ag, ax, ay); };
         if (!ranges) {
             if (active)
                 for (int q = grp; q < ntot; q += G) {
@@ -755,6 +787,23 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             // cu and cv are linear in the target's charges: scaled up together, so that a weak target keeps its digits
             const int te = max(exponent_of(gt) - (ka + 61), max(exponent_of(gut), exponent_of(gvt)) - (kb + 57));
             tau = te < -900 ? 0 : -te;
+            // Coincident particles (whose Jacobian counts as zero) are of one leaf. Looking for them here, by hashes of the
+            // positions, costs nothing that shows; a test in the loop over the close pairs 2.5% of the kernel.
+            unsigned *hash = reinterpret_cast<unsigned *>(lst);
+            constexpr int kHashes = A64_CAP * N64_THREADS / 2;
+            const unsigned mine = position_hash(xt, yt);
+            bool same = false;
+            const int own = fresh(leaf), own1 = w.start[own + 1];
+            for (int h0 = w.start[own]; h0 < own1; h0 += kHashes) {
+                const int m = min(kHashes, own1 - h0);
+                __syncthreads();
+                for (int j = tid; j < m; j += N64_THREADS)
+                    hash[j] = position_hash(w.sx[h0 + j], w.sy[h0 + j]);
+                __syncthreads();
+                for (int j = active ? grp : m; j < m; j += G)
+                    same |= hash[j] == mine && h0 + j != tpos;
+            }
+            s_same[tid] = same;
             const long long tg = to_fixed(gt, ka - tau), tgu = to_fixed(gut, kb - tau), tgv = to_fixed(gvt, kb - tau);
             const int tgh = -hi_bal(tg), tgl = (int)lo_of(tg) >> 1;  // low limb halved: it can be negated
             const int tuh = hi_bal(tgu), tul = (int)lo_of(tgu), tvh = hi_bal(tgv), tvl = (int)lo_of(tgv);
@@ -790,12 +839,6 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
                 const int4 p = pos[q];
                 const int dxh = tx.x - p.x, dyh = ty.x - p.z;
                 const int2 X = close_limbs(dxh, tx.y - p.y, cl.s), Y = close_limbs(dyh, ty.y - p.w, cl.s);
-                if ((X.x | X.y | Y.x | Y.y) == 0) {
-                    // the same fixed-point position: the Jacobian counts as zero where the FP64 positions are equal too
-                    if (R.global(q0 + q) != tpos)
-                        pair64(q0 + q);
-                    return;
-                }
                 const long long sxx = square_hi(X), syy = square_hi(Y), sxy = mul_hi(X.x, X.y, Y.x, Y.y);
                 if (max(abs(dxh), abs(dyh)) >= cl.lim || __mulhi(hi_bal(sxx + syy), cl.kmh) >= vmax) {
                     pair64(q0 + q);  // leaves so wide that far pairs are listed too
@@ -888,8 +931,12 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             red[tid] = ag;
             red[N64_THREADS + tid] = ax;
             red[2 * N64_THREADS + tid] = ay;
-            __syncthreads();
         }
+        float4 *sizes = reinterpret_cast<float4 *>(lst);  // far and close sums of dgamma, of dx and dy
+        if (fixed)
+            sizes[tid] = make_float4(acc[0].size(tid), acc[3].size(tid), fmaxf(acc[1].size(tid), acc[2].size(tid)),
+                                     fmaxf(acc[4].size(tid), acc[5].size(tid)));
+        __syncthreads();
         if (tid < cp) {
             double out[3] = {0.0, 0.0, 0.0};
 #pragma unroll
@@ -902,11 +949,30 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             if (fixed) {
                 // sums in units of 2^40: far a / r^2 2^(119 + ku) per ca, close F 2^62 in units of k2, a 2^(s - ku);
                 // charges 2^-ka and 2^-kb, the target's 2^tau up (in one exponent: 2^(ka - tau) alone may be below FP64's range)
-                out[0] += ldexp(fma(acc[3].total(tid, cp, G), k2 * pow2(42 - cl.s + ku), acc[0].total(tid, cp, G) * pow2(-79 - ku)), kb);
+                const int kq = fresh(ku);
+                const double fg = pow2(-79 - kq), cg = k2 * pow2(42 - cl.s + kq), fx = pow2(-70 - 2 * kq), cx = k2 * 0x1p42;
+                // A target whose sums are all small against the rounding of their terms is left to FP64 (as in k_near64): a
+                // far pair's dgamma is off by 2^20 (the charges' last bits, the low halves left out), its gradient by 2^16
+                // (P and Q); a close pair's by about 2^18 and 2^19, by up to 2^21 where all pairs are close. So is one with a
+                // coincident particle.
+                float4 sz = sizes[tid];
+                for (int g = 1; g < G; ++g) {
+                    const float4 q = sizes[tid + g * cp];
+                    sz = make_float4(fmaxf(sz.x, q.x), fmaxf(sz.y, q.y), fmaxf(sz.z, q.z), fmaxf(sz.w, q.w));
+                }
+                const float4 line = s_line;
+                const float lg = line_of(sz.x, sz.y, 0x1p43f, line.y), lx = line_of(sz.z, sz.w, 0x1p39f, line.w);
+                bool small = fmaxf(sz.x, sz.y * line.x) < lg;
+                if (gt != 0.0 || gut != 0.0 || gvt != 0.0)
+                    small |= fmaxf(sz.z, sz.w * line.z) < lx;
+                for (int g = 0; g < G; ++g)
+                    small |= s_same[tid + g * cp] != 0;
+                if (small)
+                    w.slot[atomicAdd(&w.cnt[w.nleaf + 2], 1)] = tpos;
+                out[0] += ldexp(fma(acc[3].total(tid, cp, G), cg, acc[0].total(tid, cp, G) * fg), kb);
 #pragma unroll
                 for (int q = 1; q < 3; ++q)
-                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, G), k2 * 0x1p42, acc[q].total(tid, cp, G) * pow2(-70 - 2 * ku)),
-                                    ka + kb - tau);
+                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, G), cx, acc[q].total(tid, cp, G) * fx), ka + kb - tau);
             }
             const int i = w.perm[tpos];
             if (odg)
@@ -918,6 +984,38 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
         }
         __syncthreads();
     }
+    }
+}
+
+// The targets that k_adjoint_near64 has listed, in FP64: a block each. A kernel of its own, since in k_adjoint_near64 this
+// loop takes registers from the loops over the sources (the gradient of 2^20 uniform particles 13.33 ms so, 13.70 with the
+// loop there).
+__global__ void __launch_bounds__(N64_THREADS) k_adjoint_weak64(Work w, double *__restrict__ odg, double *__restrict__ odx,
+                                                                double *__restrict__ ody)
+{
+    __shared__ double red[N64_THREADS / 32];
+    const int n = w.cnt[w.nleaf + 2];
+    for (int e = blockIdx.x; e < n; e += gridDim.x) {
+        const int t = w.slot[e], leaf = w.sleaf[t];
+        const SysDev &d = w.sys[w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf)];
+        const Rows64 R(w, d, leaf);
+        const double k2 = near64_of(d).k2;
+        const Adj64 me(w, t);
+        double ag = 0.0, ax = 0.0, ay = 0.0;
+        for (int q = threadIdx.x; q < R.pre[3]; q += N64_THREADS)
+            me.pair(w, R.global(q), k2, ag, ax, ay);
+        ag = block_sum(ag, red);
+        ax = block_sum(ax, red);
+        ay = block_sum(ay, red);
+        if (threadIdx.x == 0) {
+            const int i = w.perm[t];
+            if (odg)
+                odg[i] = ag * k2 / kTwoPi;
+            if (odx)
+                odx[i] = ax * k2 / kTwoPi;
+            if (ody)
+                ody[i] = ay * k2 / kTwoPi;
+        }
     }
 }
 
@@ -1004,7 +1102,8 @@ int launch_adjoint_near64(const Work &w, double *dg, double *dx, double *dy, int
     const int resident = A64_B * kSMs;
     const int parts = max(1, min(8, resident / w.nleaf));
     k_adjoint_near64<<<min(w.nleaf * parts, resident), N64_THREADS, A64_SMEM, s>>>(w, parts, dg, dx, dy, skip_plain);
-    return 1;
+    k_adjoint_weak64<<<min(w.n, 4 * kSMs), N64_THREADS, 0, s>>>(w, dg, dx, dy);
+    return 2;
 }
 
 }  // namespace fmm

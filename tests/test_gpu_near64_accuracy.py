@@ -153,3 +153,30 @@ def test_gradient_of_charges_far_from_one(lib):
     for q, t, unit, strength in zip(got, ref, (1e200, 1e-107, 1e-107), (1.0, 1e-119, 1e-119)):
         q, t = q[::10] / unit, t[::10] / strength / TWO_PI
         assert np.linalg.norm((q - t).astype(float)) < 1e-11 * np.linalg.norm(t.astype(float))
+
+
+@pytest.mark.parametrize("grads", ["normal", "like_charges"])
+@pytest.mark.parametrize("name,make", EXACT, ids=[c[0] for c in EXACT])
+def test_each_gradient(lib, name, make, grads):
+    w = make()
+    r = fi.rng(147)
+    gu, gv = r.standard_normal(w.n), r.standard_normal(w.n)
+    if grads == "like_charges":  # strong and weak like gamma, of either sign
+        gu, gv = gu * abs(w.gamma), gv * abs(w.gamma)
+    f = lib.FMM(w.depth, w.p, w.sigma, precision="fp64", domain=w.domain)
+    got = [t.cpu().numpy() for t in f.adjoint(dev(w.x), dev(w.y), dev(w.gamma), dev(gu), dev(gv))]
+    f.sync()
+    a, b, F, D = pairs(w)
+    g, gu, gv = (t.astype(Q) for t in (w.gamma, gu, gv))
+    cu = g[None, :] * gu[:, None], g[:, None] * gu[None, :]
+    cv = g[None, :] * gv[:, None], g[:, None] * gv[None, :]
+    J1, J2, ab = F + b * b * D, F + a * a * D, a * b * D  # -dKu/db, dKv/da, dKv/db = -dKu/da
+    dg = F * (gu[None, :] * b - gv[None, :] * a)
+    dx = (cv[0] - cv[1]) * J2 - (cu[0] - cu[1]) * ab
+    dy = (cv[0] - cv[1]) * ab - (cu[0] - cu[1]) * J1
+    size_g = (F * (abs(gu[None, :] * b) + abs(gv[None, :] * a))).sum(1)
+    size_xy = ((abs(cu[0]) + abs(cu[1]) + abs(cv[0]) + abs(cv[1])) * (F + (a * a + b * b) * abs(D))).sum(1)
+    worst = [float((abs(q - t.sum(1) / TWO_PI) / s).max()) / bound(w.n)
+             for q, t, s in zip(got, (dg, dx, dy), (size_g, size_xy, size_xy))]
+    print(f"{name} {grads}: {worst} of the bound")
+    assert max(worst) < 1.0
