@@ -33,45 +33,73 @@ constexpr int kTabN = 600;
 constexpr double kXCut = N64_XCUT;
 __device__ double2 g_blob_f[kTabN * 4], g_blob_d[kTabN * 4];  // F and F'
 
-long double blob_f(long double x) { return x == 0.0L ? 1.0L : -expm1l(-x) / x; }
-
-// F'(x) = ((1 + x) e^-x - 1) / x^2, below 1.5 by its Taylor series sum_k (-1)^k k x^(k-1) / (k+1)!.
-long double blob_d(long double x)
+// Double-double numbers for the tables, h + l with |l| <= ulp(h) / 2 (Knuth's two-sum, products by fma): about 2^-102 relative.
+struct DD {
+    double h, l;
+};
+__device__ __forceinline__ DD dd_fast(double a, double b)  // |a| >= |b|
 {
-    if (x >= 1.5L)
-        return ((1.0L + x) * expl(-x) - 1.0L) / (x * x);
-    long double s = 0.0L, t = 1.0L;  // t = (-1)^k x^(k-1) / (k+1)!
-    for (int k = 1; k < 40; ++k) {
-        t = k == 1 ? -0.5L : -t * x / (k + 1);
-        s += k * t;
-    }
+    const double s = __dadd_rn(a, b);
+    return {s, __dadd_rn(b, -__dadd_rn(s, -a))};
+}
+__device__ __forceinline__ DD operator+(DD a, DD b)
+{
+    const double s = __dadd_rn(a.h, b.h), t = __dadd_rn(s, -a.h);
+    const double e = __dadd_rn(__dadd_rn(a.h, -__dadd_rn(s, -t)), __dadd_rn(b.h, -t));
+    return dd_fast(s, __dadd_rn(e, __dadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ DD operator-(DD a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ DD operator*(DD a, DD b)
+{
+    const double p = __dmul_rn(a.h, b.h), e = __fma_rn(a.h, b.h, -p);
+    return dd_fast(p, __fma_rn(a.h, b.l, __fma_rn(a.l, b.h, e)));
+}
+__device__ __forceinline__ DD operator/(DD a, DD b)
+{
+    const double q = a.h / b.h;
+    const DD r = a + -(b * DD{q, 0.0});
+    return dd_fast(q, r.h / b.h);
+}
+__device__ __forceinline__ DD scaled(DD a, int k) { return {ldexp(a.h, k), ldexp(a.l, k)}; }
+__device__ __forceinline__ long long rounded(DD a)
+{
+    const long long i = __double2ll_rn(a.h);
+    return i + __double2ll_rn(__dadd_rn(__dadd_rn(a.h, -(double)i), a.l));
+}
+
+__device__ DD dd_cos(DD x)  // by its Taylor series; |x| <= pi / 2
+{
+    const DD x2 = x * x;
+    DD s = {1.0, 0.0};
+    for (int k = 28; k >= 2; k -= 2)
+        s = DD{1.0, 0.0} + -(x2 * s / DD{(double)(k * (k - 1)), 0.0});
     return s;
 }
 
-// Coefficients (monomial in t / h, |t| <= h) of the degree-D truncation of the Chebyshev interpolant of fn about c.
-template <int D>
-void cheb(long double (*fn)(long double), long double c, long double h, long double *out)
+__device__ DD dd_exp_neg(DD x)  // e^-x, 0 <= x < 128: the Taylor series at x / 4096, squared twelve times
 {
-    constexpr int N = 16;
-    const long double pi = 3.141592653589793238462643383279502884L;
-    long double a[D + 1];
-    for (int k = 0; k <= D; ++k) {
-        a[k] = 0.0L;
-        for (int j = 0; j < N; ++j)
-            a[k] += fn(c + h * cosl(pi * (j + 0.5L) / N)) * cosl(pi * k * (j + 0.5L) / N);
-        a[k] *= (k == 0 ? 1.0L : 2.0L) / N;
+    const DD t = scaled(x, -12);
+    DD s = {1.0, 0.0};
+    for (int k = 14; k >= 1; --k)
+        s = DD{1.0, 0.0} + -(t * s / DD{(double)k, 0.0});
+    for (int k = 0; k < 12; ++k)
+        s = s * s;
+    return s;
+}
+
+// F(x) = (1 - e^-x) / x = sum_k (-x)^k / (k+1)!, or F'(x) = ((1 + x) e^-x - 1) / x^2 = sum_k (-1)^(k+1) (k+1) x^k / (k+2)!:
+// the series below x = 1.5.
+__device__ DD blob_value(bool derivative, DD x)
+{
+    const DD one = {1.0, 0.0};
+    if (x.h < 1.5) {
+        DD s = {0.0, 0.0};
+        for (int k = 36; k >= 0; --k)  // s = c_k - x s / (k + 2 or 3), c_k = 1 or k + 1
+            s = DD{derivative ? k + 1.0 : 1.0, 0.0} + -(x * s / DD{k + (derivative ? 3.0 : 2.0), 0.0});
+        return derivative ? scaled(-s, -1) : s;
     }
-    long double T[D + 1][D + 1] = {};  // T_k(s) = sum_m T[k][m] s^m
-    T[0][0] = 1.0L;
-    T[1][1] = 1.0L;
-    for (int k = 2; k <= D; ++k)
-        for (int m = 0; m <= k; ++m)
-            T[k][m] = (m ? 2.0L * T[k - 1][m - 1] : 0.0L) - T[k - 2][m];
-    for (int m = 0; m <= D; ++m) {
-        out[m] = 0.0L;
-        for (int k = D; k >= m; --k)
-            out[m] += a[k] * T[k][m];
-    }
+    const DD e = dd_exp_neg(x);
+    return derivative ? ((one + x) * e + -one) / (x * x) : (one + -e) / x;
 }
 
 // The same functions for the fixed point on [0, 128): rows of degree-5 polynomials of F and of -F' in u = (x - c) / h
@@ -80,6 +108,66 @@ void cheb(long double (*fn)(long double), long double c, long double h, long dou
 // c4 2^58. Both functions are completely monotone, so the signs alternate: c2 > 0 > c5.
 constexpr int kFixN = 1536;
 __device__ int4 g_fix_f[kFixN * 2], g_fix_d[kFixN * 2];
+
+// cos(pi m / 32) from its values for m <= 16.
+__device__ DD cosine(const DD *cosines, int m)
+{
+    m &= 63;
+    m = m > 32 ? 64 - m : m;
+    return m > 16 ? -cosines[32 - m] : cosines[m];
+}
+
+// Sixteen threads per row of the four tables, one per Chebyshev node: the interpolant of F or F' about c at the nodes
+// c + h cos(pi (2 j + 1) / 32), truncated to degree 6 (5), as a polynomial in t / h, |t| <= h. Filled once per process and
+// device, in 0.33 ms (in long double on the host, which Arm has in software, they took 0.7 s of every first call).
+constexpr int kRows = 2 * (kTabN + kFixN);
+__constant__ signed char c_cheb[7][7] = {{1}, {0, 1}, {-1, 0, 2}, {0, -3, 0, 4}, {1, 0, -8, 0, 8}, {0, 5, 0, -20, 0, 16}, {-1, 0, 18, 0, -48, 0, 32}};
+__global__ void __launch_bounds__(64) k_near64_tables()  // grid: kRows / 4
+{
+    __shared__ DD cosines[17], val[4][16], coef[4][7], mono[4][7];
+    if (threadIdx.x < 17)
+        cosines[threadIdx.x] = dd_cos(DD{3.141592653589793116, 1.2246467991473532e-16} * DD{threadIdx.x / 32.0, 0.0});
+    __syncthreads();
+    const int sub = threadIdx.x >> 4, j = threadIdx.x & 15, row = 4 * blockIdx.x + sub;
+    const bool derivative = row & 1, fixed = row >= 2 * kTabN;
+    const int i = (row >> 1) - (fixed ? kTabN : 0), deg = fixed ? 5 : 6;
+    const int o = i < 512 ? 0 : (i >> 8) - 1;  // fixed: octave [4 2^o, 8 2^o) for i >= 256
+    const double c = fixed ? ldexp((i - 256 * o + 0.5) / 64.0, o) : (i + 0.5) / 16.0;
+    const double h = fixed ? ldexp(1.0 / 128.0, o) : 1.0 / 32.0;
+    val[sub][j] = blob_value(derivative, DD{c, 0.0} + DD{h, 0.0} * cosine(cosines, 2 * j + 1));
+    __syncthreads();
+    if (j <= deg) {
+        DD a = {0.0, 0.0};
+        for (int n = 0; n < 16; ++n)
+            a = a + val[sub][n] * cosine(cosines, j * (2 * n + 1));
+        coef[sub][j] = scaled(a, j == 0 ? -4 : -3);
+    }
+    __syncthreads();
+    if (j <= deg) {
+        DD a = {0.0, 0.0};
+        for (int k = deg; k >= j; --k)
+            a = a + coef[sub][k] * DD{(double)c_cheb[k][j], 0.0};
+        mono[sub][j] = fixed && derivative ? -a : a;
+    }
+    __syncthreads();
+    if (j != 0)
+        return;
+    const DD *a = mono[sub];
+    if (!fixed) {
+        double v[8];
+        for (int m = 0; m <= 6; ++m)
+            v[m] = ldexp(a[m].h, 5 * m);  // t in place of t / h
+        v[7] = c;
+        for (int m = 0; m < 4; ++m)
+            (derivative ? g_blob_d : g_blob_f)[4 * i + m] = make_double2(v[2 * m], v[2 * m + 1]);
+    } else {
+        const long long c0 = rounded(scaled(a[0], 62)), c1 = rounded(scaled(a[1], 64)),
+                        c2 = rounded(scaled(a[2], 66)) | (rounded(scaled(-a[5], 58)) << 50);
+        int4 *r = (derivative ? g_fix_d : g_fix_f) + 2 * i;
+        r[0] = make_int4((int)c0, (int)(c0 >> 32), (int)c1, (int)(c1 >> 32));
+        r[1] = make_int4((int)c2, (int)(c2 >> 32), (int)rounded(scaled(a[3], 56)), (int)rounded(scaled(a[4], 58)));
+    }
+}
 
 std::mutex g_tab_mu;
 bool g_tab_ready[64];
@@ -1029,40 +1117,8 @@ int prepare_near64(cudaStream_t s)
     std::lock_guard<std::mutex> lk(g_tab_mu);
     if (g_tab_ready[dev])
         return 0;
-    static double tab[2][kTabN][8];
-    static int fix[2][kFixN][8];
-    for (int k = 0; k < 2; ++k) {
-        long double a[7];
-        for (int i = 0; i < kTabN; ++i) {
-            const long double c = (i + 0.5L) / 16.0L;
-            cheb<6>(k ? blob_d : blob_f, c, 1.0L / 32.0L, a);
-            for (int m = 0; m <= 6; ++m)
-                tab[k][i][m] = (double)ldexpl(a[m], 5 * m);  // t in place of t / h
-            tab[k][i][7] = (double)c;
-        }
-        for (int i = 0; i < kFixN; ++i) {
-            const int o = i < 512 ? 0 : (i >> 8) - 1;  // octave [4 2^o, 8 2^o) for i >= 256
-            cheb<5>(k ? blob_d : blob_f, ldexpl((i - 256 * o + 0.5L) / 64.0L, o), ldexpl(1.0L / 128.0L, o), a);
-            for (int m = 0; m <= 5; ++m)
-                a[m] = k ? -a[m] : a[m];
-            const long long c0 = llroundl(ldexpl(a[0], 62)), c1 = llroundl(ldexpl(a[1], 64)),
-                            c2 = llroundl(ldexpl(a[2], 66)) | (llroundl(ldexpl(-a[5], 58)) << 50);
-            int *r = fix[k][i];
-            r[0] = (int)c0;
-            r[1] = (int)(c0 >> 32);
-            r[2] = (int)c1;
-            r[3] = (int)(c1 >> 32);
-            r[4] = (int)c2;
-            r[5] = (int)(c2 >> 32);
-            r[6] = (int)llroundl(ldexpl(a[3], 56));
-            r[7] = (int)llroundl(ldexpl(a[4], 58));
-        }
-    }
-    if (cudaMemcpyToSymbolAsync(g_blob_f, tab[0], sizeof tab[0], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(g_blob_d, tab[1], sizeof tab[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(g_fix_f, fix[0], sizeof fix[0], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(g_fix_d, fix[1], sizeof fix[1], 0, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
+    k_near64_tables<<<kRows / 4, 64, 0, s>>>();
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
         return -1;
     if (cudaFuncSetAttribute(k_adjoint_near64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A64_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(k_adjoint_near64, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
