@@ -163,8 +163,10 @@ __device__ __forceinline__ double inverse(double v) { return abs(exponent_of(v))
 
 __device__ __forceinline__ double2 centre(const SysDev &d, int l, int x, int y)
 {
-    const double w = ldexp(d.S, -l);
-    return make_double2(d.x0 + (x + 0.5) * w, d.y0 + (y + 0.5) * w);
+    const double w = abs(exponent_of(d.S)) < 1000 ? exp2_scaled(d.S, -l) : ldexp(d.S, -l);
+    // 2^52 + x from its bits, less 2^52 - 1/2: x + 1/2 without a conversion (which is FP64 work too)
+    const double hx = __hiloint2double(0x43300000, x) - 4503599627370495.5, hy = __hiloint2double(0x43300000, y) - 4503599627370495.5;
+    return make_double2(d.x0 + hx * w, d.y0 + hy * w);
 }
 
 // ------------------------------------------------------------------ existing boxes of every level
@@ -772,10 +774,8 @@ __global__ void __launch_bounds__(128) k_ad_lists(Work w)
                     }
                 },
                 [&](int ls, int sx, int sy) {
-                    if (nw < AD_WCAP) {
-                        o.w[nw].c = centre(d, ls, sx, sy);
-                        o.w[nw].box = pack_box(ls, sx, sy);
-                    }
+                    if (nw < AD_WCAP)
+                        o.w[nw] = pack_box(ls, sx, sy);
                     ++nw;
                 });
             if (nu > AD_UCAP || nw > AD_WCAP)
@@ -798,6 +798,7 @@ template <class Near, class Far>
 __device__ __forceinline__ void leaf_uw(const Work &w, const Tree &t, int i, int &l, int &bx, int &by, double2 &c, Near near,
                                         Far far)
 {
+    const SysDev &d = w.sys[0];
     const int slot = w.ad_leaf ? w.ad_leaf[i] : -1;
     if (slot >= 0) {
         const AdLeaf &o = w.ad_lists[slot];
@@ -809,12 +810,11 @@ __device__ __forceinline__ void leaf_uw(const Work &w, const Tree &t, int i, int
         for (int r = 0; r < nu; ++r)
             near(o.u[r].x, o.u[r].y);
         for (int r = 0; r < nw; ++r) {
-            const int b = o.w[r].box;
-            far(b >> 26, (b >> 13) & 0x1fff, b & 0x1fff, o.w[r].c);
+            const int b = o.w[r], ls = b >> 26, sx = (b >> 13) & 0x1fff, sy = b & 0x1fff;
+            far(ls, sx, sy, centre(d, ls, sx, sy));
         }
         return;
     }
-    const SysDev &d = w.sys[0];
     particle_leaf(t, (unsigned)w.sleaf[i], l, bx, by);
     c = centre(d, l, bx, by);
     walk_uw(w, t, l, bx, by, near, [&](int ls, int sx, int sy) { far(ls, sx, sy, centre(d, ls, sx, sy)); });

@@ -378,11 +378,18 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     sizes[i++] = mixed ? m2l_tc_layout_bytes(h->lv, p) : 0;     // 35 mtc (tensor-core M2L windows)
     sizes[i++] = mixed ? m2l_tc_part_bytes(h->lv, p) : 0;       // 36 m2l_part (its partial locals)
     sizes[i++] = mixed ? m2l_tc_count_bytes(h->lv, p) : 0;      // 37 m2l_cnt (its tile counters)
-    // 38, 39 the adaptive leaves' U and W lists: room for leaves an eighth full on average
-    const int ad_cap = h->adaptive_cap ? (int)std::min<int64_t>(n, n * 8 / h->adaptive_cap + 1024) : 0;
-    sizes[i++] = h->adaptive_cap ? np * 4 : 0;                              // ad_leaf
-    sizes[i++] = (size_t)ad_cap * sizeof(AdLeaf);                           // ad_lists
-    sizes[i++] = mixed ? (size_t)nleaf * 4 + 2048 : 0;                         // 40 order, order_cnt (any tile: it may change)
+    sizes[i++] = mixed ? (size_t)nleaf * 4 + 2048 : 0;                         // 38 order, order_cnt (any tile: it may change)
+    // 39 the adaptive leaves' U and W lists take the place of the caller-order records (rec64), which are free by then: one
+    // for ten particles, which capacities of 32 and more leave room in (12 to 26 particles a leaf). Where more are wanted
+    // (room for leaves an eighth full), up to 256 MB of their own; leaves beyond the lists are walked by each particle.
+    // 20000 and 2^20 particles with B = 16: lists for all leaves 195 and 1690 us, for one in ten particles 231 and 1770.
+    const int64_t ad_rec = (int64_t)(np * sizeof(Rec64) / sizeof(AdLeaf));
+    int64_t ad_cap = h->adaptive_cap ? std::min<int64_t>(std::min<int64_t>(n, n * 8 / h->adaptive_cap + 1024),
+                                                          (int64_t)((256u << 20) / sizeof(AdLeaf))) : 0;
+    const bool ad_own = ad_cap > ad_rec;
+    sizes[i++] = ad_own ? (size_t)ad_cap * sizeof(AdLeaf) : 0;
+    if (h->adaptive_cap && !ad_own)
+        ad_cap = ad_rec;
     int count = i;
     Layout lay;
     size_t total = 0;
@@ -473,11 +480,11 @@ static fmm_status ensure_workspace(fmm_handle h, int64_t n, int adjoint)
     w.adj_far = sizes[28] ? (double *)(b + lay.off[28]) : nullptr;
     w.ad_list = sizes[29] ? (int *)(b + lay.off[29]) : nullptr;
     w.ad_cnt = sizes[30] ? (int *)(b + lay.off[30]) : nullptr;
-    w.ad_leaf = sizes[38] ? (int *)(b + lay.off[38]) : nullptr;
-    w.ad_lists = sizes[39] ? (AdLeaf *)(b + lay.off[39]) : nullptr;
-    w.ad_cap = ad_cap;
-    w.order_cnt = sizes[40] ? (int *)(b + lay.off[40]) : nullptr;
-    w.order = sizes[40] ? w.order_cnt + 512 : nullptr;
+    w.ad_leaf = h->adaptive_cap ? w.key : nullptr;
+    w.ad_lists = !h->adaptive_cap ? nullptr : ad_own ? (AdLeaf *)(b + lay.off[39]) : (AdLeaf *)w.rec64;
+    w.ad_cap = (int)ad_cap;
+    w.order_cnt = sizes[38] ? (int *)(b + lay.off[38]) : nullptr;
+    w.order = sizes[38] ? w.order_cnt + 512 : nullptr;
     w.blob_f = near64_table();
     w.big = (int *)(b + lay.off[31]);
     w.cls_off = sizes[32] ? (int *)(b + lay.off[32]) : nullptr;

@@ -156,15 +156,12 @@ __device__ __forceinline__ Near64 near64_of(const SysDev &d)
     return c;
 }
 
-// U and W lists of an adaptive leaf (adaptive.cu).
+// U and W lists of an adaptive leaf (adaptive.cu): 320 bytes.
 struct AdLeaf {
     int box, nu, nw, pad;   // packed box; numbers of entries
     double2 c;              // centre
     int2 u[AD_UCAP];        // particle ranges
-    struct W {
-        double2 c;          // centre
-        int box, pad[3];
-    } w[AD_WCAP];
+    int w[AD_WCAP];         // packed boxes
 };
 
 // Per-level work lists for the tree sweeps, computed on the host and passed by value. The systems that have
@@ -222,7 +219,8 @@ struct Work {
     int *ad_cnt;              // [FMM_MAXL + 2] adaptive tree: number of existing boxes per level; then the number of
                               // leaves in the lists below
     int *ad_leaf;             // adaptive tree: [n] the list number of each sorted particle's leaf, -1: none (walked)
-    struct AdLeaf *ad_lists;  // adaptive tree: [ad_cap] the leaves' U and W lists
+    struct AdLeaf *ad_lists;  // adaptive tree: [ad_cap] the leaves' U and W lists, in their own memory or in that of rec64,
+                              // which is free once the particles are in leaf order (ad_leaf: in that of key)
     int ad_cap;
     const double2 *blob_f;    // FP64 table of F (near64_table)
     // arrays
