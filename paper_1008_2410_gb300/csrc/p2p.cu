@@ -14,6 +14,8 @@
 // each packed f32x2 instruction. Per-target sums are FP32 within a row of source leaves and compensated
 // (TwoSum) across rows. Tiles arrive by bulk asynchronous copies (cp.async.bulk, the TMA engine) into shared
 // memory, completed on an mbarrier with a bounded wait.
+#include <algorithm>
+
 #include "fmm_internal.cuh"
 
 #include <type_traits>
@@ -670,12 +672,14 @@ __global__ void __launch_bounds__(P2PBounds<LPB, KTM>::threads, P2PBounds<LPB, K
 // an SM, so registers are free and latency is what counts). The sums are those of k_p2p32 with lpb leaves a block, to
 // the last bit: the same tile boundaries (the row of the block's lpb + 2 columns cut every `tile` sources), plain FP32
 // sums within a tile, kept per row and tile in shared memory and added by TwoSum in the same order at the end. A leaf
-// with more tiles in a row than P2PW_TILES (dense) goes row by row through the first warp. Latency bound; 4096 uniform
+// with more tiles in a row than P2PW_TILES (dense) goes row by row through the first warp. OWN: buffers of `buf` records,
+// fewer than a tile, which take the leaf's own columns' part of it; a leaf with more of them goes the dense way too, the
+// three warps' buffers together holding a tile. Latency bound; 4096 uniform
 // particles (64 leaves): 73 us with k_p2p32 (32 blocks), 14 us so.
 #define P2PW_TILES 4
 #define P2PW_UNROLL 4
-template <int KTM>
-__global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
+template <int KTM, bool OWN>
+__global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int buf, int lpb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bars[3];
@@ -686,8 +690,7 @@ __global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
     float4 *TT = reinterpret_cast<float4 *>(smem_raw);            // the pass's targets: x hi, x lo, y hi, y lo
     f2 *part = reinterpret_cast<f2 *>(TT + full_pass);            // [3][P2PW_TILES][2 NPR][32] sums of a tile
     const int nbuf = w.p2p_all_plain ? 2 : 3;
-    float4 *EH = reinterpret_cast<float4 *>(part + 3 * P2PW_TILES * 2 * NPR * 32) + (size_t)warp * tile * nbuf;
-    float4 *EG = EH + tile, *EL = EG + tile;
+    float4 *EH = reinterpret_cast<float4 *>(part + 3 * P2PW_TILES * 2 * NPR * 32) + (size_t)warp * (OWN ? buf : tile) * nbuf;
     const int leaf = blockIdx.x;
     const int k = w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf);
     const SysDev &d = w.sys[k];
@@ -707,9 +710,17 @@ __global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
         const int row = iy + dyr;
         if (row >= 0 && row < ns) {
             const int rl = (int)d.leaf0 + row * ns;
-            dense |= w.start[rl + cz + 1] - w.start[rl + ca] > P2PW_TILES * tile;
+            const int r0 = w.start[rl + ca], r1 = w.start[rl + cz + 1];
+            dense |= r1 - r0 > P2PW_TILES * tile;
+            if (OWN && r1 - r0 > buf) {  // the leaf's own columns in one tile may be more than its buffer holds
+                const int own0 = w.start[rl + max(ix - 1, 0)], own1 = w.start[rl + min(ix + 1, ns - 1) + 1];
+                const int b = own0 + tile - (own0 - r0) % tile;  // the tile of own0 ends there
+                dense |= own1 - own0 > buf && max(b - own0, own1 - b) > buf;
+            }
         }
     }
+    const int hold = OWN && !dense ? buf : tile;  // records in a buffer (dense: the three warps' hold a tile)
+    float4 *EG = EH + hold, *EL = EG + hold;
     uint64_t &bar = bars[warp];
     if (lane == 0) {
         mbar_init(&bar, 1);
@@ -747,6 +758,9 @@ __global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
                 continue;
             const int rowleaf = (int)d.leaf0 + row * ns;
             const int r0 = w.start[rowleaf + ca], r1 = w.start[rowleaf + cz + 1];
+            // OWN: of the block's columns the leaf's own three are copied
+            const int own0 = OWN ? w.start[rowleaf + max(ix - 1, 0)] : r0;
+            const int own1 = OWN ? w.start[rowleaf + min(ix + 1, ns - 1) + 1] : r1;
             __syncwarp();
             if (lane < 3) {  // the row's three source leaves (see k_p2p32)
                 const int col = ix - 1 + lane;
@@ -775,32 +789,35 @@ __global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
             __syncwarp();
             for (int q0 = r0, it = 0; q0 < r1; q0 += tile, ++it) {
                 const int m = min(tile, r1 - q0);
-                __syncwarp();  // the warp is done with the previous tile
-                if (lane == 0) {
-                    fence_proxy_async();
-                    mbar_expect_tx(&bar, (uint32_t)m * (split ? 48u : 32u));
-                    bulk_g2s(EH, w.eh + q0, (uint32_t)m * 16u, &bar);
-                    bulk_g2s(EG, w.eg + q0, (uint32_t)m * 16u, &bar);
-                    if (split)
-                        bulk_g2s(EL, w.el + q0, (uint32_t)m * 16u, &bar);
+                const int base = OWN ? max(own0, q0) : q0, mine = OWN ? min(own1, q0 + m) - base : m;
+                if (!OWN || mine > 0) {
+                    __syncwarp();  // the warp is done with the previous tile
+                    if (lane == 0) {
+                        fence_proxy_async();
+                        mbar_expect_tx(&bar, (uint32_t)mine * (split ? 48u : 32u));
+                        bulk_g2s(EH, w.eh + base, (uint32_t)mine * 16u, &bar);
+                        bulk_g2s(EG, w.eg + base, (uint32_t)mine * 16u, &bar);
+                        if (split)
+                            bulk_g2s(EL, w.el + base, (uint32_t)mine * 16u, &bar);
+                    }
+                    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar, phase, w.status))) {
+                        mbar_wait_bounded(&bar, phase, w.status);  // let a late copy land before exiting
+                        ok = false;
+                        break;
+                    }
+                    phase ^= 1;
                 }
-                if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar, phase, w.status))) {
-                    mbar_wait_bounded(&bar, phase, w.status);  // let a late copy land before exiting
-                    ok = false;
-                    break;
-                }
-                phase ^= 1;
                 f2 PU[2] = {0ull, 0ull}, PV[2] = {0ull, 0ull};
 #pragma unroll 1
                 for (int k3 = 0; k3 < 3; ++k3) {
                     const int4 sg = segtab[warp][k3];
-                    const int j0 = max(q0, sg.x) - q0, j1 = min(q0 + m, sg.y) - q0;
+                    const int j0 = max(q0, sg.x) - base, j1 = min(q0 + m, sg.y) - base;
                     if (j0 >= j1)
                         continue;
                     const float sdx = (float)(k3 - 1) * s, sdy = (float)dyr * s;
                     const bool self = k3 == 1 && dyr == 0;
-                    const int t1 = min(max(segt1[warp][k3] - q0, j0), j1);
-                    const int ja = min(max(sg.z - q0, t1), j1), jb = max(min(sg.w - q0, j1), ja);
+                    const int t1 = min(max(segt1[warp][k3] - base, j0), j1);
+                    const int ja = min(max(sg.z - base, t1), j1), jb = max(min(sg.w - base, j1), ja);
 #define P2P_SEG(KT, SELF, SPLIT) \
     p2p_segment<KT, SELF, SPLIT, P2PW_UNROLL>(w, EH, EL, EG, j0, j1, t1, ja, jb, sdx, sdy, TT, n_main, PU, PV)
                     if (KTM == 4 && kt4) {
@@ -909,10 +926,10 @@ __global__ void __launch_bounds__(96, 6) k_p2p32w(Work w, int tile, int lpb)
 }
 
 template <int KTM>
-static size_t p2pw_smem(const Work &w, int tile)
+static size_t p2pw_smem(const Work &w, int buf)
 {
     return (KTM == 4 ? 128 : 64) * sizeof(float4) + 3 * P2PW_TILES * 2 * (KTM == 4 ? 2 : 1) * 32 * sizeof(f2) +
-           (size_t)3 * tile * (w.p2p_all_plain ? 32 : 48);
+           (size_t)3 * buf * (w.p2p_all_plain ? 32 : 48);
 }
 
 // ------------------------------------------------------------------ precision form, symmetric near field
@@ -1380,11 +1397,14 @@ int prepare_p2p()
     if (cudaFuncSetAttribute(k_p2p32<1, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
         cudaFuncSetAttribute(k_p2p32<2, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
         cudaFuncSetAttribute(k_p2p32<1, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-        cudaFuncSetAttribute(k_p2p32<2, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-        cudaFuncSetAttribute(k_p2p32w<2>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-        cudaFuncSetAttribute(k_p2p32w<4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess ||
-        cudaFuncSetAttribute(k_p2p32w<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess ||
-        cudaFuncSetAttribute(k_p2p32w<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess)
+        cudaFuncSetAttribute(k_p2p32<2, 4>, cudaFuncAttributePreferredSharedMemoryCarveout, c) != cudaSuccess)
+        return -1;
+    auto attributes = [&](auto k) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, c) == cudaSuccess &&
+               cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) == cudaSuccess;
+    };
+    if (!attributes(k_p2p32w<2, false>) || !attributes(k_p2p32w<4, false>) || !attributes(k_p2p32w<2, true>) ||
+        !attributes(k_p2p32w<4, true>))
         return -1;
     g_p2p_ready[dev] = 1;
     return 0;
@@ -1430,14 +1450,26 @@ int launch_p2p(const Work &w, int threads, int kt, cudaStream_t s)
     const size_t sm = (size_t)tile * (w.p2p_all_plain ? 32 : 48) + (size_t)2 * 32 * ktmax * 16;
     const bool pairs1 = w.lv.nsys_at[1] == w.nsys, quads = threads == 256 && w.lv.nsys_at[2] == w.nsys;
     // few leaves: the same sums, a warp per leaf and source row. Evaluation in a graph, k_p2p32 / k_p2p32w: 64 leaves
-    // of 64 particles 89 / 43 us, 256 of 64 101 / 55, 1024 of 98 327 / 109, 4096 of 98 353 / 292, 4096 of 64 190 / 185,
-    // but 4096 of 39 108 / 138 (two per lane leave a third of the slots empty, and a row's tile is copied per leaf)
+    // of 64 particles 89 / 43 us, 256 of 64 101 / 55, 1024 of 4, 24, 32, 39, 48, 63, 98 64 / 57, 76 / 61, 95 / 64, 95 / 66,
+    // 113 / 70, 167 / 77, 327 / 109, 4096 of 98 353 / 292, 4096 of 64 190 / 185, but 4096 of 39 108 / 138 (two per lane
+    // leave a third of the slots empty, and a row's tile is copied per leaf)
     if (threads != 192 && (w.nleaf <= 1024 || (w.nleaf <= 4096 && w.n / 64 >= w.nleaf))) {
         const int tl = quads ? (w.p2p_all_plain ? P2P_TILE4 : 288) : tile, lpb = quads ? 4 : ((threads == 64 || threads == 256) && pairs1 ? 2 : 1);
-        if (ktmax == 4)
-            k_p2p32w<4><<<w.nleaf, 96, p2pw_smem<4>(w, tl), s>>>(w, tl, lpb);
+        // Buffers of the leaf's own three columns where a whole tile would leave room for three blocks an SM (four-leaf tiles of
+        // 448): 4096 leaves of 64, 80 and 96 particles 188, 284, 358 us with k_p2p32, 236, 313, 369 with whole tiles, 185,
+        // 242, 317 so. With fewer leaves whole tiles are as good on uniform particles and up to 45% faster on clustered
+        // ones, whose rows would go through one warp.
+        const int buf = w.nleaf <= 1024 ? tl : std::min(tl, std::max(256, ((int)(4ll * w.n / w.nleaf) + 31) / 32 * 32));
+        auto run = [&](auto k4, auto k2) {
+            if (ktmax == 4)
+                k4<<<w.nleaf, 96, p2pw_smem<4>(w, buf), s>>>(w, tl, buf, lpb);
+            else
+                k2<<<w.nleaf, 96, p2pw_smem<2>(w, buf), s>>>(w, tl, buf, lpb);
+        };
+        if (buf < tl)
+            run(k_p2p32w<4, true>, k_p2p32w<2, true>);
         else
-            k_p2p32w<2><<<w.nleaf, 96, p2pw_smem<2>(w, tl), s>>>(w, tl, lpb);
+            run(k_p2p32w<4, false>, k_p2p32w<2, false>);
         return 1;
     }
     if (quads) {
