@@ -1370,8 +1370,7 @@ fmm_status fmm_velocity_adjoint(fmm_handle h, int64_t n, const double *x, const 
     cudaStream_t s = h->stream;
     int64_t nl = 0;
     bool far = w.lv.maxdepth >= 2;
-    // counts, overflow flag, the near field's next leaf, its number of weak targets
-    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 3) * sizeof(int), s));
+    CU(cudaMemsetAsync(w.cnt, 0, (size_t)(w.nleaf + 2) * sizeof(int), s));  // counts, overflow flag, the near field's next leaf
     if (!h->has_domain) {
         nl += launch_bbox(w, x, y, s);
     }

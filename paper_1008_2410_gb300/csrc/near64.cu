@@ -402,21 +402,35 @@ __device__ __forceinline__ int pick_passes(int c)
 // agree to 2.5e-16 either way).
 // Sums of 64-bit sums, one per thread: 96 bits, carried in shared memory (a conversion to FP64 and an addition on that
 // pipe cost as much as half a pair).
+// big: the largest magnitude that a sum has had at an addition, in units of 2^32 (to 2^-24 of it or 2^8; 0 only if it was
+// always zero).
 struct Acc64 {
     unsigned long long lo[N64_THREADS];
     int hi[N64_THREADS];
-    __device__ __forceinline__ void clear(int t) { lo[t] = 0, hi[t] = 0; }
+    float big[N64_THREADS];
+    __device__ __forceinline__ void clear(int t) { lo[t] = 0, hi[t] = 0, big[t] = 0.0f; }
+    __device__ __forceinline__ void store(int t, unsigned long long l, int h)
+    {
+        lo[t] = l;
+        hi[t] = h;
+        big[t] = fmaxf(big[t], fmaxf(fabsf(fmaf((float)h, 0x1p32f, (float)(unsigned)(l >> 32))), (l | (unsigned)h) ? 1.0f : 0.0f));
+    }
     __device__ __forceinline__ void add(int t, long long v)
     {
         const unsigned long long a = lo[t], b = a + (unsigned long long)v;
-        lo[t] = b;
-        hi[t] += (int)(v >> 63) + (b < a ? 1 : 0);
+        store(t, b, hi[t] + (int)(v >> 63) + (b < a ? 1 : 0));
     }
     __device__ __forceinline__ void add(int t, long long h, long long l)  // h 2^24 + l
     {
         const unsigned long long a = lo[t], b = a + ((unsigned long long)h << 24), d = b + (unsigned long long)l;
-        lo[t] = d;
-        hi[t] += (int)(h >> 40) + (b < a ? 1 : 0) + (int)(l >> 63) + (d < b ? 1 : 0);
+        store(t, d, hi[t] + (int)(h >> 40) + (b < a ? 1 : 0) + (int)(l >> 63) + (d < b ? 1 : 0));
+    }
+    __device__ __forceinline__ float biggest(int t, int step, int n) const  // of threads t, t + step, ...
+    {
+        float m = big[t];
+        for (int k = 1; k < n; ++k)
+            m = fmaxf(m, big[t + k * step]);
+        return m;
     }
     // the sum over threads t, t + step, ... (n of them), as FP64
     __device__ __forceinline__ double total(int t, int step, int n) const
@@ -429,13 +443,6 @@ struct Acc64 {
             a = b;
         }
         return fma((double)(h + (int)(a >> 63)), 0x1p64, (double)(long long)a);
-    }
-    // thread t's sum in magnitude, in units of 2^32 (to 2^-24 of it or 2^8); 0 only if it is zero
-    __device__ __forceinline__ float size(int t) const
-    {
-        const unsigned long long l = lo[t];
-        const int h = hi[t];
-        return fmaxf(fabsf(fmaf((float)h, 0x1p32f, (float)(unsigned)(l >> 32))), (l | (unsigned)h) != 0 ? 1.0f : 0.0f);
     }
 };
 // v, without the compiler's knowledge that it is the same in every pass: what is derived from it is not kept in registers
@@ -659,14 +666,11 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
         const bool some64 = __syncthreads_or(au != 0.0 || av != 0.0);
         if (some64)
             red[tid] = make_double2(au, av);
-        float2 *sizes = reinterpret_cast<float2 *>(lst);
-        unsigned short *weak = lst + 4 * N64_THREADS;
-        if (fixed)
-            sizes[tid] = make_float2(fmaxf(acc[0].size(tid), acc[1].size(tid)), fmaxf(acc[2].size(tid), acc[3].size(tid)));
         __syncthreads();
         if (tid < cp) {
+            const int ng = min(G, ntot);  // groups with sources
             double u = 0.0, v = 0.0;
-            for (int g = 0; some64 && g < G; ++g) {
+            for (int g = 0; some64 && g < ng; ++g) {
                 const double2 a = red[tid + g * cp];
                 u += a.x;
                 v += a.y;
@@ -680,27 +684,24 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
                 const double gs = pow2(ka), fs = pow2(-51 - ku), cs = k2 * pow2(66 - cl.s + ku);
                 // A term's rounding is about 0.4 of its unit (fs or cs, times gs) however small the term is, in FP64 it is
                 // relative to it: a target whose sums are all small against the unit, because the strong sources have no
-                // weight there, is left to FP64 below. At this line the two errors are about the same; the sums of groups
-                // of sources stand for the terms, so that a velocity that is small by cancellation does not count.
-                float2 sz = sizes[tid];
-                for (int g = 1; g < G; ++g) {
-                    const float2 q = sizes[tid + g * cp];
-                    sz = make_float2(fmaxf(sz.x, q.x), fmaxf(sz.y, q.y));
-                }
+                // weight there, is left to FP64 below. At this line the error is a few times that of FP64 sums. What counts is the
+                // largest that a sum has been on the way, so that a velocity that is small by cancellation does not count.
+                const float far = fmaxf(acc[0].biggest(tid, cp, ng), acc[1].biggest(tid, cp, ng));
+                const float near = fmaxf(acc[2].biggest(tid, cp, ng), acc[3].biggest(tid, cp, ng));
                 // (next to a coordinate axis a position is short of 2^(s - 3) units as well)
                 const float ratio = cl.lim ? (float)(k2 * pow2(117 - cl.s + 2 * ku)) : 0.0f;  // cs / fs
-                const float line = line_of(sz.x, sz.y, 0x1p20f, ratio * (cl.s > 3 ? 0x1p21f : (thr ? 0x1p20f : 0x1p21f)));
-                if (fmaxf(sz.x, sz.y * ratio) < line && (!some64 || fmax(fabs(u), fabs(v)) < line * 0x1p32 * fs * gs))
-                    weak[atomicAdd(&s_weak, 1)] = (unsigned short)tid;
-                u -= fma(acc[2].total(tid, cp, G), cs, acc[0].total(tid, cp, G) * fs) * gs;
-                v += fma(acc[3].total(tid, cp, G), cs, acc[1].total(tid, cp, G) * fs) * gs;
+                const float line = line_of(far, near, 0x1p19f, ratio * (cl.s > 3 ? 0x1p20f : (thr ? 0x1p19f : 0x1p21f)));
+                if (fmaxf(far, near * ratio) < line && (!some64 || fmax(fabs(u), fabs(v)) < line * 0x1p32 * fs * gs))
+                    lst[atomicAdd(&s_weak, 1)] = (unsigned short)tid;
+                u -= fma(acc[2].total(tid, cp, ng), cs, acc[0].total(tid, cp, ng) * fs) * gs;
+                v += fma(acc[3].total(tid, cp, ng), cs, acc[1].total(tid, cp, ng) * fs) * gs;
             }
             w.near64[tpos] = make_double2(u / kTwoPi, v / kTwoPi);
         }
         __syncthreads();
         const int nweak = s_weak;
         for (int e = 0; e < nweak; ++e) {  // the whole block on each weak target
-            const int t = s0 + t0 + weak[e];
+            const int t = s0 + t0 + lst[e];
             const double xw = w.sx[t], yw = w.sy[t];
             double bu = 0.0, bv = 0.0;
             for (int q = tid; q < ntot; q += N64_THREADS)
@@ -765,13 +766,37 @@ struct Adj64 {
 // for every pair; the whole adjoint (near field beside both sweeps) 108 ms then, 8.9 ms now. 112 or 128 registers keep
 // the sweeps' blocks out (11.6 to 12.0 ms), 80 spill (10.9). Errors against quad precision are below the former ones.
 // Writes the near part in caller order (the far part is added later). Targets for whom the fixed unit is too coarse, or
-// with coincident particles, are listed in slot (free after the binning) for k_adjoint_weak64.
+// with coincident particles, are listed in slot (free after the binning) and summed in FP64 at the end.
 constexpr int A64_REGS = 96, A64_B = 2;  // registers a thread, blocks an SM: room for the sweep's blocks beside them
 constexpr int A64_TILE = 640;
 constexpr int A64_CAP = 48;  // terms between two hand-overs to the 96-bit sums
 constexpr size_t A64_SMEM = A64_TILE * 40 + 6 * sizeof(Acc64) + A64_CAP * N64_THREADS * 2;
 
-__global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double *__restrict__ odg,
+// The near part of target t in FP64, by the whole block.
+__device__ __noinline__ void adjoint_block64(const Work &w, int t, double *red, double *odg, double *odx, double *ody)
+{
+    const int leaf = w.sleaf[t], i = w.perm[t];
+    const SysDev &d = w.sys[w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf)];
+    const Rows64 R(w, d, leaf);
+    const double k2 = near64_of(d).k2;
+    const Adj64 me(w, t);
+    double ag = 0.0, ax = 0.0, ay = 0.0;
+    for (int q = threadIdx.x; q < R.pre[3]; q += N64_THREADS)
+        me.pair(w, R.global(q), k2, ag, ax, ay);
+    ag = block_sum(ag, red);
+    ax = block_sum(ax, red);
+    ay = block_sum(ay, red);
+    if (threadIdx.x == 0) {
+        if (odg)
+            odg[i] = ag * k2 / kTwoPi;
+        if (odx)
+            odx[i] = ax * k2 / kTwoPi;
+        if (ody)
+            ody[i] = ay * k2 / kTwoPi;
+    }
+}
+
+__global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ Work w, int parts, double *__restrict__ odg,
                                                                                 double *__restrict__ odx,
                                                                                 double *__restrict__ ody, int skip_plain)
 {
@@ -782,12 +807,13 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
     Acc64 *acc = reinterpret_cast<Acc64 *>(gam + A64_TILE);  // dgamma, dx, dy of the far pairs, of the close ones
     unsigned short *lst = reinterpret_cast<unsigned short *>(acc + 6);
     __shared__ Stats64 st;
-    __shared__ int s_leaf;
+    __shared__ int s_leaf, s_weak;  // s_weak: head of the block's list of weak targets, linked by slot
     __shared__ float4 s_line;
-    __shared__ unsigned char s_same[N64_THREADS];  // whether the thread's target has a coincident particle
     const int tid = threadIdx.x;
     if (skip_plain && w.nsys == 1 && !(w.sys[0].s_unit > P2P_SPLIT_S))
         return;  // the only system's near field is the FP32 kernel's
+    if (tid == 0)
+        s_weak = -1;
     for (;;) {
     if (tid == 0)
         s_leaf = atomicAdd(&w.cnt[w.nleaf + 1], 1);
@@ -795,7 +821,7 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
     const int leaf = s_leaf / parts, part = s_leaf - leaf * parts;
     __syncthreads();
     if (leaf >= w.nleaf)
-        return;
+        break;
     int s0 = w.start[leaf], c = w.start[leaf + 1] - s0;
     {  // this unit's share of the leaf's targets
         const int a = (int)((long long)part * c / parts), b = (int)((long long)(part + 1) * c / parts);
@@ -826,7 +852,7 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             const float axis = cl.s > 3 ? 2.0f : 1.0f;
             const float rg = cl.lim ? (float)(k2 * pow2(121 - cl.s + 2 * ku)) : 0.0f;
             const float rx = cl.lim ? (float)(k2 * pow2(112 + 2 * ku)) : 0.0f;
-            s_line = make_float4(rg, axis * rg * (thr ? 0x1p39f : 0x1p43f), rx, axis * rx * (thr ? 0x1p40f : 0x1p42f));
+            s_line = make_float4(rg, axis * rg * (thr ? 0x1p38f : 0x1p42f), rx, axis * rx * (thr ? 0x1p38f : 0x1p40f));
         }
     }
     const int npass = pick_passes(c);
@@ -884,14 +910,16 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             const int own = fresh(leaf), own1 = w.start[own + 1];
             for (int h0 = w.start[own]; h0 < own1; h0 += kHashes) {
                 const int m = min(kHashes, own1 - h0);
-                __syncthreads();
+                if (h0 > w.start[own])
+                    __syncthreads();
                 for (int j = tid; j < m; j += N64_THREADS)
                     hash[j] = position_hash(w.sx[h0 + j], w.sy[h0 + j]);
                 __syncthreads();
                 for (int j = active ? grp : m; j < m; j += G)
                     same |= hash[j] == mine && h0 + j != tpos;
             }
-            s_same[tid] = same;
+            if (same)
+                acc[0].big[tid] = INFINITY;
             const long long tg = to_fixed(gt, ka - tau), tgu = to_fixed(gut, kb - tau), tgv = to_fixed(gvt, kb - tau);
             const int tgh = -hi_bal(tg), tgl = (int)lo_of(tg) >> 1;  // low limb halved: it can be negated
             const int tuh = hi_bal(tgu), tul = (int)lo_of(tgu), tvh = hi_bal(tgv), tvl = (int)lo_of(tgv);
@@ -1020,16 +1048,13 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
             red[N64_THREADS + tid] = ax;
             red[2 * N64_THREADS + tid] = ay;
         }
-        float4 *sizes = reinterpret_cast<float4 *>(lst);  // far and close sums of dgamma, of dx and dy
-        if (fixed)
-            sizes[tid] = make_float4(acc[0].size(tid), acc[3].size(tid), fmaxf(acc[1].size(tid), acc[2].size(tid)),
-                                     fmaxf(acc[4].size(tid), acc[5].size(tid)));
         __syncthreads();
         if (tid < cp) {
+            const int ng = min(G, ntot);  // groups with sources
             double out[3] = {0.0, 0.0, 0.0};
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                for (int g = 0; some64 && g < G; ++g)
+                for (int g = 0; some64 && g < ng; ++g)
                     out[q] += red[q * N64_THREADS + tid + g * cp];
                 if (ranges)
                     out[q] *= k2;
@@ -1043,24 +1068,19 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
                 // far pair's dgamma is off by 2^20 (the charges' last bits, the low halves left out), its gradient by 2^16
                 // (P and Q); a close pair's by about 2^18 and 2^19, by up to 2^21 where all pairs are close. So is one with a
                 // coincident particle.
-                float4 sz = sizes[tid];
-                for (int g = 1; g < G; ++g) {
-                    const float4 q = sizes[tid + g * cp];
-                    sz = make_float4(fmaxf(sz.x, q.x), fmaxf(sz.y, q.y), fmaxf(sz.z, q.z), fmaxf(sz.w, q.w));
-                }
+                const float far_g = acc[0].biggest(tid, cp, ng), near_g = acc[3].biggest(tid, cp, ng);
+                const float far_x = fmaxf(acc[1].biggest(tid, cp, ng), acc[2].biggest(tid, cp, ng));
+                const float near_x = fmaxf(acc[4].biggest(tid, cp, ng), acc[5].biggest(tid, cp, ng));
                 const float4 line = s_line;
-                const float lg = line_of(sz.x, sz.y, 0x1p43f, line.y), lx = line_of(sz.z, sz.w, 0x1p39f, line.w);
-                bool small = fmaxf(sz.x, sz.y * line.x) < lg;
+                bool small = fmaxf(far_g, near_g * line.x) < line_of(far_g, near_g, 0x1p42f, line.y) || far_g == INFINITY;
                 if (gt != 0.0 || gut != 0.0 || gvt != 0.0)
-                    small |= fmaxf(sz.z, sz.w * line.z) < lx;
-                for (int g = 0; g < G; ++g)
-                    small |= s_same[tid + g * cp] != 0;
+                    small |= fmaxf(far_x, near_x * line.z) < line_of(far_x, near_x, 0x1p37f, line.w);
                 if (small)
-                    w.slot[atomicAdd(&w.cnt[w.nleaf + 2], 1)] = tpos;
-                out[0] += ldexp(fma(acc[3].total(tid, cp, G), cg, acc[0].total(tid, cp, G) * fg), kb);
+                    w.slot[tpos] = atomicExch(&s_weak, tpos);
+                out[0] += ldexp(fma(acc[3].total(tid, cp, ng), cg, acc[0].total(tid, cp, ng) * fg), kb);
 #pragma unroll
                 for (int q = 1; q < 3; ++q)
-                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, G), cx, acc[q].total(tid, cp, G) * fx), ka + kb - tau);
+                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, ng), cx, acc[q].total(tid, cp, ng) * fx), ka + kb - tau);
             }
             const int i = w.perm[tpos];
             if (odg)
@@ -1073,38 +1093,10 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(Work w, int parts, double
         __syncthreads();
     }
     }
-}
-
-// The targets that k_adjoint_near64 has listed, in FP64: a block each. A kernel of its own, since in k_adjoint_near64 this
-// loop takes registers from the loops over the sources (the gradient of 2^20 uniform particles 13.33 ms so, 13.70 with the
-// loop there).
-__global__ void __launch_bounds__(N64_THREADS) k_adjoint_weak64(Work w, double *__restrict__ odg, double *__restrict__ odx,
-                                                                double *__restrict__ ody)
-{
-    __shared__ double red[N64_THREADS / 32];
-    const int n = w.cnt[w.nleaf + 2];
-    for (int e = blockIdx.x; e < n; e += gridDim.x) {
-        const int t = w.slot[e], leaf = w.sleaf[t];
-        const SysDev &d = w.sys[w.nsys == 1 ? 0 : find_sys_by_leaf(w.sys, w.nsys, leaf)];
-        const Rows64 R(w, d, leaf);
-        const double k2 = near64_of(d).k2;
-        const Adj64 me(w, t);
-        double ag = 0.0, ax = 0.0, ay = 0.0;
-        for (int q = threadIdx.x; q < R.pre[3]; q += N64_THREADS)
-            me.pair(w, R.global(q), k2, ag, ax, ay);
-        ag = block_sum(ag, red);
-        ax = block_sum(ax, red);
-        ay = block_sum(ay, red);
-        if (threadIdx.x == 0) {
-            const int i = w.perm[t];
-            if (odg)
-                odg[i] = ag * k2 / kTwoPi;
-            if (odx)
-                odx[i] = ax * k2 / kTwoPi;
-            if (ody)
-                ody[i] = ay * k2 / kTwoPi;
-        }
-    }
+    // the weak targets, in FP64 by the whole block (out of the loop over the leaves: within it, or in line, this takes
+    // registers from the loops over the sources and 3% of the kernel)
+    for (int t = s_weak; t >= 0; t = w.slot[t])
+        adjoint_block64(w, t, reinterpret_cast<double *>(pos), odg, odx, ody);
 }
 
 }  // namespace
@@ -1158,8 +1150,7 @@ int launch_adjoint_near64(const Work &w, double *dg, double *dx, double *dy, int
     const int resident = A64_B * kSMs;
     const int parts = max(1, min(8, resident / w.nleaf));
     k_adjoint_near64<<<min(w.nleaf * parts, resident), N64_THREADS, A64_SMEM, s>>>(w, parts, dg, dx, dy, skip_plain);
-    k_adjoint_weak64<<<min(w.n, 4 * kSMs), N64_THREADS, 0, s>>>(w, dg, dx, dy);
-    return 2;
+    return 1;
 }
 
 }  // namespace fmm
