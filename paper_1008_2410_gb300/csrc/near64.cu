@@ -249,7 +249,8 @@ constexpr int N64_FEW = 96;     // fewer sources than this run in FP64
 // The smallest e with every charge of the neighbourhood below 2^e (1 - 2^-12), or kNoFixed where the fixed point is not
 // for them: where the sum of the charges' squares, the largest left out, is below a quarter of the largest one's. A
 // term's rounding is about 0.3 2^-54 of a term of the largest charge, an FP64 sum of N such terms of size V takes about
-// sqrt(N) 2^-55 V, and V may leave out the target's own charge, so that from there on the fixed point is no worse.
+// sqrt(N) 2^-55 V, and V may leave out the target's own charge, so that from there on the fixed point is no worse for a
+// target that the large charges act on (the others: see the kernels' ends).
 // Subnormal, infinite and NaN charges run in FP64. b, if given, is a second array of charges of the same kind.
 // Block-uniform (integer sums, so the choice is the same in every run).
 constexpr int kNoFixed = -1000000;
@@ -376,7 +377,7 @@ __device__ __forceinline__ long long blob_fixed(const int4 *__restrict__ tab, lo
     return (((long long)a.y << 32) | (unsigned)a.x) + mul_hi(uh, ul, hi_bal(e1), (int)lo_of(e1));
 }
 
-// Passes over a leaf of c targets: the number of passes (at most 4 more than needed) that keeps most of the 256
+// Passes over a leaf of c targets: the number of passes (at most 2 more than needed) that keeps most of the 256
 // threads busy, threads = (targets of the pass) x (source groups).
 __device__ __forceinline__ int pick_passes(int c)
 {
@@ -393,13 +394,6 @@ __device__ __forceinline__ int pick_passes(int c)
     return best;
 }
 
-// One block per leaf. Thread = (target t, source group g of G): the pass's targets run over the threads, and the
-// groups take the sources in turn; the groups' sums of a target are added at the end in a fixed order.
-// Measured at 2^20 uniform particles (leaves of 64, 16 sigma wide): 39.0 ms with every pair by expm1 and a division
-// in FP64, 3.25 ms so, issue and integer pipes about 65 % busy. The error of the near field against quad precision fell
-// from 8.6e-16 to 1.9e-16 relative L2 (exact differences, integer sums).
-// Line of the fixed point: fewer than 96 sources in the neighbourhood have no time in it (4 to 24 particles a leaf
-// agree to 2.5e-16 either way).
 // Sums of 64-bit sums, one per thread: 96 bits, carried in shared memory (a conversion to FP64 and an addition on that
 // pipe cost as much as half a pair).
 // big: the largest magnitude that a sum has had at an addition, in units of 2^32 (to 2^-24 of it or 2^8; 0 only if it was
@@ -490,6 +484,14 @@ __device__ __forceinline__ double block_sum(double v, double *red)
     return v;
 }
 
+// Persistent blocks take units from a counter: a leaf, or one of `parts` shares of a leaf's targets (launch_near64). Thread =
+// (target t, source group g of G): a pass's targets run over the threads, and the groups take the sources in turn; the
+// groups' sums of a target are added at the end in a fixed order.
+// Measured at 2^20 uniform particles (leaves of 64, 16 sigma wide): 39.0 ms with every pair by expm1 and a division
+// in FP64, 3.25 ms so, issue and integer pipes about 65 % busy. The error of the near field against quad precision fell
+// from 8.6e-16 to 1.9e-16 relative L2 (integer differences and sums).
+// Line of the fixed point: fewer than 96 sources in the neighbourhood have no time in it (4 to 24 particles a leaf
+// agree to 2.5e-16 either way).
 __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 {
     __shared__ int s_leaf, s_weak;
@@ -690,7 +692,7 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
                 const float near = fmaxf(acc[2].biggest(tid, cp, ng), acc[3].biggest(tid, cp, ng));
                 // (next to a coordinate axis a position is short of 2^(s - 3) units as well)
                 const float ratio = cl.lim ? (float)(k2 * pow2(117 - cl.s + 2 * ku)) : 0.0f;  // cs / fs
-                const float line = line_of(far, near, 0x1p19f, ratio * (cl.s > 3 ? 0x1p20f : (thr ? 0x1p19f : 0x1p21f)));
+                const float line = line_of(far, near, 0x1p19f, ratio * (cl.s > 3 ? 0x1p20f : 0x1p19f));
                 if (fmaxf(far, near * ratio) < line && (!some64 || fmax(fabs(u), fabs(v)) < line * 0x1p32 * fs * gs))
                     lst[atomicAdd(&s_weak, 1)] = (unsigned short)tid;
                 u -= fma(acc[2].total(tid, cp, ng), cs, acc[0].total(tid, cp, ng) * fs) * gs;
@@ -852,7 +854,7 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ W
             const float axis = cl.s > 3 ? 2.0f : 1.0f;
             const float rg = cl.lim ? (float)(k2 * pow2(121 - cl.s + 2 * ku)) : 0.0f;
             const float rx = cl.lim ? (float)(k2 * pow2(112 + 2 * ku)) : 0.0f;
-            s_line = make_float4(rg, axis * rg * (thr ? 0x1p38f : 0x1p42f), rx, axis * rx * (thr ? 0x1p38f : 0x1p40f));
+            s_line = make_float4(rg, axis * rg * (thr ? 0x1p38f : 0x1p41f), rx, axis * rx * (thr ? 0x1p38f : 0x1p40f));
         }
     }
     const int npass = pick_passes(c);
