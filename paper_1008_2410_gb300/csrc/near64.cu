@@ -396,28 +396,30 @@ __device__ __forceinline__ int pick_passes(int c)
 
 // Sums of 64-bit sums, one per thread: 96 bits, carried in shared memory (a conversion to FP64 and an addition on that
 // pipe cost as much as half a pair).
-// big: the largest magnitude that a sum has had at an addition, in units of 2^32 (to 2^-24 of it or 2^8; 0 only if it was
-// always zero).
+// big: the largest magnitude that a sum has had when it was marked, in units of 2^32 (to 2^-24 of it or 2^8; 0 only if it
+// was always zero).
 struct Acc64 {
     unsigned long long lo[N64_THREADS];
     int hi[N64_THREADS];
     float big[N64_THREADS];
     __device__ __forceinline__ void clear(int t) { lo[t] = 0, hi[t] = 0, big[t] = 0.0f; }
-    __device__ __forceinline__ void store(int t, unsigned long long l, int h)
+    __device__ __forceinline__ void mark(int t)
     {
-        lo[t] = l;
-        hi[t] = h;
+        const unsigned long long l = lo[t];
+        const int h = hi[t];
         big[t] = fmaxf(big[t], fmaxf(fabsf(fmaf((float)h, 0x1p32f, (float)(unsigned)(l >> 32))), (l | (unsigned)h) ? 1.0f : 0.0f));
     }
     __device__ __forceinline__ void add(int t, long long v)
     {
         const unsigned long long a = lo[t], b = a + (unsigned long long)v;
-        store(t, b, hi[t] + (int)(v >> 63) + (b < a ? 1 : 0));
+        lo[t] = b;
+        hi[t] += (int)(v >> 63) + (b < a ? 1 : 0);
     }
     __device__ __forceinline__ void add(int t, long long h, long long l)  // h 2^24 + l
     {
         const unsigned long long a = lo[t], b = a + ((unsigned long long)h << 24), d = b + (unsigned long long)l;
-        store(t, d, hi[t] + (int)(h >> 40) + (b < a ? 1 : 0) + (int)(l >> 63) + (d < b ? 1 : 0));
+        lo[t] = d;
+        hi[t] += (int)(h >> 40) + (b < a ? 1 : 0) + (int)(l >> 63) + (d < b ? 1 : 0);
     }
     __device__ __forceinline__ float biggest(int t, int step, int n) const  // of threads t, t + step, ...
     {
@@ -592,6 +594,9 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             };
             for (int q0 = 0; q0 < ntot; q0 += N64_TILE) {
                 const int m = min(N64_TILE, ntot - q0);
+                if (q0 > 0)
+                    for (int q = 0; q < 4; ++q)
+                        acc[q].mark(tid);
                 __syncthreads();
                 for (int q = tid; q < m; q += N64_THREADS) {
                     const int j = R.global(q0 + q);
@@ -660,6 +665,8 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             acc[0].add(tid, su);
             acc[1].add(tid, sv);
             spill_close();
+            for (int q = 0; q < 4; ++q)
+                acc[q].mark(tid);
         }
         // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double2 *red = reinterpret_cast<double2 *>(pos);
@@ -687,7 +694,7 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
                 // A term's rounding is about 0.4 of its unit (fs or cs, times gs) however small the term is, in FP64 it is
                 // relative to it: a target whose sums are all small against the unit, because the strong sources have no
                 // weight there, is left to FP64 below. At this line the error is a few times that of FP64 sums. What counts is the
-                // largest that a sum has been on the way, so that a velocity that is small by cancellation does not count.
+                // largest that a sum has been at the tiles' ends, so that a velocity that is small by cancellation does not count.
                 const float far = fmaxf(acc[0].biggest(tid, cp, ng), acc[1].biggest(tid, cp, ng));
                 const float near = fmaxf(acc[2].biggest(tid, cp, ng), acc[3].biggest(tid, cp, ng));
                 // (next to a coordinate axis a position is short of 2^(s - 3) units as well)
@@ -978,6 +985,9 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ W
             };
             for (int q0 = 0; q0 < ntot; q0 += A64_TILE) {
                 const int m = min(A64_TILE, ntot - q0);
+                if (q0 > 0)
+                    for (int q = 0; q < 6; ++q)
+                        acc[q].mark(tid);
                 __syncthreads();
                 for (int q = tid; q < m; q += N64_THREADS) {
                     const int j = R.global(q0 + q);
@@ -1041,6 +1051,8 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ W
                     }
                 }
             }
+            for (int q = 0; q < 6; ++q)
+                acc[q].mark(tid);
         }
         // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double *red = reinterpret_cast<double *>(pos);
