@@ -116,7 +116,8 @@ int fmm_get_m2l_engine(fmm_handle h);
  * fmm_velocity_near / _far, fmm_velocity_host and fmm_advect, and counts the ordered pairs of its U lists
  * when pair counting is on; fmm_autotune then picks the leaf capacity (and the
  * maximum depth within its range); fmm_velocity_batched and fmm_velocity_adjoint return FMM_EINVAL while it is set.
- * Returns FMM_EINVAL for NULL or a negative capacity. */
+ * Memory beyond the uniform FP64 form's per-particle arrays: the expansions of the boxes, and for small capacities
+ * (many leaves) up to 256 MB of lists. Returns FMM_EINVAL for NULL or a negative capacity. */
 fmm_status fmm_set_adaptive(fmm_handle h, int leaf_capacity);
 
 /* The handle's leaf capacity (0: uniform tree), -1 for NULL. */
@@ -143,10 +144,13 @@ fmm_status fmm_set_graph(fmm_handle h, int enable);
 /* Near-field tile shape of the precision form: threads 32 (one leaf per thread block), 64 (two
  * horizontally adjacent leaves per block, sharing their source tiles), 256 (four such leaves, 128-thread
  * blocks; trees of depth >= 2, else as 64) or 128 (symmetric: each pair of
- * particles in adjacent leaves evaluated once and applied to both, one warp per leaf, four warps per block;
- * leaves wider than about 38 sigma still take the target-side kernel) or 192 (the 64-thread kernel with each
- * of the three source rows in its own block, summed at the end); targets_per_thread 2 or 4 (the most
- * targets one lane takes per pass; passes are balanced over the leaf). 0 = default (64, 4).
+ * particles in adjacent leaves evaluated once and applied to both; up to 1024 leaves in the call a thread block per
+ * leaf, beyond that persistent blocks that take the leaves in order of falling work, the heaviest a whole block each,
+ * the others a warp; leaves wider than about 38 sigma still take the target-side kernel) or 192 (the 64-thread kernel
+ * with each of the three source rows in its own block, summed at the end); targets_per_thread 2 or 4 (the most
+ * targets one lane takes per pass; passes are balanced over the leaf). 0 = default (64, 4). With up to 1024 leaves in
+ * the call, or 4096 of 64 particles and more on average, 32, 64 and 256 all run one warp per leaf and source row; the
+ * tile then sets how the sources are cut, and so the order of the sums, but not the blocks.
  * Set by fmm_autotune; exposed for experiments. */
 fmm_status fmm_set_p2p_tile(fmm_handle h, int threads, int targets_per_thread);
 

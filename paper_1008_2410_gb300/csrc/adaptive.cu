@@ -745,7 +745,8 @@ __device__ __forceinline__ void walk_uw(const Work &w, const Tree &t, int l, int
 // One thread per existing box of levels 2 .. L: a leaf with particles walks U and W once for all of them and writes
 // what it met, in the walk's order; its particles get the list's number. Leaves with more than the lists hold, those
 // beyond ad_cap lists and those of levels 0 and 1 stay walked by each particle. 84 us at 2^22 particles in 8 patches,
-// beside the sweep; with the FP64 divisions taken out of the W and L2P evaluations the whole went from 3.24 to 2.82 ms.
+// beside the sweep; with the FP64 divisions taken out of the W and L2P evaluations the whole went from 3.24 to 2.82 ms
+// (2.80 with the W boxes' centres made at their use instead of listed).
 __global__ void __launch_bounds__(128) k_ad_lists(Work w)
 {
     const SysDev &d = w.sys[0];

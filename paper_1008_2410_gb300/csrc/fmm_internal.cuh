@@ -62,8 +62,8 @@ struct SysDev {
     int n64_thr;
     double iu;                      // adaptive tree's precision form: 1 / u, u = sigma sqrt(2 / log2 e)
     // boundary bands of the precision form's near field: a particle whose leaf-relative position zeta (in leaf
-    // widths, |zeta| <= 1/2) has |zeta_x| * 2^52 > fbnd lies within delta = sigma (1 + 2^-8) of its leaf's left or
-    // right side (likewise y); bnd_ok = 0 when the bands would overlap (leaf narrower than 2 delta)
+    // widths, |zeta| <= 1/2) has |zeta_x| * 2^52 > fbnd lies within delta = 6 sigma (1 + 2^-8) of its leaf's left
+    // or right side (likewise y); bnd_ok = 0 when the bands would overlap (leaf narrower than 2 delta)
     long long fbnd;
     int bnd_ok;
     int n64_pack;

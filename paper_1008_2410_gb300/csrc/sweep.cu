@@ -261,7 +261,7 @@ int launch_m2m(const Work &w, const Tables &t, int l, int adj, cudaStream_t s, i
 // Measured at 2^20 particles (21840 boxes, p = 17): 1.61 ms with a warp a box and single sources, 0.51 ms so.
 __constant__ signed char c_m2l_orbit[10][2] = {{2, 0}, {3, 0}, {2, 1}, {3, 1}, {1, 2}, {2, 2}, {3, 2}, {1, 3}, {2, 3}, {3, 3}};
 
-constexpr int M2L64_T = 128;  // threads: 10 K registers a block, which fit beside the near field's blocks
+constexpr int M2L64_T = 128;  // threads: 11.5 K registers a block at p = 17, which fit beside the near field's blocks
 template <int PM>
 __global__ void __launch_bounds__(M2L64_T) k_m2l64(Work w, const double2 *__restrict__ rho, const double *__restrict__ binom,
                                                const double2 *__restrict__ M, double2 *__restrict__ Loc, int nb, int64_t gw0,
