@@ -421,9 +421,11 @@ struct Acc64 {
         lo[t] = d;
         hi[t] += (int)(h >> 40) + (b < a ? 1 : 0) + (int)(l >> 63) + (d < b ? 1 : 0);
     }
+    __device__ __forceinline__ void meet(int t, const Acc64 &o) { big[t] = fmaxf(big[t], o.big[t]); }
     __device__ __forceinline__ float biggest(int t, int step, int n) const  // of threads t, t + step, ...
     {
         float m = big[t];
+#pragma unroll 4
         for (int k = 1; k < n; ++k)
             m = fmaxf(m, big[t + k * step]);
         return m;
@@ -497,6 +499,7 @@ __device__ __forceinline__ double block_sum(double v, double *red)
 __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
 {
     __shared__ int s_leaf, s_weak;
+    __shared__ float2 s_line;
     extern __shared__ __align__(16) unsigned char sm[];  // N64_SMEM bytes
     int4 *pos = reinterpret_cast<int4 *>(sm);                        // x and y limbs
     int2 *gam = reinterpret_cast<int2 *>(pos + N64_TILE);            // gamma limbs, base 2^32
@@ -532,6 +535,10 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
     const int ge = fixed ? charge_exponent(R, ntot, w.sg, nullptr, st) : kNoFixed;
     fixed = ge != kNoFixed;
     const int ka = ge - 63;  // charges in units of 2^ka: below 2^63 - 2^50, so that their high limb fits
+    if (tid == 0 && fixed) {  // cs / fs and the close sums' line (see the sums' end): here for the registers' sake
+        const float ratio = cl.lim ? (float)(k2 * pow2(117 - cl.s + 2 * ku)) : 0.0f;
+        s_line = make_float2(ratio, ratio * (cl.s > 3 ? 0x1p20f : 0x1p19f));  // s > 3: positions next to an axis (2^(s - 3) units)
+    }
 
     const int npass = pick_passes(c);
     for (int pass = 0; pass < npass; ++pass) {
@@ -667,15 +674,18 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             spill_close();
             for (int q = 0; q < 4; ++q)
                 acc[q].mark(tid);
+            acc[0].meet(tid, acc[1]);
+            acc[2].meet(tid, acc[3]);
         }
         // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double2 *red = reinterpret_cast<double2 *>(pos);
         if (tid == 0)
             s_weak = 0;
         const bool some64 = __syncthreads_or(au != 0.0 || av != 0.0);
-        if (some64)
+        if (some64) {
             red[tid] = make_double2(au, av);
-        __syncthreads();
+            __syncthreads();
+        }
         if (tid < cp) {
             const int ng = min(G, ntot);  // groups with sources
             double u = 0.0, v = 0.0;
@@ -690,17 +700,15 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             }
             if (fixed) {
                 // a far term is gamma dx / r^2 2^(51 + ku - ka), a close one gamma F dx 2^(s - 66 - ku - ka)
-                const double gs = pow2(ka), fs = pow2(-51 - ku), cs = k2 * pow2(66 - cl.s + ku);
+                const int kq = fresh(ku);
+                const double gs = pow2(fresh(ka)), fs = pow2(-51 - kq), cs = k2 * pow2(66 - cl.s + kq);
                 // A term's rounding is about 0.4 of its unit (fs or cs, times gs) however small the term is, in FP64 it is
                 // relative to it: a target whose sums are all small against the unit, because the strong sources have no
                 // weight there, is left to FP64 below. At this line the error is a few times that of FP64 sums. What counts is the
                 // largest that a sum has been at the tiles' ends, so that a velocity that is small by cancellation does not count.
-                const float far = fmaxf(acc[0].biggest(tid, cp, ng), acc[1].biggest(tid, cp, ng));
-                const float near = fmaxf(acc[2].biggest(tid, cp, ng), acc[3].biggest(tid, cp, ng));
-                // (next to a coordinate axis a position is short of 2^(s - 3) units as well)
-                const float ratio = cl.lim ? (float)(k2 * pow2(117 - cl.s + 2 * ku)) : 0.0f;  // cs / fs
-                const float line = line_of(far, near, 0x1p19f, ratio * (cl.s > 3 ? 0x1p20f : 0x1p19f));
-                if (fmaxf(far, near * ratio) < line && (!some64 || fmax(fabs(u), fabs(v)) < line * 0x1p32 * fs * gs))
+                const float far = acc[0].biggest(tid, cp, ng), near = acc[2].biggest(tid, cp, ng);
+                const float line = line_of(far, near, 0x1p19f, s_line.y);
+                if (fmaxf(far, near * s_line.x) < line && (!some64 || fmax(fabs(u), fabs(v)) < line * 0x1p32 * fs * gs))
                     lst[atomicAdd(&s_weak, 1)] = (unsigned short)tid;
                 u -= fma(acc[2].total(tid, cp, ng), cs, acc[0].total(tid, cp, ng) * fs) * gs;
                 v += fma(acc[3].total(tid, cp, ng), cs, acc[1].total(tid, cp, ng) * fs) * gs;
@@ -720,7 +728,8 @@ __global__ void __launch_bounds__(N64_THREADS, 4) k_near64(Work w, int parts)
             if (tid == 0)
                 w.near64[t] = make_double2(bu * k2 / kTwoPi, bv * k2 / kTwoPi);
         }
-        __syncthreads();
+        if (nweak > 0)
+            __syncthreads();
     }
     }
 }
@@ -1053,6 +1062,8 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ W
             }
             for (int q = 0; q < 6; ++q)
                 acc[q].mark(tid);
+            acc[1].meet(tid, acc[2]);
+            acc[4].meet(tid, acc[5]);
         }
         // sums of a target's groups, in order; the FP64 pairs' through the (now idle) source limbs
         double *red = reinterpret_cast<double *>(pos);
@@ -1061,8 +1072,8 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ W
             red[tid] = ag;
             red[N64_THREADS + tid] = ax;
             red[2 * N64_THREADS + tid] = ay;
+            __syncthreads();
         }
-        __syncthreads();
         if (tid < cp) {
             const int ng = min(G, ntot);  // groups with sources
             double out[3] = {0.0, 0.0, 0.0};
@@ -1083,18 +1094,17 @@ __global__ void __maxnreg__(A64_REGS) k_adjoint_near64(const __grid_constant__ W
                 // (P and Q); a close pair's by about 2^18 and 2^19, by up to 2^21 where all pairs are close. So is one with a
                 // coincident particle.
                 const float far_g = acc[0].biggest(tid, cp, ng), near_g = acc[3].biggest(tid, cp, ng);
-                const float far_x = fmaxf(acc[1].biggest(tid, cp, ng), acc[2].biggest(tid, cp, ng));
-                const float near_x = fmaxf(acc[4].biggest(tid, cp, ng), acc[5].biggest(tid, cp, ng));
+                const float far_x = acc[1].biggest(tid, cp, ng), near_x = acc[4].biggest(tid, cp, ng);
                 const float4 line = s_line;
                 bool small = fmaxf(far_g, near_g * line.x) < line_of(far_g, near_g, 0x1p42f, line.y) || far_g == INFINITY;
                 if (gt != 0.0 || gut != 0.0 || gvt != 0.0)
                     small |= fmaxf(far_x, near_x * line.z) < line_of(far_x, near_x, 0x1p37f, line.w);
                 if (small)
                     w.slot[tpos] = atomicExch(&s_weak, tpos);
-                out[0] += ldexp(fma(acc[3].total(tid, cp, ng), cg, acc[0].total(tid, cp, ng) * fg), kb);
+                out[0] += ldexp(fma(acc[3].total(tid, cp, ng), cg, acc[0].total(tid, cp, ng) * fg), fresh(kb));
 #pragma unroll
                 for (int q = 1; q < 3; ++q)
-                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, ng), cx, acc[q].total(tid, cp, ng) * fx), ka + kb - tau);
+                    out[q] += ldexp(fma(acc[3 + q].total(tid, cp, ng), cx, acc[q].total(tid, cp, ng) * fx), fresh(ka) + fresh(kb) - fresh(tau));
             }
             const int i = w.perm[tpos];
             if (odg)
