@@ -781,7 +781,7 @@ struct Adj64 {
 // multiplications in fixed point (22 operations in FP64, several times the time); sums in two 64-bit parts, high
 // products and cross terms. A close one takes F and -F' from their tables, 86 wide multiplications (37 operations in
 // FP64). Measured at 2^20 uniform particles (leaves of 64, 16 sigma wide): 103 ms with exp, expm1 and divisions in FP64
-// for every pair; the whole adjoint (near field beside both sweeps) 108 ms then, 8.9 ms now. 112 or 128 registers keep
+// for every pair; the whole adjoint (near field beside both sweeps) 108 ms then, 8.9 ms now. 104 to 128 registers keep
 // the sweeps' blocks out (11.6 to 12.0 ms), 80 spill (10.9). Errors against quad precision are below the former ones.
 // Writes the near part in caller order (the far part is added later). Targets for whom the fixed unit is too coarse, or
 // with coincident particles, are listed in slot (free after the binning) and summed in FP64 at the end.
